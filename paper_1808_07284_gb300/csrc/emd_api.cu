@@ -13,6 +13,7 @@
 #include <vector>
 
 #include "emd_gb300.h"
+#include "emd_chip.cuh"
 #include "emd_kernels.cuh"
 #include "emd_lsd.cuh"
 #include "emd_march.cuh"
@@ -366,12 +367,94 @@ struct SolveExtra {
   // behind gigabytes of copies they would hold the host thread until those had finished,
   // and the prepares would be enqueued only after the copies instead of beside them.
   std::function<emd_status()> *stage = nullptr;
+  bool no_chip = false;  // not the on-chip solve (what it handed back is solved by the others)
 };
 
 emd_status solve_impl(int B, const float *const *f_obs, const float *const *f_pred, const int *nt,
                       const int *nr, const double *dt, const double *dx, const emd_params *pp,
                       float *const *phi, float *const *m, emd_result *results, void *ws,
                       size_t ws_bytes, cudaStream_t stream, const SolveExtra &x = SolveExtra{});
+
+// How the on-chip solve (emd_chip.cuh) lays a batch out: waves of gathers that are on chip side
+// by side, one cooperative launch per wave.
+struct ChipPlan {
+  std::vector<std::vector<emd::ChipJob>> waves;
+  int rows = 0;       // staged rows of the tallest CTA
+  double cost = 0.0;  // estimated time of one pass over every gather, us
+};
+
+// Estimated us per pass of a wave whose tallest CTA stages n rows.
+double chip_pass_us(int n) { return 3.0 + 0.1 * ((n + emd::kChipWorkers - 1) / emd::kChipWorkers) + 0.02 * n; }
+
+// Whether a gather's state fits on `cap` SMs (and its exchange buffers in its planes).
+bool chip_fits(int nt, int nr, int cap) {
+  const long long strips = (nt + emd::kChipTJ - 1) / emd::kChipTJ;
+  const long long segs = (nr + emd::kChipMaxRows - 4) / (emd::kChipMaxRows - 3);
+  if (strips * segs > cap) return false;
+  const size_t planes = 9 * align256(sizeof(float) * static_cast<size_t>(nr) * ntp_of(nt));
+  return emd::chip_exchange_bytes(std::max(1, (nr + 1) / 2), static_cast<int>(strips), nr, ntp_of(nt)) <= planes;
+}
+
+// The plan whose estimated pass is shortest, over the rows per warp (more rows put more gathers
+// beside each other, fewer spread one gather over more SMs); no waves when a gather is too large.
+ChipPlan chip_plan(int B, const int *nt, const int *nr, int cap) {
+  ChipPlan best;
+  constexpr int kMaxRun = (emd::kChipMaxRows + emd::kChipWorkers - 1) / emd::kChipWorkers;
+  for (int m = 1; m <= kMaxRun; ++m) {
+    const int hmax = std::min(emd::kChipWorkers * m, emd::kChipMaxRows) - 3;
+    std::vector<emd::ChipJob> g(B);
+    bool fits = true;
+    for (int b = 0; b < B && fits; ++b) {
+      emd::ChipJob &J = g[b];
+      J.gather = b;
+      J.strips = (nt[b] + emd::kChipTJ - 1) / emd::kChipTJ;
+      const int nseg = (nr[b] + hmax - 1) / hmax;
+      J.h = std::max(nr[b] > 1 ? 2 : 1, (nr[b] + nseg - 1) / nseg);
+      J.segs = (nr[b] + J.h - 1) / J.h;
+      const long long group = static_cast<long long>(J.strips) * J.segs;
+      fits = group <= cap;
+      J.group = static_cast<int>(std::min<long long>(group, cap));
+    }
+    if (!fits) continue;
+    std::vector<int> order(B);
+    for (int b = 0; b < B; ++b) order[b] = b;
+    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return g[a].group > g[b].group; });
+    std::vector<int> used, rows;
+    std::vector<std::vector<int>> members;
+    for (int b : order) {  // first fit, largest first
+      size_t w = 0;
+      while (w < used.size() && used[w] + g[b].group > cap) ++w;
+      if (w == used.size()) {
+        used.push_back(0);
+        rows.push_back(0);
+        members.emplace_back();
+      }
+      used[w] += g[b].group;
+      rows[w] = std::max(rows[w], g[b].h + 3);
+      members[w].push_back(b);
+    }
+    double cost = 0.0;
+    for (int n : rows) cost += chip_pass_us(n);
+    if (!best.waves.empty() && cost >= best.cost) continue;
+    best.cost = cost;
+    best.rows = *std::max_element(rows.begin(), rows.end());
+    best.waves.clear();
+    for (const auto &mem : members) {
+      best.waves.emplace_back();
+      for (int b : mem)
+        for (int seg = 0; seg < g[b].segs; ++seg)
+          for (int strip = 0; strip < g[b].strips; ++strip) {
+            emd::ChipJob J = g[b];
+            J.seg = seg;
+            J.strip = strip;
+            J.i0 = seg * g[b].h;
+            J.h = std::min(g[b].h, nr[b] - J.i0);
+            best.waves.back().push_back(J);
+          }
+    }
+  }
+  return best;
+}
 
 // Tile-shape autotuner of the TMA pass.  The first default-tile solve of a (device,
 // gather sizes) configuration times each TMA shape on the caller's own data -- two short
@@ -440,6 +523,171 @@ int autotune_shape(int B, const float *const *f_obs, const float *const *f_pred,
   return best;
 }
 
+// The gather's descriptor: everything but the tiling of a particular pass.
+void fill_shot(Shot &S, const float *p_obs, const float *p_pred, int nt, int nr, double dt, double dx,
+               float *phi, float *m, const float *phi_init, const float *m_init, char *planes,
+               size_t pl) {
+  std::memset(&S, 0, sizeof(S));
+  S.p_obs = p_obs;
+  S.p_pred = p_pred;
+  S.phi_out = phi;
+  S.m_out = m;
+  S.phi_init = phi_init;
+  S.m_init = m_init;
+  S.nt = nt;
+  S.nr = nr;
+  S.ntp = ntp_of(nt);
+  S.f = reinterpret_cast<float *>(planes);
+  for (int u = 0; u < 3; ++u) {
+    S.ux[u] = reinterpret_cast<float *>(planes + (1 + 2 * u) * pl);
+    S.ut[u] = reinterpret_cast<float *>(planes + (2 + 2 * u) * pl);
+  }
+  S.ph[0] = reinterpret_cast<float *>(planes + 7 * pl);
+  S.ph[1] = reinterpret_cast<float *>(planes + 8 * pl);
+  const bool one_d = nr == 1;
+  S.rdx = one_d ? 0.0f : static_cast<float>(1.0 / dx);
+  S.rdt = static_cast<float>(1.0 / dt);
+  S.area = one_d ? dt : dx * dt;
+  S.lambda = 4.0 / (dt * dt) + (one_d ? 0.0 : 4.0 / (dx * dx));
+}
+
+// The parameters of a solve that every kernel takes.
+Ctl make_ctl(const emd_params &p) {
+  Ctl ctl{};
+  ctl.eps = p.eps;
+  ctl.xi = p.xi;
+  ctl.zeta = p.zeta;
+  ctl.delta = p.delta;
+  ctl.tol = p.tol;
+  ctl.alpha0 = p.alpha0;
+  ctl.max_iter = p.max_iter;
+  ctl.check_every = p.check_every;
+  ctl.ls_max_trials = p.ls_max_trials;
+  ctl.linesearch = p.linesearch;
+  ctl.balance = p.balance;
+  ctl.debug_fault = p.debug_fault;
+  ctl.iso = p.norm == EMD_NORM_ISO;
+  ctl.trace = p.trace;
+  return ctl;
+}
+
+// The public result of a gather from its final state.
+void fill_result(emd_result &r, const State &st, const Shot &S, const emd_params &p, int launches,
+                 int tile) {
+  const double *g = st.gap_sums;  // final u and phi: sum|u|, sum u^2, <phi,f>, h* terms
+  r.dist = S.area * (g[0] + 0.5 * p.eps * g[1]);
+  r.dist_l1 = S.area * g[0];
+  r.mass_mu = st.mass_mu;
+  r.mass_nu = st.mass_nu;
+  r.imbalance = st.imbalance;
+  // residual of the last iteration from its sums (the last pass measured u^K against u^{K-1})
+  r.r_feas = st.fnorm > 0.0 ? std::sqrt(st.s_p2) / st.fnorm : std::sqrt(st.s_p2);
+  r.r_step = std::sqrt(st.s_du2) / std::max(std::sqrt(st.s_u2), 1e-30);
+  r.residual = std::max(r.r_feas, r.r_step);
+  r.duality_gap = p.eps > 0.0 ? S.area * (g[0] + 0.5 * p.eps * g[1] - g[2] + g[3] / (2.0 * p.eps))
+                              : std::nan("");
+  r.alpha = st.alpha;
+  r.theta = st.theta;
+  r.iters = st.k;
+  r.ls_trials = st.trials;
+  r.status = st.status;
+  r.launches = launches;
+  r.tile = tile;
+}
+
+// The on-chip solve of B gathers laid out by `plan`.  A gather whose iterates turn non-finite or
+// whose linesearch fails is handed to the streaming passes, which define what such a solve
+// leaves in phi and m.  *launched = false when the device cannot hold the launch (nothing done).
+emd_status solve_on_chip(int B, const float *const *f_obs, const float *const *f_pred, const int *nt,
+                         const int *nr, const double *dt, const double *dx, const emd_params &p,
+                         float *const *phi, float *const *m, emd_result *results, void *ws,
+                         size_t ws_bytes, cudaStream_t stream, const SolveExtra &x, const Layout &L,
+                         const ChipPlan &plan, bool *launched) {
+  *launched = false;
+  void (*fn)(const Ctl, const emd::ChipJobs) =
+      p.norm == EMD_NORM_ISO ? emd::k_solve_chip<true> : emd::k_solve_chip<false>;
+  const size_t smem = emd::kChipSmem;
+  int dev = 0, coop = 0, per_sm = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop ||
+      cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) !=
+          cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, emd::kChipThreads, smem) != cudaSuccess ||
+      per_sm < 1) {
+    (void)cudaGetLastError();
+    return EMD_OK;
+  }
+  *launched = true;
+  char *base = static_cast<char *>(ws);
+  std::vector<Shot> shots(B);
+  for (int b = 0; b < B; ++b)
+    fill_shot(shots[b], f_obs[b], f_pred[b], nt[b], nr[b], dt[b], dx[b], phi[b], m[b],
+              x.phi_init ? x.phi_init[b] : p.phi_init, x.m_init ? x.m_init[b] : p.m_init,
+              base + L.gather[b], L.plane[b]);
+  State *states = reinterpret_cast<State *>(base + L.states);
+  int *flags = reinterpret_cast<int *>(base + L.misc);
+  Ctl ctl = make_ctl(p);
+  ctl.shots = reinterpret_cast<Shot *>(base + L.shots);
+  ctl.states = states;
+  ctl.acc = reinterpret_cast<double *>(base + L.acc);
+  ctl.n_done = flags;
+  ctl.error = flags + 1;
+  EMD_CK(cudaMemcpyAsync(base + L.shots, shots.data(), sizeof(Shot) * B, cudaMemcpyHostToDevice, stream));
+  EMD_CK(cudaMemsetAsync(states, 0, sizeof(State) * B, stream));
+  EMD_CK(cudaMemsetAsync(flags, 0, 2 * sizeof(int), stream));
+  EMD_CK(cudaMemsetAsync(ctl.acc, 0, sizeof(double) * emd::kAccBufs * emd::kSpread * emd::kAcc * B, stream));
+  if (x.stage && *x.stage) {
+    const std::function<emd_status()> enqueue = std::move(*x.stage);
+    *x.stage = nullptr;
+    const emd_status s = enqueue();
+    if (s != EMD_OK) return s;
+  }
+  for (const auto &wave : plan.waves) {
+    emd::ChipJobs jobs{};
+    std::copy(wave.begin(), wave.end(), jobs.job);
+    if (x.ready)
+      for (size_t i = 0; i < wave.size(); ++i)
+        if (wave[i].seg == 0 && wave[i].strip == 0)
+          EMD_CK(cudaStreamWaitEvent(stream, x.ready[wave[i].gather], 0));
+    Ctl cctl = ctl;
+    void *args[] = {&cctl, &jobs};
+    EMD_CK(cudaLaunchCooperativeKernel(reinterpret_cast<void *>(fn), dim3(static_cast<unsigned>(wave.size())),
+                                       dim3(emd::kChipThreads), args, smem, stream));
+  }
+  std::vector<State> hs(B);
+  int h_flags[2] = {0, 0};
+  EMD_CK(cudaMemcpyAsync(hs.data(), states, sizeof(State) * B, cudaMemcpyDeviceToHost, stream));
+  EMD_CK(cudaMemcpyAsync(h_flags, flags, sizeof(h_flags), cudaMemcpyDeviceToHost, stream));
+  EMD_CK(cudaStreamSynchronize(stream));
+  if (h_flags[1]) {  // a bounded device wait gave up
+    for (int b = 0; b < B; ++b) results[b].status = EMD_ERR_TIMEOUT;
+    return EMD_ERR_TIMEOUT;
+  }
+  emd_status first = EMD_OK;
+  for (int b = 0; b < B; ++b) {
+    fill_result(results[b], hs[b], shots[b], p, static_cast<int>(plan.waves.size()), 0);
+    if (hs[b].status != EMD_OK) {
+      emd_params q = p;
+      if (p.trace) q.trace = p.trace + static_cast<size_t>(b) * p.max_iter * 4;
+      q.phi_init = shots[b].phi_init;
+      q.m_init = shots[b].m_init;
+      SolveExtra again;
+      again.no_chip = true;
+      again.no_tune = true;
+      again.no_graph = x.no_graph;
+      const emd_status s = solve_impl(1, f_obs + b, f_pred + b, nt + b, nr + b, dt + b, dx + b, &q, phi + b,
+                                      m + b, results + b, ws, ws_bytes, stream, again);
+      results[b].launches += static_cast<int>(plan.waves.size());
+      if (first == EMD_OK && s != EMD_OK) first = s;
+    }
+  }
+  return first;
+}
+
+// Estimated us per pass of the streaming solves (tile and marching pass) over `cells` cells:
+// about 10 us of decision chain and 5.9 us per million cells, from L2 or from HBM alike.
+double stream_pass_us(double cells) { return 10.0 + 5.9e-6 * cells; }
+
 emd_status solve_impl(int B, const float *const *f_obs, const float *const *f_pred, const int *nt,
                       const int *nr, const double *dt, const double *dx, const emd_params *pp,
                       float *const *phi, float *const *m, emd_result *results, void *ws,
@@ -466,6 +714,77 @@ emd_status solve_impl(int B, const float *const *f_obs, const float *const *f_pr
   for (int b = 0; b < B; ++b) max_cells = std::max(max_cells, static_cast<long long>(nt[b]) * nr[b]);
   // Small gathers: one CTA per gather keeps the whole solve in shared memory.
   const bool resident = p.launch_mode == 0 && p.tile == 0 && max_cells <= emd::kResidentMaxCells;
+  // Gathers whose state fits on the chip are solved there; the others of the batch stream.
+  if (p.tile == 0 && p.launch_mode == 0 && !resident && !x.no_chip) {
+    const int cap = std::min(sm_count(), emd::kChipMaxCtas);
+    std::vector<int> on, off;
+    double on_cells = 0.0;
+    for (int b = 0; b < B; ++b) {
+      if (chip_fits(nt[b], nr[b], cap)) {
+        on.push_back(b);
+        on_cells += static_cast<double>(nt[b]) * nr[b];
+      } else {
+        off.push_back(b);
+      }
+    }
+    if (!on.empty() && !(p.trace && !off.empty())) {
+      auto pick = [&](const auto *a, const std::vector<int> &idx) {
+        std::vector<std::decay_t<decltype(a[0])>> v;
+        if (a)
+          for (int b : idx) v.push_back(a[b]);
+        return v;
+      };
+      const auto on_nt = pick(nt, on), on_nr = pick(nr, on);
+      const ChipPlan plan = chip_plan(static_cast<int>(on.size()), on_nt.data(), on_nr.data(), cap);
+      const double streamed = off.empty() ? stream_pass_us(on_cells) : stream_pass_us(on_cells) - stream_pass_us(0.0);
+      if (!plan.waves.empty() && plan.cost < streamed) {
+        bool launched = false;
+        if (off.empty()) {
+          const emd_status s = solve_on_chip(B, f_obs, f_pred, nt, nr, dt, dx, p, phi, m, results, ws,
+                                             ws_bytes, stream, x, L, plan, &launched);
+          if (launched) return s;
+        } else {  // two batches, one after the other in the same workspace
+          emd_status st[2] = {EMD_OK, EMD_OK};
+          bool done = true;
+          for (int part = 0; part < 2 && done; ++part) {
+            const std::vector<int> &idx = part ? off : on;
+            const auto a_nt = pick(nt, idx), a_nr = pick(nr, idx);
+            const auto a_dt = pick(dt, idx), a_dx = pick(dx, idx);
+            const auto a_obs = pick(f_obs, idx), a_pred = pick(f_pred, idx);
+            const auto a_phi = pick(phi, idx), a_m = pick(m, idx);
+            const auto a_pi = pick(x.phi_init, idx), a_mi = pick(x.m_init, idx);
+            const auto a_ready = pick(x.ready, idx);
+            SolveExtra y = x;
+            y.phi_init = x.phi_init ? a_pi.data() : nullptr;
+            y.m_init = x.m_init ? a_mi.data() : nullptr;
+            y.ready = x.ready ? a_ready.data() : nullptr;
+            const int nb = static_cast<int>(idx.size());
+            std::vector<emd_result> res(nb);
+            if (part == 0) {
+              const Layout La = layout(nb, a_nt.data(), a_nr.data());
+              st[0] = solve_on_chip(nb, a_obs.data(), a_pred.data(), a_nt.data(), a_nr.data(), a_dt.data(),
+                                    a_dx.data(), p, a_phi.data(), a_m.data(), res.data(), ws, ws_bytes,
+                                    stream, y, La, plan, &launched);
+              if (!launched) done = false;
+            } else {
+              y.no_chip = true;
+              st[1] = solve_impl(nb, a_obs.data(), a_pred.data(), a_nt.data(), a_nr.data(), a_dt.data(),
+                                 a_dx.data(), &p, a_phi.data(), a_m.data(), res.data(), ws, ws_bytes, stream, y);
+            }
+            if (done)
+              for (int i = 0; i < nb; ++i) results[idx[i]] = res[i];
+            for (emd_status s : {st[part]})
+              if (s == EMD_ERR_CUDA || s == EMD_ERR_TIMEOUT) return s;
+          }
+          if (done) {
+            for (int b = 0; b < B; ++b)
+              if (results[b].status != EMD_OK) return static_cast<emd_status>(results[b].status);
+            return EMD_OK;
+          }
+        }
+      }
+    }
+  }
   if (p.tile == 0 && !resident && si == kTmaShape && !x.no_tune)
     si = autotune_shape(B, f_obs, f_pred, nt, nr, dt, dx, p, phi, m, results, ws, ws_bytes, stream,
                         x);
@@ -477,35 +796,15 @@ emd_status solve_impl(int B, const float *const *f_obs, const float *const *f_pr
   int nr_max = 0;
   for (int b = 0; b < B; ++b) {
     Shot &S = shots[b];
-    std::memset(&S, 0, sizeof(S));
-    S.p_obs = f_obs[b];
-    S.p_pred = f_pred[b];
-    S.phi_out = phi[b];
-    S.m_out = m[b];
-    S.phi_init = x.phi_init ? x.phi_init[b] : p.phi_init;
-    S.m_init = x.m_init ? x.m_init[b] : p.m_init;
-    S.nt = nt[b];
-    S.nr = nr[b];
-    S.ntp = ntp_of(nt[b]);
     const size_t pl = L.plane[b];
     char *g = base + L.gather[b];
-    S.f = reinterpret_cast<float *>(g);
-    for (int u = 0; u < 3; ++u) {
-      S.ux[u] = reinterpret_cast<float *>(g + (1 + 2 * u) * pl);
-      S.ut[u] = reinterpret_cast<float *>(g + (2 + 2 * u) * pl);
-    }
-    S.ph[0] = reinterpret_cast<float *>(g + 7 * pl);
-    S.ph[1] = reinterpret_cast<float *>(g + 8 * pl);
+    fill_shot(S, f_obs[b], f_pred[b], nt[b], nr[b], dt[b], dx[b], phi[b], m[b],
+              x.phi_init ? x.phi_init[b] : p.phi_init, x.m_init ? x.m_init[b] : p.m_init, g, pl);
     if (uses_tma(sh) && !encode_tmap(S, g, pl, sh.ti + 4)) return EMD_ERR_CUDA;
     S.tiles_j = (nt[b] + (sh.w - 8) - 1) / (sh.w - 8);
     S.tile0 = static_cast<int>(tile_shot.size());
     S.ntiles = tiles_of(sh, nt[b], nr[b]);
     tile_shot.insert(tile_shot.end(), S.ntiles, b);
-    const bool one_d = nr[b] == 1;
-    S.rdx = one_d ? 0.0f : static_cast<float>(1.0 / dx[b]);
-    S.rdt = static_cast<float>(1.0 / dt[b]);
-    S.area = one_d ? dt[b] : dx[b] * dt[b];
-    S.lambda = 4.0 / (dt[b] * dt[b]) + (one_d ? 0.0 : 4.0 / (dx[b] * dx[b]));
     nr_max = std::max(nr_max, nr[b]);
   }
   const int grid = static_cast<int>(tile_shot.size());
@@ -532,20 +831,7 @@ emd_status solve_impl(int B, const float *const *f_obs, const float *const *f_pr
   EMD_CK(cudaMemsetAsync(acc, 0, sizeof(double) * emd::kAccBufs * emd::kSpread * emd::kAcc * B,
                          stream));
 
-  Ctl ctl{};
-  ctl.eps = p.eps;
-  ctl.xi = p.xi;
-  ctl.zeta = p.zeta;
-  ctl.delta = p.delta;
-  ctl.tol = p.tol;
-  ctl.alpha0 = p.alpha0;
-  ctl.max_iter = p.max_iter;
-  ctl.check_every = p.check_every;
-  ctl.ls_max_trials = p.ls_max_trials;
-  ctl.linesearch = p.linesearch;
-  ctl.balance = p.balance;
-  ctl.debug_fault = p.debug_fault;
-  ctl.iso = p.norm == EMD_NORM_ISO;
+  Ctl ctl = make_ctl(p);
   ctl.shots = dshots;
   ctl.states = states;
   ctl.acc = acc;
@@ -554,7 +840,6 @@ emd_status solve_impl(int B, const float *const *f_obs, const float *const *f_pr
   ctl.march_nrun = static_cast<int>(march_run.size());
   ctl.n_done = n_done;
   ctl.error = err_flag;
-  ctl.trace = p.trace;
 
   const size_t smem = smem_bytes(sh);
   if (sh.iter_tma)
@@ -725,27 +1010,7 @@ emd_status solve_impl(int B, const float *const *f_obs, const float *const *f_pr
   emd_status first = EMD_OK;
   for (int b = 0; b < B; ++b) {
     const State &st = hs[b];
-    emd_result &r = results[b];
-    const Shot &S = shots[b];
-    const double *g = st.gap_sums;  // final u and phi: sum|u|, sum u^2, <phi,f>, h* terms
-    r.dist = S.area * (g[0] + 0.5 * p.eps * g[1]);
-    r.dist_l1 = S.area * g[0];
-    r.mass_mu = st.mass_mu;
-    r.mass_nu = st.mass_nu;
-    r.imbalance = st.imbalance;
-    // residual of the last iteration from its sums (the last pass measured u^K against u^{K-1})
-    r.r_feas = st.fnorm > 0.0 ? std::sqrt(st.s_p2) / st.fnorm : std::sqrt(st.s_p2);
-    r.r_step = std::sqrt(st.s_du2) / std::max(std::sqrt(st.s_u2), 1e-30);
-    r.residual = std::max(r.r_feas, r.r_step);
-    r.duality_gap = p.eps > 0.0 ? S.area * (g[0] + 0.5 * p.eps * g[1] - g[2] + g[3] / (2.0 * p.eps))
-                                : std::nan("");
-    r.alpha = st.alpha;
-    r.theta = st.theta;
-    r.iters = st.k;
-    r.ls_trials = st.trials;
-    r.status = st.status;
-    r.launches = n_launch;
-    r.tile = resident ? 0 : si + 1;
+    fill_result(results[b], st, shots[b], p, n_launch, resident ? 0 : si + 1);
     if (first == EMD_OK && st.status != EMD_OK) first = static_cast<emd_status>(st.status);
   }
   return first;

@@ -150,15 +150,54 @@ __device__ __forceinline__ void prox_cell(float vx, float vt, float alpha, float
 // The norm of one cell's flux and the conjugate term (|w| - 1)_+^2 of the dual, per the
 // ground cost (the duality gap's h* of Sec. 2.2's Lagrangian).
 __device__ __forceinline__ float cell_norm(float ux, float ut, bool iso) {
-  return iso ? sqrtf(ux * ux + ut * ut) : fabsf(ux) + fabsf(ut);
+  return iso ? sqrtf(fmaf(ux, ux, ut * ut)) : fabsf(ux) + fabsf(ut);
 }
 __device__ __forceinline__ float cell_conj(float gx, float gt, bool iso) {
   if (iso) {
-    const float e = fmaxf(sqrtf(gx * gx + gt * gt) - 1.0f, 0.0f);
+    const float e = fmaxf(sqrtf(fmaf(gx, gx, gt * gt)) - 1.0f, 0.0f);
     return e * e;
   }
   const float ex = fmaxf(fabsf(gx) - 1.0f, 0.0f), et = fmaxf(fabsf(gt) - 1.0f, 0.0f);
-  return ex * ex + et * et;
+  return fmaf(ex, ex, et * et);
+}
+
+// s + e = a + b exactly (Knuth's two-sum), and p + e = a b exactly.
+__device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
+  s = __fadd_rn(a, b);
+  const float bb = __fsub_rn(s, a);
+  e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+}
+
+// A sum in two floats: each term is added exactly to hi, the rounding errors collect in lo.
+struct Sum2 {
+  float hi = 0.0f, lo = 0.0f;
+  __device__ __forceinline__ void add(float x) {
+    float e;
+    two_sum(hi, x, hi, e);
+    lo += e;
+  }
+  __device__ __forceinline__ double value() const { return static_cast<double>(hi) + static_cast<double>(lo); }
+  // The warp's total, in every lane.
+  __device__ __forceinline__ void warp_total() {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      float s, e;
+      two_sum(hi, __shfl_xor_sync(0xffffffffu, hi, o), s, e);
+      lo = (lo + __shfl_xor_sync(0xffffffffu, lo, o)) + e;
+      hi = s;
+    }
+  }
+};
+
+// One cell's terms of the finalize pass's four sums: |u|, u^2, phi f, (|grad phi| - 1)_+^2.  They
+// are summed in two floats (at four times the cost of a plain addition, in a pass bound by
+// memory), so that every solver path returns the same distance of the same iterates.
+__device__ __forceinline__ void gap_terms(Sum2 (&t)[4], float ux, float ut, float ph, float f,
+                                          float gx, float gt, bool iso) {
+  t[0].add(cell_norm(ux, ut, iso));
+  t[1].add(fmaf(ux, ux, ut * ut));
+  t[2].add(ph * f);
+  t[3].add(cell_conj(gx, gt, iso));
 }
 
 // Barrier over the NW * 32 compute threads: the whole CTA, or (NAMED) the compute warps
@@ -195,6 +234,34 @@ __device__ __forceinline__ void block_accumulate(float (&v)[N], double *acc) {
 #pragma unroll
       for (int w = 0; w < h; ++w) p[w] += p[w + h];
     atomicAdd(acc + threadIdx.x, p[0]);
+  }
+}
+
+// The same for N two-float sums per thread: two-float within the warp, FP64 above (the high and
+// the low parts each by their own thread, both added to acc[0..N)).
+template <int N>
+__device__ __forceinline__ void block_accumulate2(Sum2 (&v)[N], double *acc) {
+  constexpr int NW = kThreads / 32;
+  __shared__ float part[NW][2 * N];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int n = 0; n < N; ++n) {
+    v[n].warp_total();
+    if (lane == 0) {
+      part[warp][n] = v[n].hi;
+      part[warp][N + n] = v[n].lo;
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x < 2 * N) {
+    double p[NW];
+#pragma unroll
+    for (int w = 0; w < NW; ++w) p[w] = static_cast<double>(part[w][threadIdx.x]);
+#pragma unroll
+    for (int h = NW / 2; h >= 1; h >>= 1)
+#pragma unroll
+      for (int w = 0; w < h; ++w) p[w] += p[w + h];
+    atomicAdd(acc + threadIdx.x % N, p[0]);
   }
 }
 
@@ -658,7 +725,7 @@ __global__ void __launch_bounds__(kThreads) k_pass(Ctl c) {
 
   if (FINAL) {
     // ---- duality gap terms and the caller's copies of phi^K and u^K, over the tile
-    float v[4] = {0.f, 0.f, 0.f, 0.f};  // sum|u|, sum u^2, <phi, f>, sum (|grad phi|-1)_+^2
+    Sum2 v[4];  // sum|u|, sum u^2, <phi, f>, sum (|grad phi|-1)_+^2
     if (col_in && c_ >= 4 && c_ < TJ + 4) {
       for (int r = 2 + ty; r < TI + 2; r += NRS) {
         const int gi = i0 - 2 + r;
@@ -670,14 +737,11 @@ __global__ void __launch_bounds__(kThreads) k_pass(Ctl c) {
         const size_t g = static_cast<size_t>(gi) * nt + gj;
         S.m_out[g] = ux;
         S.m_out[static_cast<size_t>(nr) * nt + g] = ut;
-        v[0] += cell_norm(ux, ut, c.iso);
-        v[1] += ux * ux + ut * ut;
-        v[2] += PH[o] * (FF[o] - fmean);
-        v[3] += cell_conj(gx, gt, c.iso);
+        gap_terms(v, ux, ut, PH[o], FF[o] - fmean, gx, gt, c.iso);
       }
     }
     double *acc = acc_of(c, s);
-    block_accumulate<4>(v, acc + (lt % kSpread) * kAcc);
+    block_accumulate2<4>(v, acc + (lt % kSpread) * kAcc);
     if (!last_block(&st->ticket, S.ntiles)) return;
     double a_[4];
     gather_totals<4>(acc, a_);

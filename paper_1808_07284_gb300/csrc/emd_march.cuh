@@ -26,6 +26,7 @@
 // values go to the gather's accumulators by FP64 atomics.
 #pragma once
 
+#include "emd_chip.cuh"
 #include "emd_pass_tma.cuh"
 
 namespace emd {
@@ -88,12 +89,6 @@ __device__ __forceinline__ void march_prefetch(const MarchUnit &m, float *ring) 
 #pragma unroll
   for (int r = 0; r < D; ++r) march_issue<D>(m, r, ring);
 }
-
-// A compile-time bool as a value (selects a lambda's instantiation).
-template <bool B>
-struct BoolConst {
-  static constexpr bool value = B;
-};
 
 // Warp sums of the nine FP32 lane sums added to the FP64 fold (lane q holds value q).
 __device__ __forceinline__ void march_fold(float (&v)[9], double &mine) {

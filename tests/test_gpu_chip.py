@@ -1,0 +1,136 @@
+"""The on-chip solve (default for gathers whose state fits in the GPU's shared and tensor memory)
+against the per-pass tile kernels on the same inputs, at the sizes where its layout can go wrong:
+runs of one row per warp, one row more, the tallest CTA and the first that needs a second segment,
+strips of 120 samples and their remainders, receivers and samples at the ends of the range.
+
+The two paths do the same arithmetic on every cell, in the same order, so phi and m may differ
+only where a linesearch decision differs; the sums behind the decisions are added in another
+order, which moves the distance by FP32 rounding of partial sums (a few 1e-8)."""
+
+import math
+
+import numpy as np
+import pytest
+import torch
+
+import synth
+
+pytestmark = pytest.mark.gpu
+
+DT, DX = 2e-3, 10.0
+TILE = 7      # the TMA tile pass
+PLAIN = 2     # the plain pass (any number of receivers)
+
+
+@pytest.fixture(scope="module")
+def P():
+    import paper_1808_07284_gb300 as pkg
+    assert torch.cuda.is_available()
+    return pkg
+
+
+def pair(nr, nt, seed=0):
+    obs, pred = synth.gather_pair_hyperbolic(nt=nt, nr=nr, seed=seed)
+    rng = np.random.default_rng(seed + 1)
+    noise = 0.05 * rng.standard_normal(obs.shape).astype(np.float32)
+    return torch.from_numpy(obs).cuda(), torch.from_numpy(pred + noise).cuda()
+
+
+def check(got, ref, what=""):
+    d, phi, m, info = got
+    d0, phi0, m0, info0 = ref
+    assert info["status"] == 0 and info0["status"] == 0, what
+    assert info["iters"] == info0["iters"] and info["ls_trials"] == info0["ls_trials"], what
+    for a, b, name in ((phi, phi0, "phi"), (m, m0, "m")):
+        rel = float((a.double() - b.double()).norm() / b.double().norm().clamp_min(1e-300))
+        assert rel <= 1e-6, (what, name, rel)
+    for key in ("dist_l1", "residual", "duality_gap"):
+        assert math.isclose(info[key], info0[key], rel_tol=1e-5, abs_tol=1e-12), (what, key)
+    for key in ("mass_mu", "mass_nu"):
+        assert math.isclose(info[key], info0[key], rel_tol=1e-12), (what, key)
+
+
+SHAPES = [(64, 256), (12, 700), (13, 700), (27, 400), (28, 400), (125, 120), (126, 121), (250, 1000),
+          (251, 999), (9, 1201), (2, 4801), (3, 2399), (1, 9001), (640, 61), (648, 1201), (400, 3000),
+          (480, 4000)]
+
+
+@pytest.mark.parametrize("nr,nt", SHAPES)
+def test_matches_the_tile_pass(P, nr, nt):
+    o, p = pair(nr, nt)
+    tile = TILE if nr > 8 else PLAIN
+    got, ref = P.emd(o, p, DT, DX, max_iter=40), P.emd(o, p, DT, DX, max_iter=40, tile=tile)
+    assert got[3]["tile"] == 0 and got[3]["launches"] == 1  # on chip
+    check(got, ref)
+    # from a warm start, in place, and on a single iteration
+    kw = dict(phi_init=ref[1], m_init=ref[2])
+    check(P.emd(o, p, DT, DX, max_iter=15, **kw), P.emd(o, p, DT, DX, max_iter=15, tile=tile, **kw), "warm")
+    check(P.emd(o, p, DT, DX, max_iter=1, **kw), P.emd(o, p, DT, DX, max_iter=1, tile=tile, **kw), "one")
+
+
+@pytest.mark.parametrize("kw", [dict(norm=2), dict(balance=0), dict(linesearch=0), dict(tol=1e-30, check_every=7),
+                                dict(xi=0.9), dict(alpha0=1e-3)])
+def test_options_match_the_tile_pass(P, kw):
+    o, p = pair(70, 500, seed=3)
+    check(P.emd(o, p, DT, DX, max_iter=60, **kw), P.emd(o, p, DT, DX, max_iter=60, tile=TILE, **kw), str(kw))
+
+
+def test_tolerance_stop_and_trace(P):
+    o, p = pair(40, 300, seed=4)
+    dt, dx = 1.0 / 299, 1.0 / 39
+    tr = [torch.zeros((1, 3000, 4), dtype=torch.float64, device="cuda") for _ in range(2)]
+    got = P.emd(o, p, dt, dx, max_iter=3000, tol=0.3, trace=tr[0])
+    ref = P.emd(o, p, dt, dx, max_iter=3000, tol=0.3, trace=tr[1], tile=TILE)
+    assert 10 <= got[3]["iters"] < 3000
+    check(got, ref)
+    assert torch.equal(tr[0][..., 2], tr[1][..., 2])
+    assert torch.allclose(tr[0], tr[1], rtol=1e-5, atol=0.0)
+
+
+def test_unaligned_inputs_and_outputs(P):
+    nr, nt = 33, 402
+    o, p = pair(nr, nt, seed=5)
+    def shifted(t, planes=1):
+        buf = torch.zeros(planes * nr * nt + 1, device="cuda")
+        v = buf[1:].view((planes, nr, nt) if planes > 1 else (nr, nt))
+        if t is not None:
+            v.copy_(t)
+        return v
+    phi, m = shifted(None), shifted(None, 2)
+    ws = P.new_workspace(P.emd_workspace_size(nt, nr), o.device)
+    res = P.emd_dyn_solve(shifted(o), shifted(p), DT, DX, P.emd_default_params(max_iter=40), phi, m, ws)
+    check((res.dist, phi, m, res.as_dict()), P.emd(o, p, DT, DX, max_iter=40, tile=TILE))
+
+
+def test_batch_of_uneven_gathers_one_too_large(P):
+    sizes = [(64, 256), (400, 3000), (1, 8000), (648, 8000), (33, 401), (200, 1500)]
+    pairs = [pair(nr, nt, seed=10 + i) for i, (nr, nt) in enumerate(sizes)]
+    obs, pred = [a for a, _ in pairs], [b for _, b in pairs]
+    d, phis, ms, infos = P.emd_batched(obs, pred, DT, DX, max_iter=30)
+    assert [i["tile"] == 0 for i in infos].count(True) >= 5
+    for b, (nr, _) in enumerate(sizes):
+        ref = P.emd(obs[b], pred[b], DT, DX, max_iter=30, tile=infos[b]["tile"] or (TILE if nr > 8 else PLAIN))
+        check((d[b], phis[b], ms[b], infos[b]), ref, str(sizes[b]))
+
+
+def test_failures_come_back_as_the_streaming_solve_reports_them(P):
+    o, p = pair(64, 256)
+    bad = p.clone()
+    bad[10, 17] = float("nan")
+    for kw in (dict(), dict(tile=TILE)):
+        _, _, _, info = P.emd(o, bad, DT, DX, max_iter=20, check=False, **kw)
+        assert info["status"] == P.EMD_ERR_NONFINITE
+        _, phi, m, info = P.emd(o, p, DT, DX, max_iter=20, check=False, debug_fault=1, **kw)
+        assert info["status"] == P.EMD_ERR_LINESEARCH and info["iters"] == 0
+        assert bool(torch.isfinite(phi).all()) and bool(torch.isfinite(m).all())
+    # a batch reports each gather by itself
+    d, _, _, infos = P.emd_batched([o, o], [bad, p], DT, DX, max_iter=20, check=False)
+    assert infos[0]["status"] == P.EMD_ERR_NONFINITE and infos[1]["status"] == 0
+    check((d[1], None, None, infos[1])[:1] + P.emd(o, p, DT, DX, max_iter=20)[1:], P.emd(o, p, DT, DX, max_iter=20, tile=TILE))
+
+
+def test_a_wait_that_runs_out_is_reported(P):
+    o, p = pair(64, 256)
+    _, _, _, info = P.emd(o, p, DT, DX, max_iter=20, check=False, debug_fault=2)
+    assert info["status"] == P.EMD_ERR_TIMEOUT
+    check(P.emd(o, p, DT, DX, max_iter=20), P.emd(o, p, DT, DX, max_iter=20, tile=TILE))
