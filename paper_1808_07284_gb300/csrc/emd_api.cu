@@ -13,7 +13,7 @@
 #include <vector>
 
 #include "emd_gb300.h"
-#include "emd_chip.cuh"
+#include "emd_chip_w.cuh"
 #include "emd_kernels.cuh"
 #include "emd_lsd.cuh"
 #include "emd_march.cuh"
@@ -87,7 +87,8 @@ const Shape kShapes[] = {EMD_SHAPE(16, 128),          EMD_SHAPE(8, 128),
 #undef EMD_MARCH_SHAPE
 constexpr int kNumShapes = sizeof(kShapes) / sizeof(kShapes[0]);
 constexpr int kTmaShape = 6;         // 13 x 120, two CTAs per SM: the untuned default
-constexpr int kTmaFirst = 6;         // shapes kTmaFirst .. kNumShapes - 1 run persistent solves
+constexpr int kTmaFirst = 6;         // shapes kTmaFirst .. kNumShapes - 1 run persistent solves,
+constexpr int kMarchFirst = 9;       // from here on by the marching pass
 
 // Dynamic shared memory of the plain pass / finalize pass of a shape, of its per-pass
 // TMA kernel (two stages of six (TI + 4) x 128 planes, plus alignment slack) and of its
@@ -368,6 +369,7 @@ struct SolveExtra {
   // and the prepares would be enqueued only after the copies instead of beside them.
   std::function<emd_status()> *stage = nullptr;
   bool no_chip = false;  // not the on-chip solve (what it handed back is solved by the others)
+  int tune_first = kTmaFirst;  // first shape that the autotuner tries
 };
 
 emd_status solve_impl(int B, const float *const *f_obs, const float *const *f_pred, const int *nt,
@@ -379,81 +381,180 @@ emd_status solve_impl(int B, const float *const *f_obs, const float *const *f_pr
 // by side, one cooperative launch per wave.
 struct ChipPlan {
   std::vector<std::vector<emd::ChipJob>> waves;
-  int rows = 0;       // staged rows of the tallest CTA
-  double cost = 0.0;  // estimated time of one pass over every gather, us
+  std::vector<int> form;  // a wave's kernel: emd::ChipForm
+  double cost = 0.0;      // estimated time of one pass over every gather, us
 };
 
-// Estimated us per pass of a wave whose tallest CTA stages n rows.
-double chip_pass_us(int n) { return 3.0 + 0.1 * ((n + emd::kChipWorkers - 1) / emd::kChipWorkers) + 0.02 * n; }
-
-// Whether a gather's state fits on `cap` SMs (and its exchange buffers in its planes).
-bool chip_fits(int nt, int nr, int cap) {
-  const long long strips = (nt + emd::kChipTJ - 1) / emd::kChipTJ;
-  const long long segs = (nr + emd::kChipMaxRows - 4) / (emd::kChipMaxRows - 3);
-  if (strips * segs > cap) return false;
-  const size_t planes = 9 * align256(sizeof(float) * static_cast<size_t>(nr) * ntp_of(nt));
-  return emd::chip_exchange_bytes(std::max(1, (nr + 1) / 2), static_cast<int>(strips), nr, ntp_of(nt)) <= planes;
+// Estimated us per pass of a wave whose tallest CTA stages n rows: the pass boundary and the rows.
+// Measured: 4.2 us at 16 rows, 6.1 at 70 and 7.5 at 123 in the tile pass's form; 9.5 at 123 in the
+// marching pass's; 19.7 at 217 and 24.7 at 327 in tall CTAs.
+double chip_pass_us(int n, bool march) {
+  if (n > emd::kChipMaxRows) return 8.8 + 0.049 * n;
+  return march ? 3.5 + 0.05 * n : 3.6 + 0.033 * n;
 }
 
-// The plan whose estimated pass is shortest, over the rows per warp (more rows put more gathers
-// beside each other, fewer spread one gather over more SMs); no waves when a gather is too large.
-ChipPlan chip_plan(int B, const int *nt, const int *nr, int cap) {
-  ChipPlan best;
-  constexpr int kMaxRun = (emd::kChipMaxRows + emd::kChipWorkers - 1) / emd::kChipWorkers;
-  for (int m = 1; m <= kMaxRun; ++m) {
-    const int hmax = std::min(emd::kChipWorkers * m, emd::kChipMaxRows) - 3;
-    std::vector<emd::ChipJob> g(B);
-    bool fits = true;
-    for (int b = 0; b < B && fits; ++b) {
+// Estimated us per pass of the streaming solves (tile and marching pass) over `cells` cells:
+// about 10 us of decision chain and 5.9 us per million cells, from L2 or from HBM alike.
+double stream_pass_us(double cells) { return 10.0 + 5.9e-6 * cells; }
+
+int chip_strips(int nt) { return (nt + emd::kChipTJ - 1) / emd::kChipTJ; }
+
+// Staged rows of a gather's CTAs at the fewest rows that `cap` CTAs allow (0: it needs more CTAs
+// however tall they are).
+int chip_min_rows(int nt, int nr, int cap) {
+  const int segs = cap / chip_strips(nt);
+  return segs < 1 ? 0 : (nr + segs - 1) / segs + 3;
+}
+
+// Whether a gather's state fits on `cap` SMs, and in its planes what the on-chip solve keeps there:
+// the exchange buffers and, for tall CTAs, their streamed values.
+bool chip_fits(int nt, int nr, int cap, bool march) {
+  const int strips = chip_strips(nt), ntp = ntp_of(nt), rows = chip_min_rows(nt, nr, cap);
+  if (rows == 0 || rows > (march ? emd::kWMaxRows : emd::kChipMaxRows)) return false;
+  const size_t planes = 9 * align256(sizeof(float) * static_cast<size_t>(nr) * ntp);
+  const int segs = std::max(1, (nr + 1) / 2);  // no layout has more
+  if (emd::chip_exchange_bytes(segs, strips, nr, ntp) > planes) return false;
+  if (!march) return true;
+  size_t need = 4 * emd::chip_w_exchange_floats(segs, strips, nr, ntp);
+  if (nr > emd::kChipMaxRows - 3) {
+    const int tall = (nr + emd::kChipMaxRows - 3) / (emd::kChipMaxRows - 2);  // segments of tall CTAs at most
+    need = std::max(need, 4 * (emd::chip_w_exchange_floats(tall, strips, nr, ntp) +
+                               static_cast<size_t>(tall) * strips * emd::chip_w_tall_floats((nr + tall - 1) / tall + 3)));
+  }
+  return need <= planes;
+}
+
+// The plan whose estimated pass is shortest, over the height of the CTAs (taller ones put more
+// gathers beside each other, lower ones spread a gather over more SMs); no waves when a gather
+// does not fit.
+ChipPlan chip_plan(int B, const int *nt, const int *nr, int cap, bool march) {
+  // staged rows of the tallest CTA: whole rows per worker warp, up to what the layout holds
+  std::vector<int> heights;
+  for (int n = emd::kChipWorkers; n < emd::kChipMaxRows; n += emd::kChipWorkers) heights.push_back(n);
+  heights.push_back(emd::kChipMaxRows);
+  if (march)
+    for (int n = emd::kChipMaxRows / emd::kTallWorkers * emd::kTallWorkers + emd::kTallWorkers; n <= emd::kWMaxRows;
+         n += emd::kTallWorkers)
+      heights.push_back(n);
+  auto is_tall = [](int n) { return n > emd::kChipMaxRows; };
+  std::vector<emd::ChipJob> g(B);
+  std::vector<int> order(B), used, rows;
+  std::vector<std::vector<int>> members;
+  auto lay_out = [&](int height) -> double {  // estimated us per pass, or -1
+    for (int b = 0; b < B; ++b) {
       emd::ChipJob &J = g[b];
       J.gather = b;
-      J.strips = (nt[b] + emd::kChipTJ - 1) / emd::kChipTJ;
-      const int nseg = (nr[b] + hmax - 1) / hmax;
+      J.strips = chip_strips(nt[b]);
+      const int nseg = (nr[b] + height - 4) / (height - 3);
       J.h = std::max(nr[b] > 1 ? 2 : 1, (nr[b] + nseg - 1) / nseg);
       J.segs = (nr[b] + J.h - 1) / J.h;
-      const long long group = static_cast<long long>(J.strips) * J.segs;
-      fits = group <= cap;
-      J.group = static_cast<int>(std::min<long long>(group, cap));
+      if (static_cast<long long>(J.strips) * J.segs > cap) return -1.0;
+      J.group = J.strips * J.segs;
+      J.rows = J.h + 3;
+      order[b] = b;
     }
-    if (!fits) continue;
-    std::vector<int> order(B);
-    for (int b = 0; b < B; ++b) order[b] = b;
     std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return g[a].group > g[b].group; });
-    std::vector<int> used, rows;
-    std::vector<std::vector<int>> members;
-    for (int b : order) {  // first fit, largest first
-      size_t w = 0;
-      while (w < used.size() && used[w] + g[b].group > cap) ++w;
+    used.clear();
+    rows.clear();
+    members.clear();
+    size_t open = 0;  // waves before this one are full
+    for (int b : order) {  // first fit, largest first; a wave's gathers share a layout
+      while (open < used.size() && used[open] + g[order.back()].group > cap) ++open;
+      size_t w = open;
+      while (w < used.size() && (used[w] + g[b].group > cap || is_tall(rows[w]) != is_tall(g[b].rows))) ++w;
       if (w == used.size()) {
         used.push_back(0);
-        rows.push_back(0);
+        rows.push_back(g[b].rows);
         members.emplace_back();
       }
       used[w] += g[b].group;
-      rows[w] = std::max(rows[w], g[b].h + 3);
+      rows[w] = std::max(rows[w], g[b].rows);
       members[w].push_back(b);
     }
     double cost = 0.0;
-    for (int n : rows) cost += chip_pass_us(n);
-    if (!best.waves.empty() && cost >= best.cost) continue;
-    best.cost = cost;
-    best.rows = *std::max_element(rows.begin(), rows.end());
-    best.waves.clear();
-    for (const auto &mem : members) {
-      best.waves.emplace_back();
-      for (int b : mem)
-        for (int seg = 0; seg < g[b].segs; ++seg)
-          for (int strip = 0; strip < g[b].strips; ++strip) {
-            emd::ChipJob J = g[b];
-            J.seg = seg;
-            J.strip = strip;
-            J.i0 = seg * g[b].h;
-            J.h = std::min(g[b].h, nr[b] - J.i0);
-            best.waves.back().push_back(J);
-          }
-    }
+    for (int n : rows) cost += chip_pass_us(n, march);
+    return cost;
+  };
+  ChipPlan plan;
+  int best = 0;
+  for (const int height : heights) {
+    const double cost = lay_out(height);
+    if (cost < 0.0 || (best && cost >= plan.cost)) continue;
+    best = height;
+    plan.cost = cost;
   }
-  return best;
+  if (!best) return plan;
+  lay_out(best);
+  for (size_t w = 0; w < members.size(); ++w) {
+    plan.waves.emplace_back();
+    plan.form.push_back(!march ? emd::kChipTile : is_tall(rows[w]) ? emd::kChipMarchTall : emd::kChipMarch);
+    for (int b : members[w])
+      for (int seg = 0; seg < g[b].segs; ++seg)
+        for (int strip = 0; strip < g[b].strips; ++strip) {
+          emd::ChipJob J = g[b];
+          J.seg = seg;
+          J.strip = strip;
+          J.i0 = seg * g[b].h;
+          J.h = std::min(g[b].h, nr[b] - J.i0);
+          plan.waves.back().push_back(J);
+        }
+  }
+  return plan;
+}
+
+// Copies of the elements `idx` of an array (empty for a null one).
+template <class T>
+std::vector<T> pick(const T *a, const std::vector<int> &idx) {
+  std::vector<T> v;
+  if (a)
+    for (int b : idx) v.push_back(a[b]);
+  return v;
+}
+
+// The gathers of a batch that are solved on chip (`on`, in order) and their plan.  Of three ways
+// the one whose estimated pass is shortest: every gather that fits, only those whose own pass
+// there is shorter than their share of a streamed pass, or none.
+//
+// *march: the form whose rounding the streaming solve of this batch has, the tile pass up to
+// about 1.4 million cells (and for thin gathers), where the autotuner takes it, the marching pass
+// above.  Measured crossing, single gathers: 400 x 3000 and 648 x 2000 take the tile pass, 400 x
+// 3500 and 300 x 5000 the march.
+ChipPlan choose_on_chip(int B, const int *nt, const int *nr, int cap, bool whole_only, std::vector<int> &on,
+                        bool *march) {
+  double cells = 0.0;
+  int receivers = 0;
+  for (int b = 0; b < B; ++b) {
+    cells += static_cast<double>(nt[b]) * nr[b];
+    receivers = std::max(receivers, nr[b]);
+  }
+  *march = cells >= 1.4e6 && receivers > 8;
+  ChipPlan plan;
+  double best = stream_pass_us(cells);
+  on.clear();
+  size_t tried = 0;
+  for (const bool all : {true, false}) {
+    std::vector<int> sub;
+    double left = cells;
+    for (int b = 0; b < B; ++b) {
+      const double n = static_cast<double>(nt[b]) * nr[b];
+      if (!chip_fits(nt[b], nr[b], cap, *march)) continue;
+      const int rows = chip_min_rows(nt[b], nr[b], cap);
+      if (!all && rows > emd::kChipMaxRows && chip_pass_us(rows, *march) > stream_pass_us(n) - stream_pass_us(0.0))
+        continue;
+      sub.push_back(b);
+      left -= n;
+    }
+    const int nb = static_cast<int>(sub.size());
+    if (nb == 0 || sub.size() == tried || (whole_only && nb < B)) continue;
+    tried = sub.size();
+    ChipPlan q = chip_plan(nb, pick(nt, sub).data(), pick(nr, sub).data(), cap, *march);
+    const double cost = q.cost + (nb < B ? stream_pass_us(left) : 0.0);
+    if (q.waves.empty() || cost >= best) continue;
+    best = cost;
+    on = std::move(sub);
+    plan = std::move(q);
+  }
+  return plan;
 }
 
 // Tile-shape autotuner of the TMA pass.  The first default-tile solve of a (device,
@@ -470,7 +571,7 @@ int autotune_shape(int B, const float *const *f_obs, const float *const *f_pred,
                    size_t ws_bytes, cudaStream_t stream, const SolveExtra &x) {
   int dev = 0;
   (void)cudaGetDevice(&dev);
-  std::vector<long long> key = {dev, B};
+  std::vector<long long> key = {dev, B, x.tune_first};
   for (int b = 0; b < B; ++b) {
     key.push_back(nt[b]);
     key.push_back(nr[b]);
@@ -504,9 +605,9 @@ int autotune_shape(int B, const float *const *f_obs, const float *const *f_pred,
       return -1.0f;
     return ms;
   };
-  int best = kTmaShape;
+  int best = std::max(kTmaShape, x.tune_first);
   float best_t = 0.0f;
-  for (int shape = kTmaFirst; shape < kNumShapes; ++shape) {
+  for (int shape = x.tune_first; shape < kNumShapes; ++shape) {
     (void)timed(shape, 4);  // first use: module load, attribute set-up
     const float t1 = timed(shape, 8), t2 = timed(shape, 40);
     if (t1 < 0.0f || t2 < 0.0f) continue;
@@ -604,16 +705,25 @@ emd_status solve_on_chip(int B, const float *const *f_obs, const float *const *f
                          size_t ws_bytes, cudaStream_t stream, const SolveExtra &x, const Layout &L,
                          const ChipPlan &plan, bool *launched) {
   *launched = false;
-  void (*fn)(const Ctl, const emd::ChipJobs) =
-      p.norm == EMD_NORM_ISO ? emd::k_solve_chip<true> : emd::k_solve_chip<false>;
+  const bool iso = p.norm == EMD_NORM_ISO;
+  using Kernel = void (*)(const Ctl, const emd::ChipJobs);
+  const Kernel fns[3] = {iso ? emd::k_solve_chip<true, 0> : emd::k_solve_chip<false, 0>,
+                         iso ? emd::k_solve_chip<true, 1> : emd::k_solve_chip<false, 1>,
+                         iso ? emd::k_solve_chip<true, 2> : emd::k_solve_chip<false, 2>};
   const size_t smem = emd::kChipSmem;
-  int dev = 0, coop = 0, per_sm = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop ||
-      cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) !=
-          cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, emd::kChipThreads, smem) != cudaSuccess ||
-      per_sm < 1) {
+  int dev = 0, coop = 0;
+  bool fits = cudaGetDevice(&dev) == cudaSuccess &&
+              cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) == cudaSuccess && coop;
+  for (int form = 0; form < 3 && fits; ++form) {
+    int per_sm = 0;
+    if (std::find(plan.form.begin(), plan.form.end(), form) == plan.form.end()) continue;
+    fits = cudaFuncSetAttribute(fns[form], cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                static_cast<int>(smem)) == cudaSuccess &&
+           cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fns[form], (emd::chip_workers(form) + 1) * 32, smem) ==
+               cudaSuccess &&
+           per_sm >= 1;
+  }
+  if (!fits) {
     (void)cudaGetLastError();
     return EMD_OK;
   }
@@ -642,7 +752,8 @@ emd_status solve_on_chip(int B, const float *const *f_obs, const float *const *f
     const emd_status s = enqueue();
     if (s != EMD_OK) return s;
   }
-  for (const auto &wave : plan.waves) {
+  for (size_t w = 0; w < plan.waves.size(); ++w) {
+    const auto &wave = plan.waves[w];
     emd::ChipJobs jobs{};
     std::copy(wave.begin(), wave.end(), jobs.job);
     if (x.ready)
@@ -651,8 +762,9 @@ emd_status solve_on_chip(int B, const float *const *f_obs, const float *const *f
           EMD_CK(cudaStreamWaitEvent(stream, x.ready[wave[i].gather], 0));
     Ctl cctl = ctl;
     void *args[] = {&cctl, &jobs};
-    EMD_CK(cudaLaunchCooperativeKernel(reinterpret_cast<void *>(fn), dim3(static_cast<unsigned>(wave.size())),
-                                       dim3(emd::kChipThreads), args, smem, stream));
+    EMD_CK(cudaLaunchCooperativeKernel(reinterpret_cast<void *>(fns[plan.form[w]]),
+                                       dim3(static_cast<unsigned>(wave.size())), dim3(static_cast<unsigned>((emd::chip_workers(plan.form[w]) + 1) * 32)), args,
+                                       smem, stream));
   }
   std::vector<State> hs(B);
   int h_flags[2] = {0, 0};
@@ -684,9 +796,50 @@ emd_status solve_on_chip(int B, const float *const *f_obs, const float *const *f
   return first;
 }
 
-// Estimated us per pass of the streaming solves (tile and marching pass) over `cells` cells:
-// about 10 us of decision chain and 5.9 us per million cells, from L2 or from HBM alike.
-double stream_pass_us(double cells) { return 10.0 + 5.9e-6 * cells; }
+// The gathers `on` of a batch on chip, then the others by the streaming solve, in the same workspace.
+emd_status solve_split(int B, const float *const *f_obs, const float *const *f_pred, const int *nt, const int *nr,
+                       const double *dt, const double *dx, const emd_params &p, float *const *phi,
+                       float *const *m, emd_result *results, void *ws, size_t ws_bytes, cudaStream_t stream,
+                       const SolveExtra &x, const std::vector<int> &on, const ChipPlan &plan, bool march,
+                       bool *launched) {
+  std::vector<int> off;
+  for (int b = 0; b < B; ++b)
+    if (!std::binary_search(on.begin(), on.end(), b)) off.push_back(b);
+  for (const bool chip : {true, false}) {
+    const std::vector<int> &idx = chip ? on : off;
+    const int nb = static_cast<int>(idx.size());
+    const auto a_nt = pick(nt, idx), a_nr = pick(nr, idx);
+    const auto a_dt = pick(dt, idx), a_dx = pick(dx, idx);
+    const auto a_obs = pick(f_obs, idx), a_pred = pick(f_pred, idx);
+    const auto a_phi = pick(phi, idx), a_m = pick(m, idx);
+    const auto a_pi = pick(x.phi_init, idx), a_mi = pick(x.m_init, idx);
+    const auto a_ready = pick(x.ready, idx);
+    SolveExtra y = x;
+    y.phi_init = x.phi_init ? a_pi.data() : nullptr;
+    y.m_init = x.m_init ? a_mi.data() : nullptr;
+    y.ready = x.ready ? a_ready.data() : nullptr;
+    std::vector<emd_result> res(nb);
+    emd_status s;
+    if (chip) {
+      s = solve_on_chip(nb, a_obs.data(), a_pred.data(), a_nt.data(), a_nr.data(), a_dt.data(), a_dx.data(), p,
+                        a_phi.data(), a_m.data(), res.data(), ws, ws_bytes, stream, y,
+                        layout(nb, a_nt.data(), a_nr.data()), plan, launched);
+      if (!*launched) return s;
+    } else {
+      y.no_chip = true;
+      y.tune_first = march ? kMarchFirst : kTmaFirst;
+      s = solve_impl(nb, a_obs.data(), a_pred.data(), a_nt.data(), a_nr.data(), a_dt.data(), a_dx.data(), &p,
+                     a_phi.data(), a_m.data(), res.data(), ws, ws_bytes, stream, y);
+    }
+    for (int i = 0; i < nb; ++i) results[idx[i]] = res[i];
+    if (s == EMD_ERR_TIMEOUT)
+      for (int b = 0; b < B; ++b) results[b].status = s;
+    if (s == EMD_ERR_CUDA || s == EMD_ERR_TIMEOUT) return s;
+  }
+  for (int b = 0; b < B; ++b)
+    if (results[b].status != EMD_OK) return static_cast<emd_status>(results[b].status);
+  return EMD_OK;
+}
 
 emd_status solve_impl(int B, const float *const *f_obs, const float *const *f_pred, const int *nt,
                       const int *nr, const double *dt, const double *dx, const emd_params *pp,
@@ -716,73 +869,17 @@ emd_status solve_impl(int B, const float *const *f_obs, const float *const *f_pr
   const bool resident = p.launch_mode == 0 && p.tile == 0 && max_cells <= emd::kResidentMaxCells;
   // Gathers whose state fits on the chip are solved there; the others of the batch stream.
   if (p.tile == 0 && p.launch_mode == 0 && !resident && !x.no_chip) {
-    const int cap = std::min(sm_count(), emd::kChipMaxCtas);
-    std::vector<int> on, off;
-    double on_cells = 0.0;
-    for (int b = 0; b < B; ++b) {
-      if (chip_fits(nt[b], nr[b], cap)) {
-        on.push_back(b);
-        on_cells += static_cast<double>(nt[b]) * nr[b];
-      } else {
-        off.push_back(b);
-      }
-    }
-    if (!on.empty() && !(p.trace && !off.empty())) {
-      auto pick = [&](const auto *a, const std::vector<int> &idx) {
-        std::vector<std::decay_t<decltype(a[0])>> v;
-        if (a)
-          for (int b : idx) v.push_back(a[b]);
-        return v;
-      };
-      const auto on_nt = pick(nt, on), on_nr = pick(nr, on);
-      const ChipPlan plan = chip_plan(static_cast<int>(on.size()), on_nt.data(), on_nr.data(), cap);
-      const double streamed = off.empty() ? stream_pass_us(on_cells) : stream_pass_us(on_cells) - stream_pass_us(0.0);
-      if (!plan.waves.empty() && plan.cost < streamed) {
-        bool launched = false;
-        if (off.empty()) {
-          const emd_status s = solve_on_chip(B, f_obs, f_pred, nt, nr, dt, dx, p, phi, m, results, ws,
-                                             ws_bytes, stream, x, L, plan, &launched);
-          if (launched) return s;
-        } else {  // two batches, one after the other in the same workspace
-          emd_status st[2] = {EMD_OK, EMD_OK};
-          bool done = true;
-          for (int part = 0; part < 2 && done; ++part) {
-            const std::vector<int> &idx = part ? off : on;
-            const auto a_nt = pick(nt, idx), a_nr = pick(nr, idx);
-            const auto a_dt = pick(dt, idx), a_dx = pick(dx, idx);
-            const auto a_obs = pick(f_obs, idx), a_pred = pick(f_pred, idx);
-            const auto a_phi = pick(phi, idx), a_m = pick(m, idx);
-            const auto a_pi = pick(x.phi_init, idx), a_mi = pick(x.m_init, idx);
-            const auto a_ready = pick(x.ready, idx);
-            SolveExtra y = x;
-            y.phi_init = x.phi_init ? a_pi.data() : nullptr;
-            y.m_init = x.m_init ? a_mi.data() : nullptr;
-            y.ready = x.ready ? a_ready.data() : nullptr;
-            const int nb = static_cast<int>(idx.size());
-            std::vector<emd_result> res(nb);
-            if (part == 0) {
-              const Layout La = layout(nb, a_nt.data(), a_nr.data());
-              st[0] = solve_on_chip(nb, a_obs.data(), a_pred.data(), a_nt.data(), a_nr.data(), a_dt.data(),
-                                    a_dx.data(), p, a_phi.data(), a_m.data(), res.data(), ws, ws_bytes,
-                                    stream, y, La, plan, &launched);
-              if (!launched) done = false;
-            } else {
-              y.no_chip = true;
-              st[1] = solve_impl(nb, a_obs.data(), a_pred.data(), a_nt.data(), a_nr.data(), a_dt.data(),
-                                 a_dx.data(), &p, a_phi.data(), a_m.data(), res.data(), ws, ws_bytes, stream, y);
-            }
-            if (done)
-              for (int i = 0; i < nb; ++i) results[idx[i]] = res[i];
-            for (emd_status s : {st[part]})
-              if (s == EMD_ERR_CUDA || s == EMD_ERR_TIMEOUT) return s;
-          }
-          if (done) {
-            for (int b = 0; b < B; ++b)
-              if (results[b].status != EMD_OK) return static_cast<emd_status>(results[b].status);
-            return EMD_OK;
-          }
-        }
-      }
+    std::vector<int> on;
+    bool march = false, launched = false;
+    const ChipPlan plan = choose_on_chip(B, nt, nr, std::min(sm_count(), emd::kChipMaxCtas), p.trace != nullptr, on,
+                                         &march);
+    if (!on.empty()) {
+      const emd_status s = static_cast<int>(on.size()) == B
+                               ? solve_on_chip(B, f_obs, f_pred, nt, nr, dt, dx, p, phi, m, results, ws, ws_bytes,
+                                               stream, x, L, plan, &launched)
+                               : solve_split(B, f_obs, f_pred, nt, nr, dt, dx, p, phi, m, results, ws, ws_bytes,
+                                             stream, x, on, plan, march, &launched);
+      if (launched) return s;
     }
   }
   if (p.tile == 0 && !resident && si == kTmaShape && !x.no_tune)

@@ -19,7 +19,8 @@
 // u^{k+1}, div u^{k+1}, p, q and the linesearch sums of row r + 1.  The last row of a run needs
 // u^{k+1} of the next run's first row and the first row needs phi and p, q of the last row
 // above it, so these are taken after three barriers of the workers.  Every cell's arithmetic
-// and rounding are those of the tile pass (emd_pass_tma.cuh), so both give the same iterates.
+// and rounding are those of the tile pass (emd_pass_tma.cuh), so both give the same iterates;
+// emd_chip_w.cuh has the same solve with the arithmetic of the marching pass.
 //
 // Pass boundary.  A CTA adds its sums to FP64 accumulators in L2 and counts itself done; the
 // decider warp of every CTA waits for the count, reads the totals and takes the same decision,
@@ -34,12 +35,12 @@
 
 namespace emd {
 
-constexpr int kChipWorkers = 15;                        // worker warps of a CTA
-constexpr int kChipThreads = (kChipWorkers + 1) * 32;   // and the decider warp
+constexpr int kChipWorkers = 15;                        // worker warps of a CTA (and a decider warp)
 constexpr int kChipTmemCols = 128;                      // tensor memory columns of a warp
 constexpr int kChipRowCols = 12;                        // ... of one row: ux, ut, phi
 constexpr int kChipMaxRows = 128;                       // staged rows of a CTA at most (shared memory)
 static_assert((kChipMaxRows + kChipWorkers - 1) / kChipWorkers * kChipRowCols <= kChipTmemCols, "a run's rows");
+
 constexpr int kChipTJ = 120;                            // owned time samples of a strip
 constexpr int kChipSets = 3;                            // accumulator sets, used in turn
 constexpr int kChipVals = 8;                            // sums of a pass
@@ -47,7 +48,8 @@ constexpr int kChipSpread = 8;                          // copies of each accumu
 
 // One CTA's part of a gather.
 struct ChipJob {
-  int gather, seg, strip, segs, strips, i0, h, group;  // group: CTAs of the gather
+  int gather, seg, strip, segs, strips, i0, h;
+  int group, rows;  // CTAs of the gather, staged rows of its tallest CTA
 };
 constexpr int kChipMaxCtas = 160;  // CTAs of a launch at most (its jobs are a kernel argument)
 struct ChipJobs {
@@ -133,6 +135,19 @@ __device__ __forceinline__ void sts4(unsigned a, const Q4 &v) {
 }
 __device__ __forceinline__ void sts1(unsigned a, float v) {
   asm volatile("st.shared.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
+}
+__device__ __forceinline__ float lds1(unsigned a) {
+  float v;
+  asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+  return v;
+}
+// Eight bytes of shared memory (a value written twice) as both pairs.
+template <unsigned OFF = 0>
+__device__ __forceinline__ Q4 lds_pair(unsigned a) {
+  Q4 v;
+  asm volatile("ld.shared.b64 %0, [%1+%2];" : "=l"(v.a) : "r"(a), "n"(OFF) : "memory");
+  v.b = v.a;
+  return v;
 }
 
 // x[j] - x[j - 1] over the lane's four samples; `left` is the last sample of the lane before.
@@ -221,16 +236,18 @@ struct BoolConst {
   static constexpr bool value = B;
 };
 
+// Barriers of a CTA of NW worker warps: the workers alone, or with the decider warp.
+template <int NW = kChipWorkers>
 __device__ __forceinline__ void bar_workers() {
-  asm volatile("bar.sync 1, %0;\n" ::"n"(kChipWorkers * 32) : "memory");
+  asm volatile("bar.sync 1, %0;\n" ::"n"(NW * 32) : "memory");
 }
-template <int ID>
+template <int ID, int NW = kChipWorkers>
 __device__ __forceinline__ void bar_all() {
-  asm volatile("bar.sync %0, %1;\n" ::"n"(ID), "n"(kChipThreads) : "memory");
+  asm volatile("bar.sync %0, %1;\n" ::"n"(ID), "n"((NW + 1) * 32) : "memory");
 }
-template <int ID>
+template <int ID, int NW = kChipWorkers>
 __device__ __forceinline__ void bar_all_arrive() {
-  asm volatile("bar.arrive %0, %1;\n" ::"n"(ID), "n"(kChipThreads) : "memory");
+  asm volatile("bar.arrive %0, %1;\n" ::"n"(ID), "n"((NW + 1) * 32) : "memory");
 }
 
 // Warp totals of eight values: lane l ends with the total of value l & 7 (all 32 lanes summed,
@@ -276,7 +293,7 @@ struct ChipShared {
   // each value four times, so that a 16-byte load gives a Q4: alpha, coef, theta,
   // 1 / (1 + eps alpha) of the pass, then 1/dx, 1/dt
   alignas(16) float sc[6][4];
-  float part[16][kChipVals];                 // warp totals of a pass (the last row stays zero)
+  float part[16][kChipVals];                 // warp totals of a pass (zero for warps that are not there)
   double dpart[16][4];                       // warp totals of the balancing sums
 };
 
@@ -286,6 +303,7 @@ struct ChipShared {
 // has read by now and which is added to again two passes on.  False when the bounded wait ran
 // out.  (Eight copies: two loads and three FP64 additions to read a total, each addition about
 // 70 cycles of a chain that every CTA waits for.)
+template <int NW>
 __device__ __forceinline__ bool chip_exchange(const Ctl &c, State *st, double *acc, int set, int cta,
                                               int group, unsigned step, bool adds, double x, double &v) {
   const int lane = threadIdx.x & 31;
@@ -294,7 +312,7 @@ __device__ __forceinline__ bool chip_exchange(const Ctl &c, State *st, double *a
   __syncwarp();
   if (lane == 0 && c.debug_fault != 2) red_release_add(&st->tiles_done, 1u);
   if (!__all_sync(0xffffffffu, wait_count(&st->tiles_done, step * static_cast<unsigned>(group)))) return false;
-  bar_all_arrive<3>();  // the workers may fetch their halos
+  bar_all_arrive<3, NW>();  // the workers may fetch their halos
   static_assert(kChipSpread == 8 && kChipVals == 8, "two copies per lane");
   const double x0 = __ldcg(a + lane), x1 = __ldcg(a + 32 + lane);  // copies lane / 8 and 4 + lane / 8
   v = sum_groups(x0 + x1);
@@ -375,6 +393,7 @@ __device__ __forceinline__ int quick_decide(const Ctl &c, const QuickPrep &p, do
   return (known & below) == below ? __ffs(pass) - 1 : -1;
 }
 
+// The prox of four cells (prox_cell of emd_kernels.cuh).
 template <bool ISO>
 __device__ __forceinline__ void chip_prox(const Q4 &ux, const Q4 &ut, const Q4 &gx, const Q4 &gt,
                                           float alpha, const Q4 &al, const Q4 &inv, Q4 &nx, Q4 &nt) {
@@ -385,7 +404,12 @@ __device__ __forceinline__ void chip_prox(const Q4 &ux, const Q4 &ut, const Q4 &
     un4(vx, x);
     un4(vt, t);
 #pragma unroll
-    for (int q = 0; q < 4; ++q) prox_cell(x[q], t[q], alpha, iv, true, a[q], b[q]);
+    for (int q = 0; q < 4; ++q) {
+      const float n = sqrtf(__fmaf_rn(x[q], x[q], __fmul_rn(t[q], t[q])));
+      const float s = n > alpha ? (1.0f - alpha / n) * iv : 0.0f;
+      a[q] = s * x[q];
+      b[q] = s * t[q];
+    }
     nx = q4(a[0], a[1], a[2], a[3]);
     nt = q4(b[0], b[1], b[2], b[3]);
   } else {
@@ -394,560 +418,602 @@ __device__ __forceinline__ void chip_prox(const Q4 &ux, const Q4 &ut, const Q4 &
   }
 }
 
-template <bool ISO>
-__global__ void __launch_bounds__(kChipThreads, 1) k_solve_chip(const Ctl c, const __grid_constant__ ChipJobs jobs) {
-  extern __shared__ float4 dyn4[];
-  __shared__ ChipShared sh;
-  const ChipJob J = jobs.job[blockIdx.x];
-  const Shot &S = c.shots[J.gather];
-  State *st = c.states + J.gather;
-  const int lane = threadIdx.x & 31, warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0);
-  const int nr = S.nr, nt = S.nt, ntp = S.ntp;
-  const int n = J.h + 3, cta = J.seg * J.strips + J.strip;
-  const float rdx = S.rdx, rdt = S.rdt;
-  double *acc = acc_of(c, J.gather);
-  static_assert(kChipSets * kChipVals <= kAccBufs * kAcc, "the accumulator sets of a gather");
+// What the warps of a CTA share: its part of the gather and its storage.
+struct ChipCta {
+  const Ctl &c;
+  const ChipJob &J;
+  const Shot &S;
+  ChipShared &sh;
+  State *st;
+  int lane, warp, nr, nt, ntp;
+  int n, cta;        // staged rows, index in the group
+  int ra, rb;        // rows of this warp's run
+  int gj0;           // time index of this lane's first sample
+  uint32_t taddr;    // this warp's tensor memory
+  unsigned smem;     // this lane's column of the first 512-byte row of shared memory
+};
 
+// The balancing sums over a lane's cells: f, f^2, |Pcal| + |Pobs| and Pcal - Pobs, each to about
+// 48 bits in FP32 pairs.
+struct BalanceSums {
+  Sum2 f, f2, ab;
+  float de = 0.0f;  // rounding errors of the differences f = Pcal - Pobs
+  __device__ __forceinline__ void add(float po, float pp) {
+    float d, e;
+    two_sum(pp, -po, d, e);
+    de += e;
+    f.add(d);
+    const float dd = d * d;
+    f2.add(dd);
+    f2.lo += fmaf(d, d, -dd);
+    two_sum(fabsf(pp), fabsf(po), d, e);
+    ab.add(d);
+    ab.lo += e;
+  }
+  __device__ __forceinline__ void store(const ChipCta &X) {
+    const double t0 = warp_sum_d(f.value()), t1 = warp_sum_d(f2.value()), t2 = warp_sum_d(ab.value());
+    const double t3 = warp_sum_d(f.value() + static_cast<double>(de));
+    if (X.lane < 4) X.sh.dpart[X.warp][X.lane] = X.lane == 0 ? t0 : X.lane == 1 ? t1 : X.lane == 2 ? t2 : t3;
+  }
+};
+
+// u of a warm start at (gi, gj), plane 0 (x) or 1 (t); the outer faces carry none.
+__device__ __forceinline__ float chip_init_flux(const ChipCta &X, int plane, int gi, int gj) {
+  const bool in = gi >= 0 && gi < X.nr && gj >= 0 && gj < X.nt && (plane ? gj > 0 : gi > 0);
+  return in ? X.S.m_init[(static_cast<size_t>(plane) * X.nr + gi) * X.nt + gj] : 0.0f;
+}
+
+// An owned row of the solution to the caller's arrays, and its terms of the gap sums (up: phi of
+// the row above, gtv: phi[j] - phi[j - 1]).
+template <bool ISO>
+__device__ __forceinline__ void chip_output_row(const ChipCta &X, bool vec, int gi, const Q4 &ux4, const Q4 &ut4,
+                                                const Q4 &ph4, const Q4 &up, const Q4 &gtv, const Q4 &f4,
+                                                Sum2 (&t)[4]) {
+  const Shot &S = X.S;
+  float ph[4], pu[4], gt[4], ux[4], ut[4], fb[4];
+  un4(ph4, ph);
+  un4(up, pu);
+  un4(gtv, gt);
+  un4(ux4, ux);
+  un4(ut4, ut);
+  un4(f4, fb);
+  const size_t g = static_cast<size_t>(gi) * X.nt + X.gj0, m_t = static_cast<size_t>(X.nr) * X.nt;
+  if (vec && X.gj0 < X.nt) {
+    *reinterpret_cast<float4 *>(S.phi_out + g) = make_float4(ph[0], ph[1], ph[2], ph[3]);
+    *reinterpret_cast<float4 *>(S.m_out + g) = make_float4(ux[0], ux[1], ux[2], ux[3]);
+    *reinterpret_cast<float4 *>(S.m_out + m_t + g) = make_float4(ut[0], ut[1], ut[2], ut[3]);
+  }
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int gj = X.gj0 + q;
+    if (gj >= X.nt) continue;
+    if (!vec) {
+      S.phi_out[g + q] = ph[q];
+      S.m_out[g + q] = ux[q];
+      S.m_out[m_t + g + q] = ut[q];
+    }
+    const float gx = gi > 0 ? (ph[q] - pu[q]) * S.rdx : 0.0f, gtt = gj > 0 ? gt[q] * S.rdt : 0.0f;
+    gap_terms(t, ux[q], ut[q], ph[q], fb[q], gx, gtt, ISO);
+  }
+}
+// Whether rows of the outputs can be written sixteen bytes at a time.
+__device__ __forceinline__ bool chip_vec_out(const ChipCta &X) {
+  return (X.nt & 3) == 0 &&
+         ((reinterpret_cast<uintptr_t>(X.S.phi_out) | reinterpret_cast<uintptr_t>(X.S.m_out)) & 15u) == 0;
+}
+// This warp's gap sums for the decider: the high and the low parts as eight values.
+__device__ __forceinline__ void chip_store_gap(const ChipCta &X, Sum2 (&t)[4]) {
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    t[q].warp_total();
+    if (X.lane == 0) {
+      X.sh.part[X.warp][q] = t[q].hi;
+      X.sh.part[X.warp][4 + q] = t[q].lo;
+    }
+  }
+}
+
+// A lane's samples: whether f of each is needed (one halo sample more on the left than right), and
+// 1/dt of the face left of each, 0 for outer faces and samples that nobody needs.
+struct ChipLane {
+  bool use[4];
+  float rm[4];
+  bool own;  // lanes 1..30 own their samples, 0 and 31 only feed their neighbours
+};
+__device__ __forceinline__ ChipLane chip_lane(const ChipCta &X) {
+  ChipLane l;
+  const int lane = X.lane;
+  l.own = lane >= 1 && lane <= 30;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int gj = X.gj0 + q;
+    l.use[q] = gj >= 0 && gj < X.nt && (lane > 0 || q >= 2) && (lane < 31 || q == 0);
+    l.rm[q] = gj > 0 && gj < X.nt && (lane > 0 || q == 3) && (lane < 31 || q == 0) ? X.S.rdt : 0.0f;
+  }
+  return l;
+}
+
+// Warp totals of a pass's eight packed sums (the two lanes that only feed neighbours leave theirs
+// out), for the decider.
+__device__ __forceinline__ void chip_store_sums(const ChipCta &X, const f32x2 (&v)[8], bool own) {
+  float t[8];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    float x, y;
+    upk(v[q], x, y);
+    t[q] = own ? x + y : 0.0f;
+  }
+  const float tot = warp_sum8(t);
+  if (X.lane < 8) X.sh.part[X.warp][X.lane] = tot;
+}
+
+// The decider warp: the balancing constants, every pass's decision and the gather's final state.
+template <int NW>
+__device__ __forceinline__ void chip_decider(const ChipCta &X) {
+  const Ctl &c = X.c;
+  const ChipJob &J = X.J;
+  const Shot &S = X.S;
+  ChipShared &sh = X.sh;
+  State *const st = X.st;
+  const int lane = X.lane, nr = X.nr, nt = X.nt, cta = X.cta;
+  const float rdx = S.rdx, rdt = S.rdt;
+  double *const acc = acc_of(c, J.gather);
+  static_assert(kChipSets * kChipSpread * kChipVals <= kAccBufs * kSpread * kAcc, "a gather's accumulators");
+  // the balancing sums: f, f^2, |Pcal| + |Pobs|, Pcal - Pobs
+  bar_all<2, NW>();
+  double v = 0.0;
+  if ((lane & 7) < 4) {
+    double p[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) p[i] = sh.dpart[(lane >> 3) + 4 * i][lane & 7];
+    v = (p[0] + p[1]) + (p[2] + p[3]);
+  }
+  v = sum_groups(v);
+  unsigned step = 1;
+  int set = 0;
+  bool ok = chip_exchange<NW>(c, st, acc, set, cta, J.group, step, lane < 8, v, v);
+  if (!ok) bar_all_arrive<3, NW>();
+  DecidePrep pr;
+  pr.k = 0;
+  double m4[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) m4[q] = __shfl_sync(0xffffffffu, v, q);
+  const double N = static_cast<double>(nr) * nt;
+  const double fmean = c.balance ? m4[0] / N : 0.0;
+  pr.fnorm = sqrt(fmax(m4[1] - 2.0 * fmean * m4[0] + N * fmean * fmean, 0.0));
+  pr.alpha = c.alpha0 > 0.0 ? c.alpha0 : (c.linesearch ? 1.0 / sqrt(c.delta * S.lambda) : 1.0 / sqrt(S.lambda));
+  pr.beta_fixed = 1.0 / (S.lambda * pr.alpha);
+  pr.theta = 1.0;
+  pr.coef = 0.0;  // pass 0: phi^0 is the initial potential
+  // the values of the next pass, each written four times (lane 4 q + i: copy i of value q)
+  auto publish_sc = [&](float alpha, float coef, float theta, float inv) {
+    const int q = lane >> 2;
+    if (lane < 16) sh.sc[q][lane & 3] = q == 0 ? alpha : q == 1 ? coef : q == 2 ? theta : inv;
+  };
+  publish_sc(static_cast<float>(pr.alpha), 0.0f, 1.0f, 1.0f / (1.0f + static_cast<float>(c.eps * pr.alpha)));
+  if (lane >= 16 && lane < 24) sh.sc[lane >> 2][lane & 3] = lane < 20 ? rdx : rdt;
+  if (lane == 0) {
+    sh.fmean = static_cast<float>(fmean);
+    if (!ok) sh.bad = 1;
+  }
+  bar_all<4, NW>();
+  int trials = 0;
+  double r_feas = -1.0, r_step = -1.0;
+  bool done = false;
+  int status = ST_OK;
+  const bool quick = c.linesearch && c.debug_fault != 1;
+  while (ok && !done) {
+    decide_prep_lanes(c, pr);  // overlaps the pass
+    const QuickPrep qp = quick_prep(pr);
+    bar_all<2, NW>();
+    const double mine = chip_block_total(sh);
+    ++step;
+    set = (set + 1) % kChipSets;
+    ok = chip_exchange<NW>(c, st, acc, set, cta, J.group, step, lane < 16, mine, v);
+    if (!ok) {
+      bar_all_arrive<3, NW>();
+      if (lane == 0) sh.bad = 1;
+      bar_all<4, NW>();
+      break;
+    }
+    const int w = quick && !pr.check ? quick_decide(c, qp, v) : -1;
+    if (w >= 0) {
+      constexpr unsigned FULL = 0xffffffffu;
+      publish_sc(__shfl_sync(FULL, pr.alpha_lf, w), __shfl_sync(FULL, pr.coef_lf, w),
+                 __shfl_sync(FULL, pr.theta_lf, w), __shfl_sync(FULL, pr.inv_lf, w));
+      done = pr.k + 1 >= c.max_iter;
+      if (lane == 0) sh.done = done;
+      bar_all<4, NW>();
+      trials += w + 1;
+      if (c.trace && cta == 0) {
+        Decision o;
+        o.alpha = __shfl_sync(FULL, pr.alpha_l, w);
+        o.theta = __shfl_sync(FULL, pr.s_lane, w);
+        o.trials_now = w + 1;
+        const double ppp = __shfl_sync(FULL, v, 0);
+        if (lane == 0) write_trace(c, J.gather, pr.k, o, ppp, pr.fnorm);
+      }
+      pr.alpha = __shfl_sync(FULL, pr.alpha_l, w);
+      pr.theta = __shfl_sync(FULL, pr.s_lane, w);
+      pr.coef = __shfl_sync(FULL, pr.coef_l, w);
+      ++pr.k;
+    } else {
+      double a_[9];
+#pragma unroll
+      for (int q = 0; q < 6; ++q) a_[q] = __shfl_sync(0xffffffffu, v, q);
+      a_[6] = 0.0;
+      a_[7] = __shfl_sync(0xffffffffu, v, 6);
+      a_[8] = __shfl_sync(0xffffffffu, v, 7);
+      const Decision o = decide_core(c, pr, a_);
+      trials += o.trials_now;
+      done = o.done;
+      status = o.status;
+      if (o.status == ST_OK) publish_sc(o.alpha_f, o.coef_f, o.theta_f, o.inv_f);
+      if (lane == 0) {
+        sh.status = o.status;
+        sh.done = o.done;
+      }
+      bar_all<4, NW>();
+      if (cta == 0 && lane == 0) write_trace(c, J.gather, pr.k, o, a_[0], pr.fnorm);
+      if (o.checked && cta == 0) residuals(pr, a_, r_feas, r_step);
+      if (o.status == ST_OK) {
+        pr.k = o.k_new;
+        pr.alpha = o.alpha;
+        pr.theta = o.theta;
+        pr.coef = o.coef;
+      }
+    }
+  }
+  // the last pass's sums (or, when no pass ran, the balancing ones, which nobody reads)
+  const double s_p2 = __shfl_sync(0xffffffffu, v, 0), s_u2 = __shfl_sync(0xffffffffu, v, 6),
+               s_du2 = __shfl_sync(0xffffffffu, v, 7);
+  double gap = 0.0;
+  if (ok && status == ST_OK) {  // the finalize pass's sums
+    bar_all<2, NW>();
+    const double mine = chip_block_total(sh);
+    ++step;
+    set = (set + 1) % kChipSets;
+    ok = chip_exchange<NW>(c, st, acc, set, cta, J.group, step, lane < 16, mine, gap);
+    if (!ok) bar_all_arrive<3, NW>();
+  }
+  if (!ok && lane == 0) atomicExch(c.error, 1);
+  double g4[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q)
+    g4[q] = __shfl_sync(0xffffffffu, gap, q) + __shfl_sync(0xffffffffu, gap, 4 + q);
+  if (ok && cta == 0 && lane == 0) {
+    st->k = pr.k;
+    st->trials = trials;
+    st->status = status;
+    st->alpha = pr.alpha;
+    st->theta = pr.theta;
+    st->coef = pr.coef;
+    st->fmean = fmean;
+    st->fnorm = pr.fnorm;
+    st->mass_mu = S.area * 0.5 * (m4[2] + m4[3]);
+    st->mass_nu = S.area * 0.5 * (m4[2] - m4[3]);
+    st->imbalance = S.area * m4[3];
+    st->r_feas = r_feas;
+    st->r_step = r_step;
+    st->s_p2 = s_p2;
+    st->s_u2 = s_u2;
+    st->s_du2 = s_du2;
+    for (int q = 0; q < 4; ++q) st->gap_sums[q] = g4[q];
+    st->done = 1;
+    atomicAdd(c.n_done, 1);
+  }
+}
+
+// A worker warp with the arithmetic of the tile pass.
+template <bool ISO>
+__device__ __forceinline__ void chip_worker(const ChipCta &X) {
+  const Ctl &c = X.c;
+  const ChipJob &J = X.J;
+  const Shot &S = X.S;
+  ChipShared &sh = X.sh;
+  const int lane = X.lane, warp = X.warp, nr = X.nr, nt = X.nt, ntp = X.ntp, n = X.n, ra = X.ra, rb = X.rb;
+  const int gj0 = X.gj0;
+  const float rdx = S.rdx, rdt = S.rdt;
   // shared memory, this lane's column of every row: planes div u, q, f; then the boundary rows
-  const unsigned plane = ((smem_u32(dyn4) + 127u) & ~127u) + 16u * lane;
+  const unsigned plane = X.smem;
   const unsigned bound = plane + 3 * kChipPlane;  // + 0: phi^k of a run's last row
   constexpr unsigned kBUx = kChipBound;           // u^{k+1} (x) of a run's first row
   constexpr unsigned kBP = 2 * kChipBound, kBQ = 3 * kChipBound;  // p, q of a run's last row
-
   // exchange buffers
-  float *xrow = S.f;
-  float2 *xcol = reinterpret_cast<float2 *>(S.f + chip_row_floats(J.segs, ntp));
+  float *const xrow = S.f;
+  float2 *const xcol = reinterpret_cast<float2 *>(S.f + chip_row_floats(J.segs, ntp));
+  const ChipLane ln = chip_lane(X);
+  const bool own_lane = ln.own;
+  const Q4 rdt_m = q4(ln.rm[0], ln.rm[1], ln.rm[2], ln.rm[3]);
+  auto row_addr = [&](int r) { return plane + static_cast<unsigned>(r) * kChipRowBytes; };
+  const unsigned brow = bound + static_cast<unsigned>(warp) * kChipRowBytes;  // this run's boundary row
 
-  if (warp == 0) tmem_alloc_all(&sh.tmem);
-  if (threadIdx.x == 0) {
-    sh.done = 0;
-    sh.status = ST_OK;
-    sh.bad = 0;
-  }
-  if (threadIdx.x < kChipVals) sh.part[15][threadIdx.x] = 0.0f;
-  if (threadIdx.x < 4) sh.dpart[15][threadIdx.x] = 0.0;
-  asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-  __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-
-  // a worker's run: rows [ra, rb), the leftover rows to the first warps, empty runs at the end
-  const int base = n / kChipWorkers, rem = n % kChipWorkers;
-  const int ra = warp * base + min(warp, rem), rb = ra + base + (warp < rem ? 1 : 0);
-  const uint32_t taddr = sh.tmem + (static_cast<uint32_t>(warp & 3) << 21) + (warp >> 2) * kChipTmemCols;
-  const int gj0 = J.strip * kChipTJ - 4 + 4 * lane;  // time index of this lane's first sample
-
-  if (warp == kChipWorkers) {
-    // ================================================================ decider warp
-    // the balancing sums: f, f^2, |Pcal| + |Pobs|, Pcal - Pobs
-    bar_all<2>();
-    double v = 0.0;
-    if ((lane & 7) < 4) {
-      double p[4];
+  // ---- inputs, warm start and the balancing sums
+  {
+    BalanceSums sums;
+    for (int r = ra; r < rb; ++r) {
+      const int gi = J.i0 - 2 + r;
+      const bool rin = gi >= 0 && gi < nr, rown = r >= 2 && r < J.h + 2;
+      float f[4], ph[4], ux[4], ut[4], d[4];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) p[i] = sh.dpart[(lane >> 3) + 4 * i][lane & 7];
-      v = (p[0] + p[1]) + (p[2] + p[3]);
-    }
-    v = sum_groups(v);
-    unsigned step = 1;
-    int set = 0;
-    bool ok = chip_exchange(c, st, acc, set, cta, J.group, step, lane < 8, v, v);
-    if (!ok) bar_all_arrive<3>();
-    DecidePrep pr;
-    pr.k = 0;
-    double m4[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) m4[q] = __shfl_sync(0xffffffffu, v, q);
-    const double N = static_cast<double>(nr) * nt;
-    const double fmean = c.balance ? m4[0] / N : 0.0;
-    pr.fnorm = sqrt(fmax(m4[1] - 2.0 * fmean * m4[0] + N * fmean * fmean, 0.0));
-    pr.alpha = c.alpha0 > 0.0 ? c.alpha0 : (c.linesearch ? 1.0 / sqrt(c.delta * S.lambda) : 1.0 / sqrt(S.lambda));
-    pr.beta_fixed = 1.0 / (S.lambda * pr.alpha);
-    pr.theta = 1.0;
-    pr.coef = 0.0;  // pass 0: phi^0 is the initial potential
-    // the values of the next pass, each written four times (lane 4 q + i: copy i of value q)
-    auto publish_sc = [&](float alpha, float coef, float theta, float inv) {
-      const int q = lane >> 2;
-      if (lane < 16) sh.sc[q][lane & 3] = q == 0 ? alpha : q == 1 ? coef : q == 2 ? theta : inv;
-    };
-    publish_sc(static_cast<float>(pr.alpha), 0.0f, 1.0f, 1.0f / (1.0f + static_cast<float>(c.eps * pr.alpha)));
-    if (lane >= 16 && lane < 24) sh.sc[lane >> 2][lane & 3] = lane < 20 ? rdx : rdt;
-    if (lane == 0) {
-      sh.fmean = static_cast<float>(fmean);
-      if (!ok) sh.bad = 1;
-    }
-    bar_all<4>();
-    int trials = 0;
-    double r_feas = -1.0, r_step = -1.0;
-    bool done = false;
-    int status = ST_OK;
-    const bool quick = c.linesearch && c.debug_fault != 1;
-    while (ok && !done) {
-      decide_prep_lanes(c, pr);  // overlaps the pass
-      const QuickPrep qp = quick_prep(pr);
-      bar_all<2>();
-      const double mine = chip_block_total(sh);
-      ++step;
-      set = (set + 1) % kChipSets;
-      ok = chip_exchange(c, st, acc, set, cta, J.group, step, lane < 16, mine, v);
-      if (!ok) {
-        bar_all_arrive<3>();
-        if (lane == 0) sh.bad = 1;
-        bar_all<4>();
-        break;
-      }
-      const int w = quick && !pr.check ? quick_decide(c, qp, v) : -1;
-      if (w >= 0) {
-        constexpr unsigned FULL = 0xffffffffu;
-        publish_sc(__shfl_sync(FULL, pr.alpha_lf, w), __shfl_sync(FULL, pr.coef_lf, w),
-                   __shfl_sync(FULL, pr.theta_lf, w), __shfl_sync(FULL, pr.inv_lf, w));
-        done = pr.k + 1 >= c.max_iter;
-        if (lane == 0) sh.done = done;
-        bar_all<4>();
-        trials += w + 1;
-        if (c.trace && cta == 0) {
-          Decision o;
-          o.alpha = __shfl_sync(FULL, pr.alpha_l, w);
-          o.theta = __shfl_sync(FULL, pr.s_lane, w);
-          o.trials_now = w + 1;
-          const double ppp = __shfl_sync(FULL, v, 0);
-          if (lane == 0) write_trace(c, J.gather, pr.k, o, ppp, pr.fnorm);
+      for (int q = 0; q < 4; ++q) {
+        const int gj = gj0 + q;
+        const bool in = rin && ln.use[q];
+        const size_t g = static_cast<size_t>(gi) * nt + gj;
+        const float po = in ? S.p_obs[g] : 0.0f, pp = in ? S.p_pred[g] : 0.0f;
+        f[q] = pp - po;
+        ph[q] = in && S.phi_init ? S.phi_init[g] : 0.0f;
+        ux[q] = ut[q] = d[q] = 0.0f;
+        if (in && S.m_init) {
+          ux[q] = chip_init_flux(X, 0, gi, gj);
+          ut[q] = chip_init_flux(X, 1, gi, gj);
+          d[q] = fmaf(chip_init_flux(X, 0, gi + 1, gj) - ux[q], rdx, (chip_init_flux(X, 1, gi, gj + 1) - ut[q]) * rdt);
         }
-        pr.alpha = __shfl_sync(FULL, pr.alpha_l, w);
-        pr.theta = __shfl_sync(FULL, pr.s_lane, w);
-        pr.coef = __shfl_sync(FULL, pr.coef_l, w);
-        ++pr.k;
-      } else {
-        double a_[9];
-#pragma unroll
-        for (int q = 0; q < 6; ++q) a_[q] = __shfl_sync(0xffffffffu, v, q);
-        a_[6] = 0.0;
-        a_[7] = __shfl_sync(0xffffffffu, v, 6);
-        a_[8] = __shfl_sync(0xffffffffu, v, 7);
-        const Decision o = decide_core(c, pr, a_);
-        trials += o.trials_now;
-        done = o.done;
-        status = o.status;
-        if (o.status == ST_OK) publish_sc(o.alpha_f, o.coef_f, o.theta_f, o.inv_f);
-        if (lane == 0) {
-          sh.status = o.status;
-          sh.done = o.done;
-        }
-        bar_all<4>();
-        if (cta == 0 && lane == 0) write_trace(c, J.gather, pr.k, o, a_[0], pr.fnorm);
-        if (o.checked && cta == 0) residuals(pr, a_, r_feas, r_step);
-        if (o.status == ST_OK) {
-          pr.k = o.k_new;
-          pr.alpha = o.alpha;
-          pr.theta = o.theta;
-          pr.coef = o.coef;
-        }
+        if (in && rown && own_lane) sums.add(po, pp);
       }
-    }
-    // the last pass's sums (or, when no pass ran, the balancing ones, which nobody reads)
-    const double s_p2 = __shfl_sync(0xffffffffu, v, 0), s_u2 = __shfl_sync(0xffffffffu, v, 6),
-                 s_du2 = __shfl_sync(0xffffffffu, v, 7);
-    double gap = 0.0;
-    if (ok && status == ST_OK) {  // the finalize pass's sums
-      bar_all<2>();
-      const double mine = chip_block_total(sh);
-      ++step;
-      set = (set + 1) % kChipSets;
-      ok = chip_exchange(c, st, acc, set, cta, J.group, step, lane < 16, mine, gap);
-      if (!ok) bar_all_arrive<3>();
-    }
-    if (!ok && lane == 0) atomicExch(c.error, 1);
-    double g4[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q)
-      g4[q] = __shfl_sync(0xffffffffu, gap, q) + __shfl_sync(0xffffffffu, gap, 4 + q);
-    if (ok && cta == 0 && lane == 0) {
-      st->k = pr.k;
-      st->trials = trials;
-      st->status = status;
-      st->alpha = pr.alpha;
-      st->theta = pr.theta;
-      st->coef = pr.coef;
-      st->fmean = fmean;
-      st->fnorm = pr.fnorm;
-      st->mass_mu = S.area * 0.5 * (m4[2] + m4[3]);
-      st->mass_nu = S.area * 0.5 * (m4[2] - m4[3]);
-      st->imbalance = S.area * m4[3];
-      st->r_feas = r_feas;
-      st->r_step = r_step;
-      st->s_p2 = s_p2;
-      st->s_u2 = s_u2;
-      st->s_du2 = s_du2;
-      for (int q = 0; q < 4; ++q) st->gap_sums[q] = g4[q];
-      st->done = 1;
-      atomicAdd(c.n_done, 1);
-    }
-  } else {
-    // ================================================================ worker warps
-    bool use[4];  // samples whose f this CTA needs (one halo sample more on the left than right)
-    float rm[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int gj = gj0 + q;
-      use[q] = gj >= 0 && gj < nt && (lane > 0 || q >= 2) && (lane < 31 || q == 0);
-      // 1/dt of the face left of the sample, 0 for outer faces and samples nobody needs
-      rm[q] = gj > 0 && gj < nt && (lane > 0 || q == 3) && (lane < 31 || q == 0) ? rdt : 0.0f;
-    }
-    const Q4 rdt_m = q4(rm[0], rm[1], rm[2], rm[3]);
-    const bool own_lane = lane >= 1 && lane <= 30;
-    auto row_addr = [&](int r) { return plane + static_cast<unsigned>(r) * kChipRowBytes; };
-    const unsigned brow = bound + static_cast<unsigned>(warp) * kChipRowBytes;  // this run's boundary row
-
-    // ---- inputs, warm start and the balancing sums
-    {
-      Sum2 s_f, s_f2, s_ab;
-      float s_de = 0.0f;  // rounding errors of the differences f = Pcal - Pobs
-      auto flux = [&](int plane, int gi, int gj) -> float {
-        const bool in = gi >= 0 && gi < nr && gj >= 0 && gj < nt && (plane ? gj > 0 : gi > 0);
-        return in ? S.m_init[(static_cast<size_t>(plane) * nr + gi) * nt + gj] : 0.0f;
-      };
-      for (int r = ra; r < rb; ++r) {
-        const int gi = J.i0 - 2 + r;
-        const bool rin = gi >= 0 && gi < nr, rown = r >= 2 && r < J.h + 2;
-        float f[4], ph[4], ux[4], ut[4], d[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const int gj = gj0 + q;
-          const bool in = rin && use[q];
-          const size_t g = static_cast<size_t>(gi) * nt + gj;
-          const float po = in ? S.p_obs[g] : 0.0f, pp = in ? S.p_pred[g] : 0.0f;
-          f[q] = pp - po;
-          ph[q] = in && S.phi_init ? S.phi_init[g] : 0.0f;
-          ux[q] = ut[q] = d[q] = 0.0f;
-          if (in && S.m_init) {
-            ux[q] = flux(0, gi, gj);
-            ut[q] = flux(1, gi, gj);
-            d[q] = fmaf(flux(0, gi + 1, gj) - ux[q], rdx, (flux(1, gi, gj + 1) - ut[q]) * rdt);
-          }
-          if (in && rown && own_lane) {
-            float e, df;
-            two_sum(pp, -po, df, e);
-            s_de += e;
-            s_f.add(f[q]);
-            const float f2 = f[q] * f[q];
-            s_f2.add(f2);
-            s_f2.lo += fmaf(f[q], f[q], -f2);
-            two_sum(fabsf(pp), fabsf(po), df, e);
-            s_ab.add(df);
-            s_ab.lo += e;
-          }
-        }
-        const unsigned a = row_addr(r);
-        sts4(a, q4(d[0], d[1], d[2], d[3]));
-        sts4<kChipPlane>(a, q4s(0.0f));
-        sts4<2 * kChipPlane>(a, q4(f[0], f[1], f[2], f[3]));
-        tmem_store_row(taddr + (r - ra) * kChipRowCols,
-                       {q4(ux[0], ux[1], ux[2], ux[3]), q4(ut[0], ut[1], ut[2], ut[3]),
-                        q4(ph[0], ph[1], ph[2], ph[3])});
-      }
-      tmem_stores_done();
-      const double t0 = warp_sum_d(s_f.value()), t1 = warp_sum_d(s_f2.value());
-      const double t2 = warp_sum_d(s_ab.value());
-      const double t3 = warp_sum_d(s_f.value() + static_cast<double>(s_de));
-      if (lane < 4) sh.dpart[warp][lane] = lane == 0 ? t0 : lane == 1 ? t1 : lane == 2 ? t2 : t3;
-      bar_all<2>();
-      bar_all<3>();
-      bar_all<4>();
-      const float fm = sh.fmean;
-      for (int r = ra; r < rb; ++r) {  // the balanced f, zero outside the gather
-        const int gi = J.i0 - 2 + r;
-        const bool rin = gi >= 0 && gi < nr;
-        float x[4];
-        un4(lds4<2 * kChipPlane>(row_addr(r)), x);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) x[q] = rin && use[q] ? x[q] - fm : 0.0f;
-        sts4<2 * kChipPlane>(row_addr(r), q4(x[0], x[1], x[2], x[3]));
-      }
-    }
-
-    // row r with phi^k completed from the last pass's div u and q (received ones at the halo)
-    auto dual = [&](int r, const Q4 &cf, const Q4 &th) -> RowState {
-      RowState s = tmem_load_row(taddr + (r - ra) * kChipRowCols);
       const unsigned a = row_addr(r);
-      const Q4 p = add4(lds4(a), lds4<2 * kChipPlane>(a));
-      s.ph = fma4(cf, fma4(th, lds4<kChipPlane>(a), p), s.ph);
-      return s;
-    };
-    // div u and q of the strip's first and last-but-one sample go to the neighbouring strips
-    const bool edge_lane = lane == 1 || lane == 30;
-    float2 *const xedge = xcol + (static_cast<size_t>(J.strip) * 2 + (lane == 30 ? 1 : 0)) * nr + J.i0 - 2;
-    const size_t xcol_set = static_cast<size_t>(J.strips) * 2 * nr;  // pairs of one parity
-    // the halo sample that this lane fetches: even lanes sample -2, odd ones sample 120 of the
-    // run's row lane / 2 (rows 0 and n - 1 come whole)
-    const float2 *halo_src = nullptr;
-    unsigned halo_dst = 0;
-    {
-      const int r = ra + (lane >> 1), side = lane & 1, gi = J.i0 - 2 + r, strip = J.strip + (side ? 1 : -1);
-      if (r < rb && r > 0 && r < n - 1 && gi >= 0 && gi < nr && strip >= 0 && strip < J.strips) {
-        halo_src = xcol + (static_cast<size_t>(strip) * 2 + (side ? 0 : 1)) * nr + gi;
-        halo_dst = row_addr(r) - 16u * lane + (side ? 4 * 124 : 4 * 2);
-      }
+      sts4(a, q4(d[0], d[1], d[2], d[3]));
+      sts4<kChipPlane>(a, q4s(0.0f));
+      sts4<2 * kChipPlane>(a, q4(f[0], f[1], f[2], f[3]));
+      tmem_store_row(X.taddr + (r - ra) * kChipRowCols,
+                     {q4(ux[0], ux[1], ux[2], ux[3]), q4(ut[0], ut[1], ut[2], ut[3]),
+                      q4(ph[0], ph[1], ph[2], ph[3])});
     }
-    const unsigned sc_addr = smem_u32(&sh.sc[0][0]);
-
-    int k = 0;
-    while (!sh.bad) {
-      if (sh.done) break;
-      const float alpha = sh.sc[0][0];
-      const Q4 al4 = lds4(sc_addr), cf = lds4<16>(sc_addr), th = lds4<32>(sc_addr), inv4 = lds4<48>(sc_addr);
-      const Q4 rdx4 = lds4<64>(sc_addr), rdt4 = lds4<80>(sc_addr);
-      const bool need_res = (c.tol > 0.0 && (k + 1) % c.check_every == 0) || k + 1 >= c.max_iter;
-      f32x2 v[8];
+    tmem_stores_done();
+    sums.store(X);
+    bar_all<2>();
+    bar_all<3>();
+    bar_all<4>();
+    const float fm = sh.fmean;
+    for (int r = ra; r < rb; ++r) {  // the balanced f, zero outside the gather
+      const int gi = J.i0 - 2 + r;
+      const bool rin = gi >= 0 && gi < nr;
+      float x[4];
+      un4(lds4<2 * kChipPlane>(row_addr(r)), x);
 #pragma unroll
-      for (int q = 0; q < 8; ++q) v[q] = 0ull;
+      for (int q = 0; q < 4; ++q) x[q] = rin && ln.use[q] ? x[q] - fm : 0.0f;
+      sts4<2 * kChipPlane>(row_addr(r), q4(x[0], x[1], x[2], x[3]));
+    }
+  }
 
-      // u^{k+1} of a row from phi^k of it and of the row above
-      // (PLAIN: an owned row away from the gather's first receiver, no residual sums)
-      auto prox_row = [&](auto plain, int r, const RowState &s, const Q4 &ph_up, Q4 &nx, Q4 &nv) {
-        constexpr bool PLAIN = decltype(plain)::value;
-        const int gi = J.i0 - 2 + r;
-        const Q4 rx = PLAIN || (gi > 0 && gi < nr) ? rdx4 : q4s(0.0f);
-        const Q4 gx = mul4(sub4(s.ph, ph_up), rx), gt = mul4(diff_left(s.ph), rdt_m);
-        chip_prox<ISO>(s.ux, s.ut, gx, gt, alpha, al4, inv4, nx, nv);
-        if (!PLAIN && need_res && r >= 2 && r < J.h + 2) {
-          const Q4 dx_ = sub4(nx, s.ux), dt_ = sub4(nv, s.ut);
-          v[6] = fma2(nx.a, nx.a, fma2(nv.a, nv.a, v[6]));
-          v[6] = fma2(nx.b, nx.b, fma2(nv.b, nv.b, v[6]));
-          v[7] = fma2(dx_.a, dx_.a, fma2(dt_.a, dt_.a, v[7]));
-          v[7] = fma2(dx_.b, dx_.b, fma2(dt_.b, dt_.b, v[7]));
-        }
-      };
-      float *const xr = xrow + static_cast<size_t>(k & 1) * J.segs * 4 * ntp;
-      float2 *const xe = xedge + (k & 1 ? xcol_set : 0);
-      // p, q of a row, its sums that need no other row, and the halo cells others hold
-      // (PLAIN: an owned row that no other segment holds as halo)
-      auto flux_row = [&](auto plain, int r, const Q4 &ux, const Q4 &ut, const Q4 &ux_dn, Q4 &p, Q4 &q) {
-        constexpr bool PLAIN = decltype(plain)::value;
-        const unsigned a = row_addr(r);
-        const Q4 dn = div4(sub4(ux_dn, ux), diff_right(ut), rdx4, rdt4);
-        p = add4(dn, lds4<2 * kChipPlane>(a));
-        q = sub4(dn, lds4(a));
-        sts4(a, dn);
-        sts4<kChipPlane>(a, q);
-        if (PLAIN || (r >= 2 && r < J.h + 2)) {
-          const Q4 gp = mul4(diff_left(p), rdt_m), gq = mul4(diff_left(q), rdt_m);
-          v[0] = fma2(p.b, p.b, fma2(p.a, p.a, v[0]));
-          v[1] = fma2(p.b, q.b, fma2(p.a, q.a, v[1]));
-          v[2] = fma2(q.b, q.b, fma2(q.a, q.a, v[2]));
-          v[3] = fma2(gp.b, gp.b, fma2(gp.a, gp.a, v[3]));
-          v[4] = fma2(gp.b, gq.b, fma2(gp.a, gq.a, v[4]));
-          v[5] = fma2(gq.b, gq.b, fma2(gq.a, gq.a, v[5]));
-          const f32x2 de = lane == 30 ? dn.b : dn.a, qe = lane == 30 ? q.b : q.a;
-          float d0, q0, unused;
-          upk(de, d0, unused);
-          upk(qe, q0, unused);
-          if (edge_lane) __stcg(xe + r, make_float2(d0, q0));
-          if (!PLAIN && (r == 2 || r == J.h)) {  // rows that the neighbouring segments hold as halo
-            float d_[4], q_[4];
-            un4(dn, d_);
-            un4(q, q_);
-            if (own_lane && gj0 < ntp) {
+  // row r with phi^k completed from the last pass's div u and q (received ones at the halo)
+  auto dual = [&](int r, const Q4 &cf, const Q4 &th) -> RowState {
+    RowState s = tmem_load_row(X.taddr + (r - ra) * kChipRowCols);
+    const unsigned a = row_addr(r);
+    const Q4 p = add4(lds4(a), lds4<2 * kChipPlane>(a));
+    s.ph = fma4(cf, fma4(th, lds4<kChipPlane>(a), p), s.ph);
+    return s;
+  };
+  // div u and q of the strip's first and last-but-one sample go to the neighbouring strips
+  const bool edge_lane = lane == 1 || lane == 30;
+  float2 *const xedge = xcol + (static_cast<size_t>(J.strip) * 2 + (lane == 30 ? 1 : 0)) * nr + J.i0 - 2;
+  const size_t xcol_set = static_cast<size_t>(J.strips) * 2 * nr;  // pairs of one parity
+  // the halo sample that this lane fetches: even lanes sample -2, odd ones sample 120 of the
+  // run's row lane / 2 (rows 0 and n - 1 come whole)
+  const float2 *halo_src = nullptr;
+  unsigned halo_dst = 0;
+  {
+    const int r = ra + (lane >> 1), side = lane & 1, gi = J.i0 - 2 + r, strip = J.strip + (side ? 1 : -1);
+    if (r < rb && r > 0 && r < n - 1 && gi >= 0 && gi < nr && strip >= 0 && strip < J.strips) {
+      halo_src = xcol + (static_cast<size_t>(strip) * 2 + (side ? 0 : 1)) * nr + gi;
+      halo_dst = row_addr(r) - 16u * lane + (side ? 4 * 124 : 4 * 2);
+    }
+  }
+  const unsigned sc_addr = smem_u32(&sh.sc[0][0]);
+
+  int k = 0;
+  while (!sh.bad) {
+    if (sh.done) break;
+    const float alpha = sh.sc[0][0];
+    const Q4 al4 = lds_pair(sc_addr), cf = lds_pair<16>(sc_addr), th = lds_pair<32>(sc_addr);
+    const Q4 inv4 = lds_pair<48>(sc_addr), rdx4 = lds_pair<64>(sc_addr), rdt4 = lds_pair<80>(sc_addr);
+    const bool need_res = (c.tol > 0.0 && (k + 1) % c.check_every == 0) || k + 1 >= c.max_iter;
+    f32x2 v[8];
 #pragma unroll
-              for (int w = 0; w < 2; ++w) {
-                if (r != (w ? J.h : 2)) continue;
-                float *o = xr + (static_cast<size_t>(J.seg) * 2 + w) * 2 * ntp + gj0;
-                __stcg(reinterpret_cast<float4 *>(o), make_float4(d_[0], d_[1], d_[2], d_[3]));
-                __stcg(reinterpret_cast<float4 *>(o + ntp), make_float4(q_[0], q_[1], q_[2], q_[3]));
-              }
-            }
-          }
-        }
-      };
-      // receiver-direction gradient sums of row r from p, q of it and of the row above
-      auto grad_row = [&](auto plain, int r, const Q4 &p, const Q4 &q, const Q4 &pu, const Q4 &qu) {
-        if (!decltype(plain)::value && !(r >= 2 && r < J.h + 2 && J.i0 - 2 + r > 0)) return;
-        const Q4 gp = mul4(sub4(p, pu), rdx4), gq = mul4(sub4(q, qu), rdx4);
+    for (int q = 0; q < 8; ++q) v[q] = 0ull;
+
+    // u^{k+1} of a row from phi^k of it and of the row above
+    // (PLAIN: an owned row away from the gather's first receiver, no residual sums)
+    auto prox_row = [&](auto plain, int r, const RowState &s, const Q4 &ph_up, Q4 &nx, Q4 &nv) {
+      constexpr bool PLAIN = decltype(plain)::value;
+      const int gi = J.i0 - 2 + r;
+      const Q4 rx = PLAIN || (gi > 0 && gi < nr) ? rdx4 : q4s(0.0f);
+      const Q4 gx = mul4(sub4(s.ph, ph_up), rx), gt = mul4(diff_left(s.ph), rdt_m);
+      chip_prox<ISO>(s.ux, s.ut, gx, gt, alpha, al4, inv4, nx, nv);
+      if (!PLAIN && need_res && r >= 2 && r < J.h + 2) {
+        const Q4 dx_ = sub4(nx, s.ux), dt_ = sub4(nv, s.ut);
+        v[6] = fma2(nx.a, nx.a, fma2(nv.a, nv.a, v[6]));
+        v[6] = fma2(nx.b, nx.b, fma2(nv.b, nv.b, v[6]));
+        v[7] = fma2(dx_.a, dx_.a, fma2(dt_.a, dt_.a, v[7]));
+        v[7] = fma2(dx_.b, dx_.b, fma2(dt_.b, dt_.b, v[7]));
+      }
+    };
+    float *const xr = xrow + static_cast<size_t>(k & 1) * J.segs * 4 * ntp;
+    float2 *const xe = xedge + (k & 1 ? xcol_set : 0);
+    // p, q of a row, its sums that need no other row, and the halo cells others hold
+    // (PLAIN: an owned row that no other segment holds as halo)
+    auto flux_row = [&](auto plain, int r, const Q4 &ux, const Q4 &ut, const Q4 &ux_dn, Q4 &p, Q4 &q) {
+      constexpr bool PLAIN = decltype(plain)::value;
+      const unsigned a = row_addr(r);
+      const Q4 dn = div4(sub4(ux_dn, ux), diff_right(ut), rdx4, rdt4);
+      p = add4(dn, lds4<2 * kChipPlane>(a));
+      q = sub4(dn, lds4(a));
+      sts4(a, dn);
+      sts4<kChipPlane>(a, q);
+      if (PLAIN || (r >= 2 && r < J.h + 2)) {
+        const Q4 gp = mul4(diff_left(p), rdt_m), gq = mul4(diff_left(q), rdt_m);
+        v[0] = fma2(p.b, p.b, fma2(p.a, p.a, v[0]));
+        v[1] = fma2(p.b, q.b, fma2(p.a, q.a, v[1]));
+        v[2] = fma2(q.b, q.b, fma2(q.a, q.a, v[2]));
         v[3] = fma2(gp.b, gp.b, fma2(gp.a, gp.a, v[3]));
         v[4] = fma2(gp.b, gq.b, fma2(gp.a, gq.a, v[4]));
         v[5] = fma2(gq.b, gq.b, fma2(gq.a, gq.a, v[5]));
-      };
-
-      // ---- the run, upwards: row r's phi^k, then row r + 1's flux and sums.  The rows go two
-      // per trip, so what one row hands to the next changes registers instead of being copied.
-      struct Carry {
-        RowState cur;          // the row below with phi^k completed (u still u^k)
-        Q4 ux_dn, p_dn, q_dn;  // of the row below that: u^{k+1} (x), p, q
-      };
-      auto step = [&](auto plain, int r, const Carry &in, Carry &out) {
-        out.cur = dual(r, cf, th);
-        Q4 nx, nv;
-        prox_row(plain, r + 1, in.cur, out.cur.ph, nx, nv);
-        tmem_store_row(taddr + (r + 1 - ra) * kChipRowCols, {nx, nv, in.cur.ph});
-        out.ux_dn = nx;
-        flux_row(plain, r + 1, nx, nv, in.ux_dn, out.p_dn, out.q_dn);
-        if (r + 2 < rb - 1) grad_row(plain, r + 2, in.p_dn, in.q_dn, out.p_dn, out.q_dn);
-      };
-      const BoolConst<true> plain{};
-      const BoolConst<false> any{};
-      Carry x, y;
-      x.p_dn = x.q_dn = x.ux_dn = q4s(0.0f);
-      if (ra < rb) {
-        const RowState s = dual(rb - 1, cf, th);
-        sts4(brow, s.ph);
-        x.cur = s;
-        if (ra < rb - 1) {  // the last row's flux waits for the next run's first row
-          x.cur = dual(rb - 2, cf, th);
-          Q4 nx, nv;
-          prox_row(any, rb - 1, s, x.cur.ph, nx, nv);
-          tmem_store_row(taddr + (rb - 1 - ra) * kChipRowCols, {nx, nv, s.ph});
-          x.ux_dn = nx;
-        }
-        int r = rb - 3;
-#pragma unroll 1
-        while (r >= ra) {
-          if (!need_res && r + 1 < J.h && r >= 3 && r > ra) {  // rows r + 1 and r are plain
-            step(plain, r, x, y);
-            step(plain, r - 1, y, x);
-            r -= 2;
-          } else {
-            step(any, r, x, y);
-            x = y;
-            --r;
-          }
-        }
-      }
-      // ---- the first row of the run: phi^k of the row above comes from the run before
-      bar_workers();
-      Q4 p_a = q4s(0.0f), q_a = q4s(0.0f);  // p, q of row ra
-      if (ra < rb) {
-        if (ra > 0) {
-          Q4 nx, nv;
-          prox_row(any, ra, x.cur, lds4(brow - kChipRowBytes), nx, nv);
-          sts4<kBUx>(brow, nx);
-          tmem_store_row(taddr, {nx, nv, x.cur.ph});
-          if (ra < rb - 1) {
-            flux_row(any, ra, nx, nv, x.ux_dn, p_a, q_a);
-            if (ra + 1 < rb - 1) grad_row(any, ra + 1, x.p_dn, x.q_dn, p_a, q_a);
-          }
-        } else {
-          tmem_store_row(taddr, x.cur);  // row 0 carries phi^k only
-        }
-      }
-      tmem_stores_done();
-      bar_workers();
-      // ---- the last row of the run: u^{k+1} of the row below comes from the next run
-      const int L = rb - 1;
-      if (ra < rb && L >= 1 && L < n - 1) {
-        const RowState s = tmem_load_row(taddr + (L - ra) * kChipRowCols);
-        Q4 p, q;
-        flux_row(any, L, s.ux, s.ut, lds4<kBUx + kChipRowBytes>(brow), p, q);
-        sts4<kBP>(brow, p);
-        sts4<kBQ>(brow, q);
-        if (L == ra) {
-          p_a = p;
-          q_a = q;
-        } else if (L - 1 >= 1) {  // the row above in this run: p = div u + f, q as stored
-          const unsigned a = row_addr(L - 1);
-          grad_row(any, L, p, q, add4(lds4(a), lds4<2 * kChipPlane>(a)), lds4<kChipPlane>(a));
-        }
-      }
-      bar_workers();
-      if (ra < rb && ra >= 2 && ra < n - 1)
-        grad_row(any, ra, p_a, q_a, lds4<kBP - kChipRowBytes>(brow), lds4<kBQ - kChipRowBytes>(brow));
-
-      // ---- totals of the warp (the two lanes that only feed neighbours leave theirs out)
-      float t[8];
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        float x, y;
-        upk(v[q], x, y);
-        t[q] = own_lane ? x + y : 0.0f;
-      }
-      const float tot = warp_sum8(t);
-      if (lane < 8) sh.part[warp][lane] = tot;
-      bar_all_arrive<2>();
-      bar_all<3>();  // every CTA of the group has finished the pass
-      // ---- halo values of the pass: received div u and q
-      if (!sh.bad) {
-        if (halo_src) {
-          const float2 e = __ldcg(halo_src + (k & 1 ? xcol_set : 0));
-          sts1(halo_dst, e.x);
-          sts1(halo_dst + kChipPlane, e.y);
-        }
-        for (int w = 0; w < 2; ++w) {
-          const int r = w ? n - 1 : 0, gi = J.i0 - 2 + r, seg = J.seg + (w ? 1 : -1);
-          if (r < ra || r >= rb || seg < 0 || seg >= J.segs || gi < 0 || gi >= nr) continue;
-          const float *o = xr + (static_cast<size_t>(seg) * 2 + (w ? 0 : 1)) * 2 * ntp;
+        const f32x2 de = lane == 30 ? dn.b : dn.a, qe = lane == 30 ? q.b : q.a;
+        float d0, q0, unused;
+        upk(de, d0, unused);
+        upk(qe, q0, unused);
+        if (edge_lane) __stcg(xe + r, make_float2(d0, q0));
+        if (!PLAIN && (r == 2 || r == J.h)) {  // rows that the neighbouring segments hold as halo
           float d_[4], q_[4];
+          un4(dn, d_);
+          un4(q, q_);
+          if (own_lane && gj0 < ntp) {
 #pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            const bool in = use[q];
-            d_[q] = in ? __ldcg(o + gj0 + q) : 0.0f;
-            q_[q] = in ? __ldcg(o + ntp + gj0 + q) : 0.0f;
-          }
-          sts4(row_addr(r), q4(d_[0], d_[1], d_[2], d_[3]));
-          sts4<kChipPlane>(row_addr(r), q4(q_[0], q_[1], q_[2], q_[3]));
-        }
-      }
-      bar_all<4>();  // the decision
-      ++k;
-    }
-
-    // ---- finalize: phi^K, the outputs and the duality gap's sums
-    if (!sh.bad && sh.status == ST_OK) {
-      const Q4 cf = lds4<16>(sc_addr), th = lds4<32>(sc_addr);
-      Sum2 t[4];
-      for (int r = ra; r < rb; ++r) {
-        const RowState s = dual(r, cf, th);
-        tmem_store_row(taddr + (r - ra) * kChipRowCols, s);
-        if (r == rb - 1) sts4(brow, s.ph);
-      }
-      tmem_stores_done();
-      bar_workers();
-      const bool vec = (nt & 3) == 0 && ((reinterpret_cast<uintptr_t>(S.phi_out) | reinterpret_cast<uintptr_t>(S.m_out)) & 15u) == 0;
-      Q4 up = ra < rb && ra > 0 ? lds4(brow - kChipRowBytes) : q4s(0.0f);
-      for (int r = ra; r < rb; ++r) {
-        const int gi = J.i0 - 2 + r;
-        const RowState s = tmem_load_row(taddr + (r - ra) * kChipRowCols);
-        const Q4 gtv = diff_left(s.ph);
-        if (r >= 2 && r < J.h + 2 && own_lane) {
-          float ph[4], pu[4], gt[4], ux[4], ut[4], fb[4];
-          un4(s.ph, ph);
-          un4(up, pu);
-          un4(gtv, gt);
-          un4(s.ux, ux);
-          un4(s.ut, ut);
-          un4(lds4<2 * kChipPlane>(row_addr(r)), fb);
-          const size_t g = static_cast<size_t>(gi) * nt + gj0, m_t = static_cast<size_t>(nr) * nt;
-          if (vec && gj0 < nt) {
-            *reinterpret_cast<float4 *>(S.phi_out + g) = make_float4(ph[0], ph[1], ph[2], ph[3]);
-            *reinterpret_cast<float4 *>(S.m_out + g) = make_float4(ux[0], ux[1], ux[2], ux[3]);
-            *reinterpret_cast<float4 *>(S.m_out + m_t + g) = make_float4(ut[0], ut[1], ut[2], ut[3]);
-          }
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            const int gj = gj0 + q;
-            if (gj >= nt) continue;
-            if (!vec) {
-              S.phi_out[g + q] = ph[q];
-              S.m_out[g + q] = ux[q];
-              S.m_out[m_t + g + q] = ut[q];
+            for (int w = 0; w < 2; ++w) {
+              if (r != (w ? J.h : 2)) continue;
+              float *o = xr + (static_cast<size_t>(J.seg) * 2 + w) * 2 * ntp + gj0;
+              __stcg(reinterpret_cast<float4 *>(o), make_float4(d_[0], d_[1], d_[2], d_[3]));
+              __stcg(reinterpret_cast<float4 *>(o + ntp), make_float4(q_[0], q_[1], q_[2], q_[3]));
             }
-            const float gx = gi > 0 ? (ph[q] - pu[q]) * rdx : 0.0f, gtt = gj > 0 ? gt[q] * rdt : 0.0f;
-            gap_terms(t, ux[q], ut[q], ph[q], fb[q], gx, gtt, ISO);
           }
         }
-        up = s.ph;
       }
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        t[q].warp_total();
-        if (lane == 0) {
-          sh.part[warp][q] = t[q].hi;
-          sh.part[warp][4 + q] = t[q].lo;
+    };
+    // receiver-direction gradient sums of row r from p, q of it and of the row above
+    auto grad_row = [&](auto plain, int r, const Q4 &p, const Q4 &q, const Q4 &pu, const Q4 &qu) {
+      if (!decltype(plain)::value && !(r >= 2 && r < J.h + 2 && J.i0 - 2 + r > 0)) return;
+      const Q4 gp = mul4(sub4(p, pu), rdx4), gq = mul4(sub4(q, qu), rdx4);
+      v[3] = fma2(gp.b, gp.b, fma2(gp.a, gp.a, v[3]));
+      v[4] = fma2(gp.b, gq.b, fma2(gp.a, gq.a, v[4]));
+      v[5] = fma2(gq.b, gq.b, fma2(gq.a, gq.a, v[5]));
+    };
+
+    // ---- the run, upwards: row r's phi^k, then row r + 1's flux and sums.  The rows go two
+    // per trip, so what one row hands to the next changes registers instead of being copied.
+    struct Carry {
+      RowState cur;          // the row below with phi^k completed (u still u^k)
+      Q4 ux_dn, p_dn, q_dn;  // of the row below that: u^{k+1} (x), p, q
+    };
+    auto step = [&](auto plain, int r, const Carry &in, Carry &out) {
+      out.cur = dual(r, cf, th);
+      Q4 nx, nv;
+      prox_row(plain, r + 1, in.cur, out.cur.ph, nx, nv);
+      tmem_store_row(X.taddr + (r + 1 - ra) * kChipRowCols, {nx, nv, in.cur.ph});
+      out.ux_dn = nx;
+      flux_row(plain, r + 1, nx, nv, in.ux_dn, out.p_dn, out.q_dn);
+      if (r + 2 < rb - 1) grad_row(plain, r + 2, in.p_dn, in.q_dn, out.p_dn, out.q_dn);
+    };
+    const BoolConst<true> plain{};
+    const BoolConst<false> any{};
+    Carry x, y;
+    x.p_dn = x.q_dn = x.ux_dn = q4s(0.0f);
+    if (ra < rb) {
+      const RowState s = dual(rb - 1, cf, th);
+      sts4(brow, s.ph);
+      x.cur = s;
+      if (ra < rb - 1) {  // the last row's flux waits for the next run's first row
+        x.cur = dual(rb - 2, cf, th);
+        Q4 nx, nv;
+        prox_row(any, rb - 1, s, x.cur.ph, nx, nv);
+        tmem_store_row(X.taddr + (rb - 1 - ra) * kChipRowCols, {nx, nv, s.ph});
+        x.ux_dn = nx;
+      }
+      int r = rb - 3;
+#pragma unroll 1
+      while (r >= ra) {
+        if (!need_res && r + 1 < J.h && r >= 3 && r > ra) {  // rows r + 1 and r are plain
+          step(plain, r, x, y);
+          step(plain, r - 1, y, x);
+          r -= 2;
+        } else {
+          step(any, r, x, y);
+          x = y;
+          --r;
         }
       }
-      bar_all_arrive<2>();
-      bar_all<3>();
     }
+    // ---- the first row of the run: phi^k of the row above comes from the run before
+    bar_workers();
+    Q4 p_a = q4s(0.0f), q_a = q4s(0.0f);  // p, q of row ra
+    if (ra < rb) {
+      if (ra > 0) {
+        Q4 nx, nv;
+        prox_row(any, ra, x.cur, lds4(brow - kChipRowBytes), nx, nv);
+        sts4<kBUx>(brow, nx);
+        tmem_store_row(X.taddr, {nx, nv, x.cur.ph});
+        if (ra < rb - 1) {
+          flux_row(any, ra, nx, nv, x.ux_dn, p_a, q_a);
+          if (ra + 1 < rb - 1) grad_row(any, ra + 1, x.p_dn, x.q_dn, p_a, q_a);
+        }
+      } else {
+        tmem_store_row(X.taddr, x.cur);  // row 0 carries phi^k only
+      }
+    }
+    tmem_stores_done();
+    bar_workers();
+    // ---- the last row of the run: u^{k+1} of the row below comes from the next run
+    const int L = rb - 1;
+    if (ra < rb && L >= 1 && L < n - 1) {
+      const RowState s = tmem_load_row(X.taddr + (L - ra) * kChipRowCols);
+      Q4 p, q;
+      flux_row(any, L, s.ux, s.ut, lds4<kBUx + kChipRowBytes>(brow), p, q);
+      sts4<kBP>(brow, p);
+      sts4<kBQ>(brow, q);
+      if (L == ra) {
+        p_a = p;
+        q_a = q;
+      } else if (L - 1 >= 1) {  // the row above in this run: p = div u + f, q as stored
+        const unsigned a = row_addr(L - 1);
+        grad_row(any, L, p, q, add4(lds4(a), lds4<2 * kChipPlane>(a)), lds4<kChipPlane>(a));
+      }
+    }
+    bar_workers();
+    if (ra < rb && ra >= 2 && ra < n - 1)
+      grad_row(any, ra, p_a, q_a, lds4<kBP - kChipRowBytes>(brow), lds4<kBQ - kChipRowBytes>(brow));
+
+    chip_store_sums(X, v, own_lane);
+    bar_all_arrive<2>();
+    bar_all<3>();  // every CTA of the group has finished the pass
+    // ---- halo values of the pass: received div u and q
+    if (!sh.bad) {
+      if (halo_src) {
+        const float2 e = __ldcg(halo_src + (k & 1 ? xcol_set : 0));
+        sts1(halo_dst, e.x);
+        sts1(halo_dst + kChipPlane, e.y);
+      }
+      for (int w = 0; w < 2; ++w) {
+        const int r = w ? n - 1 : 0, gi = J.i0 - 2 + r, seg = J.seg + (w ? 1 : -1);
+        if (r < ra || r >= rb || seg < 0 || seg >= J.segs || gi < 0 || gi >= nr) continue;
+        const float *o = xr + (static_cast<size_t>(seg) * 2 + (w ? 0 : 1)) * 2 * ntp;
+        float d_[4], q_[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const bool in = ln.use[q];
+          d_[q] = in ? __ldcg(o + gj0 + q) : 0.0f;
+          q_[q] = in ? __ldcg(o + ntp + gj0 + q) : 0.0f;
+        }
+        sts4(row_addr(r), q4(d_[0], d_[1], d_[2], d_[3]));
+        sts4<kChipPlane>(row_addr(r), q4(q_[0], q_[1], q_[2], q_[3]));
+      }
+    }
+    bar_all<4>();  // the decision
+    ++k;
   }
-  asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-  __syncthreads();
-  if (warp == 0) tmem_free_all(sh.tmem);
+
+  // ---- finalize: phi^K, the outputs and the duality gap's sums
+  if (!sh.bad && sh.status == ST_OK) {
+    const Q4 cf = lds_pair<16>(sc_addr), th = lds_pair<32>(sc_addr);
+    Sum2 t[4];
+    for (int r = ra; r < rb; ++r) {
+      const RowState s = dual(r, cf, th);
+      tmem_store_row(X.taddr + (r - ra) * kChipRowCols, s);
+      if (r == rb - 1) sts4(brow, s.ph);
+    }
+    tmem_stores_done();
+    bar_workers();
+    const bool vec = chip_vec_out(X);
+    Q4 up = ra < rb && ra > 0 ? lds4(brow - kChipRowBytes) : q4s(0.0f);
+    for (int r = ra; r < rb; ++r) {
+      const RowState s = tmem_load_row(X.taddr + (r - ra) * kChipRowCols);
+      const Q4 gtv = diff_left(s.ph);
+      if (r >= 2 && r < J.h + 2 && own_lane)
+        chip_output_row<ISO>(X, vec, J.i0 - 2 + r, s.ux, s.ut, s.ph, up, gtv, lds4<2 * kChipPlane>(row_addr(r)), t);
+      up = s.ph;
+    }
+    chip_store_gap(X, t);
+    bar_all_arrive<2>();
+    bar_all<3>();
+  }
 }
 
 }  // namespace emd

@@ -1,11 +1,13 @@
 """The on-chip solve (default for gathers whose state fits in the GPU's shared and tensor memory)
-against the per-pass tile kernels on the same inputs, at the sizes where its layout can go wrong:
-runs of one row per warp, one row more, the tallest CTA and the first that needs a second segment,
-strips of 120 samples and their remainders, receivers and samples at the ends of the range.
+against the streaming pass of the same rounding (the tile pass below 1.4 million cells, the marching
+pass above) on the same inputs, at the sizes where its layout can go wrong: runs of one row per
+warp, one row more, the tallest CTA and the first that needs a second segment, tall CTAs, strips of
+120 samples and their remainders, receivers and samples at the ends of the range.
 
 The two paths do the same arithmetic on every cell, in the same order, so phi and m may differ
 only where a linesearch decision differs; the sums behind the decisions are added in another
-order, which moves the distance by FP32 rounding of partial sums (a few 1e-8)."""
+order, which moves the reported residual by FP32 rounding of partial sums (a few 1e-8).  Physical
+spacings keep the receiver flux shut for the first iterations; the unit square opens both."""
 
 import math
 
@@ -20,6 +22,15 @@ pytestmark = pytest.mark.gpu
 DT, DX = 2e-3, 10.0
 TILE = 7      # the TMA tile pass
 PLAIN = 2     # the plain pass (any number of receivers)
+MARCH = 10    # the marching pass
+
+
+def streaming(cells, nr):
+    return PLAIN if nr <= 8 else TILE if cells < 1.4e6 else MARCH
+
+
+def spacings(nr, nt):
+    return [(DT, DX), (1.0 / (nt - 1), 1.0 / max(nr - 1, 1))]
 
 
 @pytest.fixture(scope="module")
@@ -52,27 +63,34 @@ def check(got, ref, what=""):
 
 SHAPES = [(64, 256), (12, 700), (13, 700), (27, 400), (28, 400), (125, 120), (126, 121), (250, 1000),
           (251, 999), (9, 1201), (2, 4801), (3, 2399), (1, 9001), (640, 61), (648, 1201), (400, 3000),
-          (480, 4000)]
+(480, 4000), (353, 4001), (648, 2761), (9, 156001), (300, 5041), (648, 8000)]
 
 
+@pytest.mark.parametrize("norm", [1, 2])
 @pytest.mark.parametrize("nr,nt", SHAPES)
-def test_matches_the_tile_pass(P, nr, nt):
+def test_matches_the_streaming_pass(P, nr, nt, norm):
     o, p = pair(nr, nt)
-    tile = TILE if nr > 8 else PLAIN
-    got, ref = P.emd(o, p, DT, DX, max_iter=40), P.emd(o, p, DT, DX, max_iter=40, tile=tile)
-    assert got[3]["tile"] == 0 and got[3]["launches"] == 1  # on chip
-    check(got, ref)
-    # from a warm start, in place, and on a single iteration
-    kw = dict(phi_init=ref[1], m_init=ref[2])
-    check(P.emd(o, p, DT, DX, max_iter=15, **kw), P.emd(o, p, DT, DX, max_iter=15, tile=tile, **kw), "warm")
-    check(P.emd(o, p, DT, DX, max_iter=1, **kw), P.emd(o, p, DT, DX, max_iter=1, tile=tile, **kw), "one")
+    tile = streaming(nr * nt, nr)
+    for dt, dx in spacings(nr, nt):
+        kw = dict(norm=norm)
+        got, ref = P.emd(o, p, dt, dx, max_iter=25, **kw), P.emd(o, p, dt, dx, max_iter=25, tile=tile, **kw)
+        if (nr, nt) != (9, 156001):  # more strips than SMs: streams
+            assert got[3]["tile"] == 0 and got[3]["launches"] == 1  # on chip
+        check(got, ref)
+        # from a warm start, in place, and on a single iteration
+        kw.update(phi_init=ref[1], m_init=ref[2])
+        check(P.emd(o, p, dt, dx, max_iter=9, **kw), P.emd(o, p, dt, dx, max_iter=9, tile=tile, **kw), "warm")
+        check(P.emd(o, p, dt, dx, max_iter=1, **kw), P.emd(o, p, dt, dx, max_iter=1, tile=tile, **kw), "one")
 
 
 @pytest.mark.parametrize("kw", [dict(norm=2), dict(balance=0), dict(linesearch=0), dict(tol=1e-30, check_every=7),
                                 dict(xi=0.9), dict(alpha0=1e-3)])
-def test_options_match_the_tile_pass(P, kw):
-    o, p = pair(70, 500, seed=3)
-    check(P.emd(o, p, DT, DX, max_iter=60, **kw), P.emd(o, p, DT, DX, max_iter=60, tile=TILE, **kw), str(kw))
+def test_options_match_the_streaming_pass(P, kw):
+    for nr, nt in ((70, 500), (300, 4700), (420, 5000)):
+        o, p = pair(nr, nt, seed=3)
+        tile = streaming(nr * nt, nr)
+        for dt, dx in spacings(nr, nt):
+            check(P.emd(o, p, dt, dx, max_iter=30, **kw), P.emd(o, p, dt, dx, max_iter=30, tile=tile, **kw), str(kw))
 
 
 def test_tolerance_stop_and_trace(P):
@@ -103,13 +121,14 @@ def test_unaligned_inputs_and_outputs(P):
 
 
 def test_batch_of_uneven_gathers_one_too_large(P):
-    sizes = [(64, 256), (400, 3000), (1, 8000), (648, 8000), (33, 401), (200, 1500)]
+    sizes = [(64, 256), (400, 3000), (20, 8000), (700, 9000), (33, 401), (200, 1500)]
     pairs = [pair(nr, nt, seed=10 + i) for i, (nr, nt) in enumerate(sizes)]
     obs, pred = [a for a, _ in pairs], [b for _, b in pairs]
     d, phis, ms, infos = P.emd_batched(obs, pred, DT, DX, max_iter=30)
     assert [i["tile"] == 0 for i in infos].count(True) >= 5
-    for b, (nr, _) in enumerate(sizes):
-        ref = P.emd(obs[b], pred[b], DT, DX, max_iter=30, tile=infos[b]["tile"] or (TILE if nr > 8 else PLAIN))
+    total = sum(nr * nt for nr, nt in sizes)
+    for b, (nr, nt) in enumerate(sizes):
+        ref = P.emd(obs[b], pred[b], DT, DX, max_iter=30, tile=infos[b]["tile"] or streaming(total, 9))
         check((d[b], phis[b], ms[b], infos[b]), ref, str(sizes[b]))
 
 
