@@ -412,14 +412,12 @@ bool chip_fits(int nt, int nr, int cap, bool march) {
   const int strips = chip_strips(nt), ntp = ntp_of(nt), rows = chip_min_rows(nt, nr, cap);
   if (rows == 0 || rows > (march ? emd::kWMaxRows : emd::kChipMaxRows)) return false;
   const size_t planes = 9 * align256(sizeof(float) * static_cast<size_t>(nr) * ntp);
-  const int segs = std::max(1, (nr + 1) / 2);  // no layout has more
-  if (emd::chip_exchange_bytes(segs, strips, nr, ntp) > planes) return false;
-  if (!march) return true;
-  size_t need = 4 * emd::chip_w_exchange_floats(segs, strips, nr, ntp);
-  if (nr > emd::kChipMaxRows - 3) {
+  const int lowest = emd::kChipWorkers - 3;  // receivers of the lowest CTAs (chip_plan)
+  size_t need = emd::chip_exchange_bytes((nr + lowest - 1) / lowest, strips, nr, ntp);
+  if (march && nr > emd::kChipMaxRows - 3) {
     const int tall = (nr + emd::kChipMaxRows - 3) / (emd::kChipMaxRows - 2);  // segments of tall CTAs at most
-    need = std::max(need, 4 * (emd::chip_w_exchange_floats(tall, strips, nr, ntp) +
-                               static_cast<size_t>(tall) * strips * emd::chip_w_tall_floats((nr + tall - 1) / tall + 3)));
+    need = std::max(need, emd::chip_exchange_bytes(tall, strips, nr, ntp) +
+                              4 * static_cast<size_t>(tall) * strips * emd::chip_w_tall_floats((nr + tall - 1) / tall + 3));
   }
   return need <= planes;
 }

@@ -22,13 +22,14 @@
 // and rounding are those of the tile pass (emd_pass_tma.cuh), so both give the same iterates;
 // emd_chip_w.cuh has the same solve with the arithmetic of the marching pass.
 //
-// Pass boundary.  A CTA adds its sums to FP64 accumulators in L2 and counts itself done; the
-// decider warp of every CTA waits for the count, reads the totals and takes the same decision,
-// so no result has to be broadcast.  (Measured on 152 CTAs, with nothing else in the loop:
-// 2.2 us for add, count and read, 4.8 us for an all-to-all exchange of tagged partial sums,
-// 1.9 us through thread-block clusters of two, which would cap the grid shapes.)  div u and q
-// of the cells that neighbours hold as halo go through a small L2 buffer, ordered by the same
-// count; the workers fetch theirs while the decider warp decides.
+// Pass boundary.  No CTA waits for a broadcast or a memory barrier.  Every CTA's decider warp adds
+// the CTA's sums to a few 64-bit words in L2 whose low byte counts the CTAs that have added
+// (chip_exchange_fast); once the counts are full, every CTA reads the same totals and takes the
+// same decision.  The cells that neighbours hold as halo travel as 16-byte packets that carry the
+// pass they belong to, and the workers fetch theirs while the decider decides.  (An exchange by
+// FP64 sums, a release of a counter and its acquisition, which the first form had everywhere and
+// passes with residual sums still take, costs about 5400 cycles from the last row to the next
+// pass; see chip_exchange_fast.)
 #pragma once
 
 #include "emd_pass_tma.cuh"
@@ -45,6 +46,8 @@ constexpr int kChipTJ = 120;                            // owned time samples of
 constexpr int kChipSets = 3;                            // accumulator sets, used in turn
 constexpr int kChipVals = 8;                            // sums of a pass
 constexpr int kChipSpread = 8;                          // copies of each accumulator
+constexpr int kChipWordCopies = 4;                      // copies of the words of the fast exchange
+constexpr int kChipWords = 16;                          // two words of each value
 
 // One CTA's part of a gather.
 struct ChipJob {
@@ -56,14 +59,14 @@ struct ChipJobs {
   ChipJob job[kChipMaxCtas];
 };
 
-// Exchange buffers of a gather, in the workspace of its planes: div u and q of the first and
-// the last-but-one owned row of every segment ([parity][seg][which][2][ntp]) and of the first
-// and the last-but-one owned sample of every strip ([parity][strip][side][nr] pairs).
-__host__ __device__ inline size_t chip_row_floats(int segs, int ntp) {
-  return static_cast<size_t>(2) * segs * 2 * 2 * ntp;
+// Exchange buffers of a gather, in the workspace of its planes: packets of the cells that other CTAs
+// hold as halo, two rows of every segment ([parity][seg][which][ntp]) and two samples of every
+// strip ([parity][strip][side][nr]).
+__host__ __device__ inline size_t chip_row_packets(int segs, int ntp) {
+  return segs > 1 ? static_cast<size_t>(2) * segs * 2 * ntp : 0;
 }
 __host__ __device__ inline size_t chip_exchange_bytes(int segs, int strips, int nr, int ntp) {
-  return 4 * (chip_row_floats(segs, ntp) + static_cast<size_t>(2) * strips * 2 * nr * 2);
+  return 16 * (chip_row_packets(segs, ntp) + static_cast<size_t>(2) * strips * 2 * nr);
 }
 // Dynamic shared memory of a CTA: the planes div u, q and f at a fixed stride (so that one row
 // address serves the three of them), then four boundary rows per warp.
@@ -177,6 +180,44 @@ __device__ __forceinline__ Q4 shrink4(const Q4 &v, float al, const Q4 &inv) {
 // div u of one row from the differences of its face fluxes.
 __device__ __forceinline__ Q4 div4(const Q4 &dx_, const Q4 &dt_, const Q4 &rdx, const Q4 &rdt) {
   return fma4(dx_, rdx, mul4(dt_, rdt));
+}
+
+// ------------------------------------------------------------------ halo packets
+// Two values of a cell and the pass they belong to, written and read as one 128-bit access, so a
+// reader that sees the pass's tag has its values.
+
+struct Packet {
+  float x, y;
+  int tag;
+};
+using PacketMem = uint4;
+__device__ __forceinline__ void put_packet(PacketMem *p, float x, float y, int tag) {
+  asm volatile(
+      "{\n .reg .b64 lo, hi;\n .reg .b128 q;\n mov.b64 lo, {%1, %2};\n mov.b64 hi, {%3, %3};\n"
+      " mov.b128 q, {lo, hi};\n st.relaxed.gpu.global.b128 [%0], q;\n}\n" ::"l"(p),
+      "f"(x), "f"(y), "r"(tag)
+      : "memory");
+}
+__device__ __forceinline__ Packet get_packet(const PacketMem *p) {
+  Packet v;
+  asm volatile(
+      "{\n .reg .b32 again;\n .reg .b64 lo, hi;\n .reg .b128 q;\n ld.relaxed.gpu.global.b128 q, [%3];\n"
+      " mov.b128 {lo, hi}, q;\n mov.b64 {%0, %1}, lo;\n mov.b64 {%2, again}, hi;\n}\n"
+      : "=f"(v.x), "=f"(v.y), "=r"(v.tag)
+      : "l"(p)
+      : "memory");
+  return v;
+}
+// Repeats `ready` (a warp's attempt, true in every lane that has what it needs) until it is true in
+// all lanes; false when the bound runs out.
+template <class F>
+__device__ __forceinline__ bool poll_warp(F ready) {
+  if (__all_sync(0xffffffffu, ready())) return true;
+  const unsigned long long t0 = global_ns();
+  for (unsigned n = 0;; ++n) {
+    if (__all_sync(0xffffffffu, ready())) return true;
+    if ((n & 63u) == 63u && global_ns() - t0 > kSpinLimitNs) return false;
+  }
 }
 
 // ------------------------------------------------------------------ tensor memory as a store
@@ -293,6 +334,7 @@ struct ChipShared {
   // each value four times, so that a 16-byte load gives a Q4: alpha, coef, theta,
   // 1 / (1 + eps alpha) of the pass, then 1/dx, 1/dt
   alignas(16) float sc[6][4];
+  float warm[6][4];                          // takes what the decision writes when it runs for nothing
   float part[16][kChipVals];                 // warp totals of a pass (zero for warps that are not there)
   double dpart[16][4];                       // warp totals of the balancing sums
 };
@@ -303,7 +345,6 @@ struct ChipShared {
 // has read by now and which is added to again two passes on.  False when the bounded wait ran
 // out.  (Eight copies: two loads and three FP64 additions to read a total, each addition about
 // 70 cycles of a chain that every CTA waits for.)
-template <int NW>
 __device__ __forceinline__ bool chip_exchange(const Ctl &c, State *st, double *acc, int set, int cta,
                                               int group, unsigned step, bool adds, double x, double &v) {
   const int lane = threadIdx.x & 31;
@@ -312,7 +353,6 @@ __device__ __forceinline__ bool chip_exchange(const Ctl &c, State *st, double *a
   __syncwarp();
   if (lane == 0 && c.debug_fault != 2) red_release_add(&st->tiles_done, 1u);
   if (!__all_sync(0xffffffffu, wait_count(&st->tiles_done, step * static_cast<unsigned>(group)))) return false;
-  bar_all_arrive<3, NW>();  // the workers may fetch their halos
   static_assert(kChipSpread == 8 && kChipVals == 8, "two copies per lane");
   const double x0 = __ldcg(a + lane), x1 = __ldcg(a + 32 + lane);  // copies lane / 8 and 4 + lane / 8
   v = sum_groups(x0 + x1);
@@ -324,16 +364,15 @@ __device__ __forceinline__ bool chip_exchange(const Ctl &c, State *st, double *a
   return true;
 }
 
-// This CTA's totals over its worker warps, exactly rounded to a pair (hi, lo) of floats that
-// every lane holds for value lane & 7; returned is hi in lanes 0..7 and lo in the others, so
-// that lanes 0..15 add both.  (Two-sums are 4-cycle operations; FP64 takes 64 cycles for each
-// of the nine conversions and additions.)
-__device__ __forceinline__ double chip_block_total(const ChipShared &sh) {
+// The totals over a CTA's warps of their FP32 totals, to a pair (hi, lo) of floats that every lane
+// holds for value lane & 7.  (Two-sums are 4-cycle operations; FP64 takes 64 cycles for each of
+// the nine conversions and additions.)
+__device__ __forceinline__ void chip_block_pair(const float (&part)[16][kChipVals], float &s, float &e) {
   constexpr unsigned FULL = 0xffffffffu;
   const int lane = threadIdx.x & 31, g = lane >> 3, q = lane & 7;
-  float s0, e0, s1, e1, s, e;
-  two_sum(sh.part[g][q], sh.part[g + 4][q], s0, e0);
-  two_sum(sh.part[g + 8][q], sh.part[g + 12][q], s1, e1);
+  float s0, e0, s1, e1;
+  two_sum(part[g][q], part[g + 4][q], s0, e0);
+  two_sum(part[g + 8][q], part[g + 12][q], s1, e1);
   two_sum(s0, s1, s, e);
   e += e0 + e1;
 #pragma unroll
@@ -343,7 +382,79 @@ __device__ __forceinline__ double chip_block_total(const ChipShared &sh) {
     s = s0;
     e = (e + eo) + e0;
   }
-  return static_cast<double>(lane < 8 ? s : e);
+}
+// hi in lanes 0..7 and lo in the others, so that lanes 0..15 add both.
+__device__ __forceinline__ double chip_block_total(const ChipShared &sh) {
+  float s, e;
+  chip_block_pair(sh.part, s, e);
+  return static_cast<double>((threadIdx.x & 31) < 8 ? s : e);
+}
+
+// The exchange of a pass's six linesearch sums.  A value x of a CTA (the pair s + e of lane & 7) is
+// taken in fixed point, x = (A + B 2^-46) 2^-sa with integers |A| < 2^38 and |B| <= 2^46, and
+// added as the two words 256 A + 1 and 256 B + 1: the low byte of a word counts the CTAs that have
+// added to it, so one poll brings the totals and says whether they are complete, with no barrier
+// between data and counter (1000 cycles) and no second read (700).  The integers add exactly in
+// any order.  sa puts the last pass's total of the value's family (p: P_pp, P_qq; grad p: G_pp,
+// G_qq) at 2^24, so a value keeps 24 bits down to 2^-46 of it and may grow 2^14 fold; a CTA whose
+// value does not fit adds 2^47 for it, every CTA sees the total beyond 2^46 and all of them take
+// the FP64 exchange for this pass.  v: the total in FP32; a, b: in fixed point.
+struct FastTotal {
+  long long a, b;
+  float v;
+  bool fits;
+};
+__device__ __forceinline__ void chip_fast_add(const Ctl &c, unsigned long long *words, int set, int cta, float s, float e,
+                                              int sa) {
+  const int lane = threadIdx.x & 31, q = lane & 7;
+  unsigned long long *const w = words + set * (kChipWordCopies * kChipWords);
+  const float scale = __int_as_float((127 + sa) << 23);
+  const float hs = q < 6 ? s * scale : 0.0f, ls = q < 6 ? e * scale : 0.0f;
+  const bool fits = fabsf(hs) < 0x1p38f;  // false for a NaN too
+  const float a1 = rintf(hs), a2 = rintf(ls);
+  const long long ia = fits ? __float2ll_rn(a1) + __float2ll_rn(a2) : 1ll << 47;
+  const long long ib = fits ? __float2ll_rn((hs - a1) * 0x1p46f) + __float2ll_rn((ls - a2) * 0x1p46f) : 0;
+  if (lane < 16 && c.debug_fault != 2)
+    atomicAdd(w + (cta % kChipWordCopies) * kChipWords + 2 * q + (lane >> 3),
+              (static_cast<unsigned long long>(lane < 8 ? ia : ib) << 8) + 1u);
+}
+__device__ __forceinline__ bool chip_fast_poll(unsigned long long *words, int set, int cta, int group, int sa,
+                                               FastTotal &o) {
+  constexpr unsigned FULL = 0xffffffffu;
+  const int lane = threadIdx.x & 31, q = lane & 7;
+  unsigned long long *const w = words + set * (kChipWordCopies * kChipWords);
+  unsigned long long x = 0, y = 0;
+  const unsigned long long *const src = w + (lane >> 3) * kChipWords + 2 * q;
+  const bool ok = poll_warp([&] {
+    asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];\n" : "=l"(x), "=l"(y) : "l"(src) : "memory");
+#pragma unroll
+    for (int d = 8; d <= 16; d <<= 1) {
+      x += __shfl_xor_sync(FULL, x, d);
+      y += __shfl_xor_sync(FULL, y, d);
+    }
+    return static_cast<int>(x & 255u) == group && static_cast<int>(y & 255u) == group;
+  });
+  o.a = static_cast<long long>(x) >> 8;
+  o.b = static_cast<long long>(y) >> 8;
+  o.v = fmaf(__ll2float_rn(o.b), 0x1p-46f, __ll2float_rn(o.a)) * __int_as_float((127 - sa) << 23);
+  o.fits = __all_sync(FULL, llabs(o.a) < (1ll << 46));
+  if (cta == 0) {  // the set of the exchange before, which every CTA has read; added to again two exchanges on
+    unsigned long long *const z = words + ((set + kChipSets - 1) % kChipSets) * (kChipWordCopies * kChipWords);
+    z[lane] = 0u;
+    z[32 + lane] = 0u;
+  }
+  return ok;
+}
+
+// xi^lane, by the multiplications of decide_prep_lanes.
+__device__ __forceinline__ double xi_power(double xi) {
+  double xl = 1.0, base = xi;
+#pragma unroll
+  for (int b = 0; b < 5; ++b) {
+    if (((threadIdx.x & 31) >> b) & 1) xl *= base;
+    base *= base;
+  }
+  return xl;
 }
 
 // FP32 copies of a decision's prepared coefficients, for the quick test below.
@@ -351,33 +462,50 @@ struct QuickPrep {
   float s2x, s2, cl;
   bool usable;
 };
-__device__ __forceinline__ QuickPrep quick_prep(const DecidePrep &d) {
+// What a decision needs besides the sums, while the pass runs: per lane the step sizes that trial
+// would accept, and the quick test's coefficients from their FP32 copies.  (The FP64 test's own
+// coefficients, decide_prep_lanes, only when that runs: with them, the FP64 of this preparation
+// took 4600 cycles, longer than the pass of a small gather.)
+__device__ __forceinline__ QuickPrep step_prep(const Ctl &c, DecidePrep &d, double xl) {
+  d.s_lane = sqrt(1.0 + d.theta) * xl;
+  d.alpha_l = d.alpha * d.s_lane;
+  d.coef_l = c.delta * d.alpha_l;
+  d.alpha_lf = static_cast<float>(d.alpha_l);
+  d.coef_lf = static_cast<float>(d.coef_l);
+  d.theta_lf = static_cast<float>(d.s_lane);
+  d.inv_lf = 1.0f / (1.0f + static_cast<float>(c.eps * d.alpha_l));
+  const float zeta = static_cast<float>(c.zeta);
   QuickPrep p;
-  p.s2x = static_cast<float>(d.s2x);
-  p.s2 = static_cast<float>(d.s_lane2);
-  p.cl = static_cast<float>(d.cl);
+  p.s2x = 2.0f * d.theta_lf;
+  p.s2 = d.theta_lf * d.theta_lf;
+  p.cl = d.coef_lf * d.alpha_lf / (zeta * zeta);
   p.usable = p.cl > 1e-25f && p.cl < 1e25f;
   return p;
 }
 
-// The linesearch decision from FP32 copies of the totals (v: value lane & 7), where those settle
+// An FP64 total cut to FP32 by integer operations (a conversion would take the FP64 pipe): exact
+// to 23 bits within 2^-60 .. 2^60, else 0 (an infinity for one that is not finite).
+__device__ __forceinline__ float cut_f32(double v) {
+  const int hi = __double2hiint(v), lo = __double2loint(v);
+  const int ex = (hi >> 20) & 0x7ff;
+  const float f = __int_as_float((hi & 0x80000000) | ((ex - 896) << 23) | ((hi & 0xfffff) << 3) |
+                                 static_cast<int>(static_cast<unsigned>(lo) >> 29));
+  return ex > 1023 - 60 && ex < 1023 + 60 ? f : ex == 0x7ff ? INFINITY : 0.0f;
+}
+
+// The linesearch decision from FP32 copies of the totals (f: value lane & 7), where those settle
 // it: a trial counts as decided when the two sides of its test differ by more than 1e-5 of the
-// magnitudes that enter them, ten times what truncating the totals to 24 bits and the few FP32
+// magnitudes that enter them, ten times what rounding the totals to 24 bits and the few FP32
 // operations can move them, so the FP64 test would decide alike.  Returns the trial (0-based),
 // or -1 where FP64 has to look (near ties, zeros, values outside 2^-60 .. 2^60, non-finite
 // sums, no passing trial among the first 32).  The FP64 test is five dependent operations of
 // about 70 cycles for every CTA to wait for.
-__device__ __forceinline__ int quick_decide(const Ctl &c, const QuickPrep &p, double v) {
+__device__ __forceinline__ int quick_decide(const Ctl &c, const QuickPrep &p, float f) {
   constexpr unsigned FULL = 0xffffffffu;
   const int lane = threadIdx.x & 31;
-  const int hi = __double2hiint(v), lo = __double2loint(v);
-  const int ex = (hi >> 20) & 0x7ff;
-  const bool in_range = ex > 1023 - 60 && ex < 1023 + 60;
-  const float f = in_range ? __int_as_float((hi & 0x80000000) | ((ex - 896) << 23) | ((hi & 0xfffff) << 3) |
-                                            static_cast<int>(static_cast<unsigned>(lo) >> 29))
-                           : 0.0f;
   // values 6 and 7 (the residual's) only have to be finite
-  if (!__all_sync(FULL, (lane & 7) < 6 ? in_range : ex != 0x7ff)) return -1;
+  const float mag_f = fabsf(f);
+  if (!__all_sync(FULL, (lane & 7) < 6 ? mag_f > 0x1p-60f && mag_f < 0x1p60f : mag_f < INFINITY)) return -1;
   float a[6];
 #pragma unroll
   for (int q = 0; q < 6; ++q) a[q] = __shfl_sync(FULL, f, q);
@@ -558,7 +686,9 @@ __device__ __forceinline__ void chip_decider(const ChipCta &X) {
   const int lane = X.lane, nr = X.nr, nt = X.nt, cta = X.cta;
   const float rdx = S.rdx, rdt = S.rdt;
   double *const acc = acc_of(c, J.gather);
-  static_assert(kChipSets * kChipSpread * kChipVals <= kAccBufs * kSpread * kAcc, "a gather's accumulators");
+  constexpr int kSlow = kChipSets * kChipSpread * kChipVals;  // doubles of the FP64 exchange, then the words
+  static_assert(kSlow + kChipSets * kChipWordCopies * kChipWords <= kAccBufs * kSpread * kAcc, "a gather's accumulators");
+  unsigned long long *const words = reinterpret_cast<unsigned long long *>(acc + kSlow);
   // the balancing sums: f, f^2, |Pcal| + |Pobs|, Pcal - Pobs
   bar_all<2, NW>();
   double v = 0.0;
@@ -571,8 +701,7 @@ __device__ __forceinline__ void chip_decider(const ChipCta &X) {
   v = sum_groups(v);
   unsigned step = 1;
   int set = 0;
-  bool ok = chip_exchange<NW>(c, st, acc, set, cta, J.group, step, lane < 8, v, v);
-  if (!ok) bar_all_arrive<3, NW>();
+  bool ok = chip_exchange(c, st, acc, set, cta, J.group, step, lane < 8, v, v);
   DecidePrep pr;
   pr.k = 0;
   double m4[4];
@@ -586,11 +715,11 @@ __device__ __forceinline__ void chip_decider(const ChipCta &X) {
   pr.theta = 1.0;
   pr.coef = 0.0;  // pass 0: phi^0 is the initial potential
   // the values of the next pass, each written four times (lane 4 q + i: copy i of value q)
-  auto publish_sc = [&](float alpha, float coef, float theta, float inv) {
+  auto publish_sc = [&](float (&dst)[6][4], float alpha, float coef, float theta, float inv) {
     const int q = lane >> 2;
-    if (lane < 16) sh.sc[q][lane & 3] = q == 0 ? alpha : q == 1 ? coef : q == 2 ? theta : inv;
+    if (lane < 16) dst[q][lane & 3] = q == 0 ? alpha : q == 1 ? coef : q == 2 ? theta : inv;
   };
-  publish_sc(static_cast<float>(pr.alpha), 0.0f, 1.0f, 1.0f / (1.0f + static_cast<float>(c.eps * pr.alpha)));
+  publish_sc(sh.sc, static_cast<float>(pr.alpha), 0.0f, 1.0f, 1.0f / (1.0f + static_cast<float>(c.eps * pr.alpha)));
   if (lane >= 16 && lane < 24) sh.sc[lane >> 2][lane & 3] = lane < 20 ? rdx : rdt;
   if (lane == 0) {
     sh.fmean = static_cast<float>(fmean);
@@ -602,25 +731,59 @@ __device__ __forceinline__ void chip_decider(const ChipCta &X) {
   bool done = false;
   int status = ST_OK;
   const bool quick = c.linesearch && c.debug_fault != 1;
+  // fixed-point exponents of the two families for the next fast exchange
+  int fset = 0, e_p = 0, e_g = 0;
+  bool scaled = false;
+  const double xl = xi_power(c.xi);
+  constexpr unsigned FULL = 0xffffffffu;
   while (ok && !done) {
-    decide_prep_lanes(c, pr);  // overlaps the pass
-    const QuickPrep qp = quick_prep(pr);
+    const QuickPrep qp = step_prep(c, pr, xl);  // overlaps the pass
+    // passes with residual sums (and those without a scale yet) take the FP64 exchange
+    const bool check = c.tol > 0.0 && (pr.k + 1) % c.check_every == 0;
+    bool slow = !scaled || check || pr.k + 1 >= c.max_iter;
     bar_all<2, NW>();
-    const double mine = chip_block_total(sh);
-    ++step;
-    set = (set + 1) % kChipSets;
-    ok = chip_exchange<NW>(c, st, acc, set, cta, J.group, step, lane < 16, mine, v);
+    float hi, lo, f = 0.0f;
+    chip_block_pair(sh.part, hi, lo);
+    FastTotal ft;
+    const int sa = 24 - ((lane & 7) < 3 ? e_p : e_g);
+    // The decision's instructions have left the instruction cache since the last pass (1300 cycles
+    // against 300): they run once for nothing (into sh.warm) while the other CTAs' sums arrive.
+    int w = -1;
+    if (!slow) chip_fast_add(c, words, fset, cta, hi, lo, sa);
+#pragma unroll 1
+    for (int real = slow ? 2 : 0; real < 2; ++real) {
+      if (real) {
+        ok = chip_fast_poll(words, fset, cta, J.group, sa, ft);
+        f = ft.v;
+      } else {
+        f = hi;
+      }
+      w = quick ? quick_decide(c, qp, f) : -1;
+      publish_sc(real ? sh.sc : sh.warm, __shfl_sync(FULL, pr.alpha_lf, w & 31), __shfl_sync(FULL, pr.coef_lf, w & 31),
+                 __shfl_sync(FULL, pr.theta_lf, w & 31), __shfl_sync(FULL, pr.inv_lf, w & 31));
+    }
+    if (!slow) {
+      fset = (fset + 1) % kChipSets;
+      slow = !ft.fits;
+    }
+    if (ok && slow) {
+      ++step;
+      set = (set + 1) % kChipSets;
+      ok = chip_exchange(c, st, acc, set, cta, J.group, step, lane < 16, static_cast<double>(lane < 8 ? hi : lo), v);
+      f = cut_f32(v);
+      w = quick && !check ? quick_decide(c, qp, f) : -1;
+      if (w >= 0)
+        publish_sc(sh.sc, __shfl_sync(FULL, pr.alpha_lf, w), __shfl_sync(FULL, pr.coef_lf, w),
+                   __shfl_sync(FULL, pr.theta_lf, w), __shfl_sync(FULL, pr.inv_lf, w));
+    }
     if (!ok) {
-      bar_all_arrive<3, NW>();
       if (lane == 0) sh.bad = 1;
       bar_all<4, NW>();
       break;
     }
-    const int w = quick && !pr.check ? quick_decide(c, qp, v) : -1;
+    if (!slow && (w < 0 || c.trace))
+      v = fma(static_cast<double>(ft.b), 0x1p-46, static_cast<double>(ft.a)) * __hiloint2double((1023 - sa) << 20, 0);
     if (w >= 0) {
-      constexpr unsigned FULL = 0xffffffffu;
-      publish_sc(__shfl_sync(FULL, pr.alpha_lf, w), __shfl_sync(FULL, pr.coef_lf, w),
-                 __shfl_sync(FULL, pr.theta_lf, w), __shfl_sync(FULL, pr.inv_lf, w));
       done = pr.k + 1 >= c.max_iter;
       if (lane == 0) sh.done = done;
       bar_all<4, NW>();
@@ -644,11 +807,12 @@ __device__ __forceinline__ void chip_decider(const ChipCta &X) {
       a_[6] = 0.0;
       a_[7] = __shfl_sync(0xffffffffu, v, 6);
       a_[8] = __shfl_sync(0xffffffffu, v, 7);
+      decide_prep_lanes(c, pr);
       const Decision o = decide_core(c, pr, a_);
       trials += o.trials_now;
       done = o.done;
       status = o.status;
-      if (o.status == ST_OK) publish_sc(o.alpha_f, o.coef_f, o.theta_f, o.inv_f);
+      if (o.status == ST_OK) publish_sc(sh.sc, o.alpha_f, o.coef_f, o.theta_f, o.inv_f);
       if (lane == 0) {
         sh.status = o.status;
         sh.done = o.done;
@@ -663,6 +827,15 @@ __device__ __forceinline__ void chip_decider(const ChipCta &X) {
         pr.coef = o.coef;
       }
     }
+    if (sh.bad) ok = false;  // a worker's wait ran out
+    {
+      const float p2 = fmaxf(__shfl_sync(FULL, f, 0), __shfl_sync(FULL, f, 2));
+      const float g2 = fmaxf(__shfl_sync(FULL, f, 3), __shfl_sync(FULL, f, 5));
+      scaled = p2 > 0x1p-60f && p2 < 0x1p60f && g2 > 0x1p-60f && g2 < 0x1p60f;
+      e_p = (__float_as_int(p2) >> 23) - 127;
+      e_g = (__float_as_int(g2) >> 23) - 127;
+    }
+    fence_acq_rel_gpu();  // orders this pass's reads and zeros before the next pass's sums
   }
   // the last pass's sums (or, when no pass ran, the balancing ones, which nobody reads)
   const double s_p2 = __shfl_sync(0xffffffffu, v, 0), s_u2 = __shfl_sync(0xffffffffu, v, 6),
@@ -673,8 +846,7 @@ __device__ __forceinline__ void chip_decider(const ChipCta &X) {
     const double mine = chip_block_total(sh);
     ++step;
     set = (set + 1) % kChipSets;
-    ok = chip_exchange<NW>(c, st, acc, set, cta, J.group, step, lane < 16, mine, gap);
-    if (!ok) bar_all_arrive<3, NW>();
+    ok = chip_exchange(c, st, acc, set, cta, J.group, step, lane < 16, mine, gap);
   }
   if (!ok && lane == 0) atomicExch(c.error, 1);
   double g4[4];
@@ -720,13 +892,49 @@ __device__ __forceinline__ void chip_worker(const ChipCta &X) {
   constexpr unsigned kBUx = kChipBound;           // u^{k+1} (x) of a run's first row
   constexpr unsigned kBP = 2 * kChipBound, kBQ = 3 * kChipBound;  // p, q of a run's last row
   // exchange buffers
-  float *const xrow = S.f;
-  float2 *const xcol = reinterpret_cast<float2 *>(S.f + chip_row_floats(J.segs, ntp));
+  PacketMem *const xrow = reinterpret_cast<PacketMem *>(S.f), *const xcol = xrow + chip_row_packets(J.segs, ntp);
+  const size_t xrow_set = static_cast<size_t>(J.segs) * 2 * ntp, xcol_set = static_cast<size_t>(J.strips) * 2 * nr;
   const ChipLane ln = chip_lane(X);
   const bool own_lane = ln.own;
   const Q4 rdt_m = q4(ln.rm[0], ln.rm[1], ln.rm[2], ln.rm[3]);
   auto row_addr = [&](int r) { return plane + static_cast<unsigned>(r) * kChipRowBytes; };
   const unsigned brow = bound + static_cast<unsigned>(warp) * kChipRowBytes;  // this run's boundary row
+
+  // div u and q of the strip's first and last-but-one sample go to the neighbouring strips, those of
+  // the segment's first and last-but-one row to the neighbouring segments
+  const bool edge_lane = lane == 1 || lane == 30;
+  PacketMem *const xedge = xcol + (static_cast<size_t>(J.strip) * 2 + (lane == 30 ? 1 : 0)) * nr + J.i0 - 2;
+  PacketMem *const xmine = xrow + static_cast<size_t>(J.seg) * 2 * ntp + gj0;
+  auto put_row = [&](int which, int parity, const Q4 &d, const Q4 &q, int tag) {
+    float d_[4], q_[4];
+    un4(d, d_);
+    un4(q, q_);
+    PacketMem *const o = xmine + (parity ? xrow_set : 0) + which * ntp;
+    if (own_lane && gj0 < ntp && J.segs > 1) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) put_packet(o + i, d_[i], q_[i], tag);
+    }
+  };
+  // this CTA's packets start without a tag
+  for (int r = max(ra, 2); r < min(rb, J.h + 2); ++r) {
+#pragma unroll
+    for (int m = 0; m < 2; ++m) {
+      if (edge_lane) put_packet(xedge + (m ? xcol_set : 0) + r, 0.0f, 0.0f, 0);
+      if (r == 2) put_row(0, m, q4s(0.0f), q4s(0.0f), 0);
+      if (r == J.h) put_row(1, m, q4s(0.0f), q4s(0.0f), 0);
+    }
+  }
+  // the halo sample that this lane fetches: even lanes sample -2, odd ones sample 120 of the
+  // run's row lane / 2 (rows 0 and n - 1 come whole)
+  const PacketMem *halo_src = nullptr;
+  unsigned halo_dst = 0;
+  {
+    const int r = ra + (lane >> 1), side = lane & 1, gi = J.i0 - 2 + r, strip = J.strip + (side ? 1 : -1);
+    if (r < rb && r > 0 && r < n - 1 && gi >= 0 && gi < nr && strip >= 0 && strip < J.strips) {
+      halo_src = xcol + (static_cast<size_t>(strip) * 2 + (side ? 0 : 1)) * nr + gi;
+      halo_dst = row_addr(r) - 16u * lane + (side ? 4 * 124 : 4 * 2);
+    }
+  }
 
   // ---- inputs, warm start and the balancing sums
   {
@@ -762,7 +970,6 @@ __device__ __forceinline__ void chip_worker(const ChipCta &X) {
     tmem_stores_done();
     sums.store(X);
     bar_all<2>();
-    bar_all<3>();
     bar_all<4>();
     const float fm = sh.fmean;
     for (int r = ra; r < rb; ++r) {  // the balanced f, zero outside the gather
@@ -784,21 +991,6 @@ __device__ __forceinline__ void chip_worker(const ChipCta &X) {
     s.ph = fma4(cf, fma4(th, lds4<kChipPlane>(a), p), s.ph);
     return s;
   };
-  // div u and q of the strip's first and last-but-one sample go to the neighbouring strips
-  const bool edge_lane = lane == 1 || lane == 30;
-  float2 *const xedge = xcol + (static_cast<size_t>(J.strip) * 2 + (lane == 30 ? 1 : 0)) * nr + J.i0 - 2;
-  const size_t xcol_set = static_cast<size_t>(J.strips) * 2 * nr;  // pairs of one parity
-  // the halo sample that this lane fetches: even lanes sample -2, odd ones sample 120 of the
-  // run's row lane / 2 (rows 0 and n - 1 come whole)
-  const float2 *halo_src = nullptr;
-  unsigned halo_dst = 0;
-  {
-    const int r = ra + (lane >> 1), side = lane & 1, gi = J.i0 - 2 + r, strip = J.strip + (side ? 1 : -1);
-    if (r < rb && r > 0 && r < n - 1 && gi >= 0 && gi < nr && strip >= 0 && strip < J.strips) {
-      halo_src = xcol + (static_cast<size_t>(strip) * 2 + (side ? 0 : 1)) * nr + gi;
-      halo_dst = row_addr(r) - 16u * lane + (side ? 4 * 124 : 4 * 2);
-    }
-  }
   const unsigned sc_addr = smem_u32(&sh.sc[0][0]);
 
   int k = 0;
@@ -828,8 +1020,8 @@ __device__ __forceinline__ void chip_worker(const ChipCta &X) {
         v[7] = fma2(dx_.b, dx_.b, fma2(dt_.b, dt_.b, v[7]));
       }
     };
-    float *const xr = xrow + static_cast<size_t>(k & 1) * J.segs * 4 * ntp;
-    float2 *const xe = xedge + (k & 1 ? xcol_set : 0);
+    PacketMem *const xe = xedge + (k & 1 ? xcol_set : 0);
+    const int tag = k + 1;
     // p, q of a row, its sums that need no other row, and the halo cells others hold
     // (PLAIN: an owned row that no other segment holds as halo)
     auto flux_row = [&](auto plain, int r, const Q4 &ux, const Q4 &ut, const Q4 &ux_dn, Q4 &p, Q4 &q) {
@@ -852,21 +1044,9 @@ __device__ __forceinline__ void chip_worker(const ChipCta &X) {
         float d0, q0, unused;
         upk(de, d0, unused);
         upk(qe, q0, unused);
-        if (edge_lane) __stcg(xe + r, make_float2(d0, q0));
-        if (!PLAIN && (r == 2 || r == J.h)) {  // rows that the neighbouring segments hold as halo
-          float d_[4], q_[4];
-          un4(dn, d_);
-          un4(q, q_);
-          if (own_lane && gj0 < ntp) {
-#pragma unroll
-            for (int w = 0; w < 2; ++w) {
-              if (r != (w ? J.h : 2)) continue;
-              float *o = xr + (static_cast<size_t>(J.seg) * 2 + w) * 2 * ntp + gj0;
-              __stcg(reinterpret_cast<float4 *>(o), make_float4(d_[0], d_[1], d_[2], d_[3]));
-              __stcg(reinterpret_cast<float4 *>(o + ntp), make_float4(q_[0], q_[1], q_[2], q_[3]));
-            }
-          }
-        }
+        if (edge_lane) put_packet(xe + r, d0, q0, tag);
+        if (!PLAIN && r == 2) put_row(0, k & 1, dn, q, tag);
+        if (!PLAIN && r == J.h) put_row(1, k & 1, dn, q, tag);
       }
     };
     // receiver-direction gradient sums of row r from p, q of it and of the row above
@@ -963,29 +1143,40 @@ __device__ __forceinline__ void chip_worker(const ChipCta &X) {
 
     chip_store_sums(X, v, own_lane);
     bar_all_arrive<2>();
-    bar_all<3>();  // every CTA of the group has finished the pass
     // ---- halo values of the pass: received div u and q
-    if (!sh.bad) {
+    bool got = true;
+    if (ra < rb) {
+      Packet e;
+      got = poll_warp([&] {
+        if (halo_src) e = get_packet(halo_src + (k & 1 ? xcol_set : 0));
+        return !halo_src || e.tag == tag;
+      });
       if (halo_src) {
-        const float2 e = __ldcg(halo_src + (k & 1 ? xcol_set : 0));
         sts1(halo_dst, e.x);
         sts1(halo_dst + kChipPlane, e.y);
       }
       for (int w = 0; w < 2; ++w) {
         const int r = w ? n - 1 : 0, gi = J.i0 - 2 + r, seg = J.seg + (w ? 1 : -1);
         if (r < ra || r >= rb || seg < 0 || seg >= J.segs || gi < 0 || gi >= nr) continue;
-        const float *o = xr + (static_cast<size_t>(seg) * 2 + (w ? 0 : 1)) * 2 * ntp;
-        float d_[4], q_[4];
+        const PacketMem *const o = xrow + (k & 1 ? xrow_set : 0) + (static_cast<size_t>(seg) * 2 + (w ? 0 : 1)) * ntp + gj0;
+        float d_[4] = {0.f, 0.f, 0.f, 0.f}, q_[4] = {0.f, 0.f, 0.f, 0.f};
+        got = poll_warp([&] {
+          bool all = true;
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const bool in = ln.use[q];
-          d_[q] = in ? __ldcg(o + gj0 + q) : 0.0f;
-          q_[q] = in ? __ldcg(o + ntp + gj0 + q) : 0.0f;
-        }
+          for (int i = 0; i < 4; ++i) {
+            if (!ln.use[i]) continue;
+            const Packet x = get_packet(o + i);
+            d_[i] = x.x;
+            q_[i] = x.y;
+            all = all && x.tag == tag;
+          }
+          return all;
+        }) && got;
         sts4(row_addr(r), q4(d_[0], d_[1], d_[2], d_[3]));
         sts4<kChipPlane>(row_addr(r), q4(q_[0], q_[1], q_[2], q_[3]));
       }
     }
+    if (!got && lane == 0) sh.bad = 1;
     bar_all<4>();  // the decision
     ++k;
   }
@@ -1012,7 +1203,6 @@ __device__ __forceinline__ void chip_worker(const ChipCta &X) {
     }
     chip_store_gap(X, t);
     bar_all_arrive<2>();
-    bar_all<3>();
   }
 }
 

@@ -46,15 +46,9 @@ static_assert(2 * ((kChipMaxRows + kChipWorkers - 1) / kChipWorkers) + 4 <= WLay
                   (kChipMaxRows + kChipWorkers - 1) / kChipWorkers <= WLayout<kChipWorkers>::kTmemRows + 1,
               "a run of 9 rows has no streamed values");
 
-// Exchange buffers, in floats: [parity][seg][3][ntp] rows (ux and ut of the last-but-one owned row,
-// ux of the second one), then [parity][strip][3][nr] samples (ut of the second owned sample and of
-// the last-but-one, and ux of the latter, which the isotropic cost couples to ut), then, for tall CTAs, [cta][5][rows][128] streamed values.
-__host__ __device__ inline size_t chip_w_row_floats(int segs, int ntp) {
-  return static_cast<size_t>(2) * segs * 3 * ntp;
-}
-__host__ __device__ inline size_t chip_w_exchange_floats(int segs, int strips, int nr, int ntp) {
-  return chip_w_row_floats(segs, ntp) + ((static_cast<size_t>(2) * strips * 3 * nr + 3) & ~static_cast<size_t>(3));
-}
+// The exchange buffers (packets: ux, ut of the last-but-one owned row; ux of the second one; ut of the
+// second owned sample and ut, ux of the last-but-one) are followed, for tall CTAs, by [cta][5][rows]
+// [128] streamed values.
 __host__ __device__ inline size_t chip_w_tall_floats(int rows) { return static_cast<size_t>(rows) * 5 * 128; }
 
 __device__ __forceinline__ Q4 ldg4(const float *p) {
@@ -156,7 +150,7 @@ __device__ __forceinline__ void chip_worker_w(const ChipCta &X) {
     a_u = slots + static_cast<unsigned>(run - 4 * kWTmemRows) * kChipRowBytes;
     a_f = slots + static_cast<unsigned>(run + 4 * nu - f_lo) * kChipRowBytes;
     tall_plane = static_cast<size_t>(J.rows) * 128;
-    tall = S.f + chip_w_exchange_floats(J.segs, J.strips, nr, ntp) + X.cta * chip_w_tall_floats(J.rows) + 4 * lane;
+    tall = S.f + chip_exchange_bytes(J.segs, J.strips, nr, ntp) / 4 + X.cta * chip_w_tall_floats(J.rows) + 4 * lane;
   } else {
     constexpr unsigned kRun = (kChipMaxRows + kChipWorkers - 1) / kChipWorkers;
     a_f = slots + kRun * kChipRowBytes;
@@ -200,6 +194,32 @@ __device__ __forceinline__ void chip_worker_w(const ChipCta &X) {
   };
   const unsigned brow = X.smem + kWBound + static_cast<unsigned>(warp) * kChipRowBytes;  // this run's boundary row
   auto bux = [&](int m) { return brow + kWBUx + static_cast<unsigned>(m) * kWBUxSlot; };
+  // exchange buffers
+  PacketMem *const xrow = reinterpret_cast<PacketMem *>(S.f), *const xcol = xrow + chip_row_packets(J.segs, ntp);
+  const size_t xrow_set = static_cast<size_t>(J.segs) * 2 * ntp, xcol_set = static_cast<size_t>(J.strips) * 2 * nr;
+  const bool edge_lane = lane == 1 || lane == 30;
+  PacketMem *const xedge = xcol + (static_cast<size_t>(J.strip) * 2 + (lane == 30 ? 1 : 0)) * nr + J.i0 - 2;
+  PacketMem *const xmine = xrow + static_cast<size_t>(J.seg) * 2 * ntp + gj0;
+  auto put_row = [&](int which, int parity, const Q4 &ux, const Q4 &ut, int tag) {
+    float x[4], t[4];
+    un4(ux, x);
+    un4(ut, t);
+    PacketMem *const o = xmine + (parity ? xrow_set : 0) + which * ntp;
+    if (own_lane && gj0 < ntp && J.segs > 1) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) put_packet(o + i, x[i], t[i], tag);
+    }
+  };
+  // this CTA's packets start without a tag
+  for (int r = max(ra, 2); r < min(rb, J.h + 2); ++r) {
+#pragma unroll
+    for (int m = 0; m < 2; ++m) {
+      if (edge_lane) put_packet(xedge + (m ? xcol_set : 0) + r, 0.0f, 0.0f, 0);
+      if (r == J.h) put_row(0, m, q4s(0.0f), q4s(0.0f), 0);
+      if (r == 3) put_row(1, m, q4s(0.0f), q4s(0.0f), 0);
+    }
+  }
+
   // ---- inputs, warm start and the balancing sums
   {
     BalanceSums sums;
@@ -239,7 +259,6 @@ __device__ __forceinline__ void chip_worker_w(const ChipCta &X) {
     tmem_stores_done();
     sums.store(X);
     bar_all<2, NW>();
-    bar_all<3, NW>();
     bar_all<4, NW>();
     const float fm = sh.fmean;
     for (int r = ra; r < rb; ++r) {  // the balanced f, zero outside the gather
@@ -253,11 +272,6 @@ __device__ __forceinline__ void chip_worker_w(const ChipCta &X) {
     }
   }
 
-  // exchange buffers
-  const size_t xrow_set = static_cast<size_t>(J.segs) * 3 * ntp, xcol_set = static_cast<size_t>(J.strips) * 3 * nr;
-  float *const xcol = S.f + chip_w_row_floats(J.segs, ntp);
-  const bool edge_lane = lane == 1 || lane == 30;
-  float *const xedge = xcol + (static_cast<size_t>(J.strip) * 3 + (lane == 30 ? 1 : 0)) * nr + J.i0 - 2;
   const unsigned sc_addr = smem_u32(&sh.sc[0][0]);
 
   struct Row {
@@ -280,8 +294,8 @@ __device__ __forceinline__ void chip_worker_w(const ChipCta &X) {
     f32x2 v[8];
 #pragma unroll
     for (int q = 0; q < 8; ++q) v[q] = 0ull;
-    float *const xr = S.f + (mb ? xrow_set : 0);
-    float *const xe = xedge + (mb ? xcol_set : 0);
+    PacketMem *const xe = xedge + (mb ? xcol_set : 0);
+    const int tag = k + 1;
     const uint32_t tb = X.taddr + 8 * mb, tn = X.taddr + 8 * mn;
 
     auto fetch = [&](int r, Pre &p) {
@@ -310,15 +324,11 @@ __device__ __forceinline__ void chip_worker_w(const ChipCta &X) {
       chip_prox<ISO>(s.bx, s.bt, gx, gt, alpha, al4, inv4, nx, nv);
     };
     // the samples of an owned row that the neighbouring strips hold as halo; e: the row's place
-    auto give_edge = [&](float *e, const Q4 &nx, const Q4 &nv) {
-      float t[4];
+    auto give_edge = [&](PacketMem *e, const Q4 &nx, const Q4 &nv) {
+      float t[4], x[4];
       un4(nv, t);
-      const float v1 = t[1], v2 = t[2];
-      if (edge_lane) __stcg(e, lane == 30 ? v2 : v1);
-      if (ISO) {
-        un4(nx, t);
-        if (lane == 30) __stcg(e + nr, t[2]);
-      }
+      un4(nx, x);
+      if (edge_lane) put_packet(e, lane == 30 ? t[2] : t[1], x[2], tag);
     };
     // any row: the flux, stored and handed to the CTAs that hold it as halo
     auto prox_row = [&](int r, const Row &s, const Q4 &ph_up, Q4 &nx, Q4 &nv) {
@@ -328,14 +338,8 @@ __device__ __forceinline__ void chip_worker_w(const ChipCta &X) {
       sts4(phi_addr(r), s.ph);
       if (r >= 2 && r < J.h + 2) {
         give_edge(xe + r, nx, nv);
-        if (own_lane && gj0 < ntp) {
-          float *const o = xr + static_cast<size_t>(J.seg) * 3 * ntp + gj0;
-          if (r == J.h) {
-            stg4(o, nx);
-            stg4(o + ntp, nv);
-          }
-          if (r == 3) stg4(o + 2 * ntp, nx);
-        }
+        if (r == J.h) put_row(0, mb, nx, nv, tag);
+        if (r == 3) put_row(1, mb, nx, nv, tag);
       }
     };
     // p, q of a row and its sums that need no other row; ddx: its step (x)
@@ -404,7 +408,8 @@ __device__ __forceinline__ void chip_worker_w(const ChipCta &X) {
     struct At {
       unsigned ph, f;
       uint32_t tb, tn;
-      float *xe, *g;
+      PacketMem *xe;
+      float *g;
     };
     auto plain_step = [&](auto stream, const At &a, int off, const Carry &in, Carry &out) {
       constexpr bool STREAM = decltype(stream)::value;
@@ -548,34 +553,74 @@ __device__ __forceinline__ void chip_worker_w(const ChipCta &X) {
 
     chip_store_sums(X, v, own_lane);
     bar_all_arrive<2, NW>();
-    bar_all<3, NW>();  // every CTA of the group has finished the pass
     // ---- halo flux of the pass
-    if (!sh.bad) {
-      // Lane l fetches side l & 1 of the run's rows ra + l / 2 (+ 16, ...): samples -2 and 121 (t flux),
-      // or sample -2 (x flux), and puts it in its row: an element of the row where that is in
-      // shared or global memory; rows in tensor memory are rewritten by the warp.
-      const int e_strip = J.strip + (lane & 1 ? 1 : -1);
+    bool got = true;
+    if (run > 0) {
+      // rows -2 and h + 1
+      auto halo_row = [&](int seg, int which, Q4 &ux, Q4 &ut) {
+        const PacketMem *const o = xrow + (mb ? xrow_set : 0) + (static_cast<size_t>(seg) * 2 + which) * ntp + gj0;
+        float x[4] = {0.f, 0.f, 0.f, 0.f}, t[4] = {0.f, 0.f, 0.f, 0.f};
+        got = poll_warp([&] {
+          bool all = true;
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            if (!ln.use[i]) continue;
+            const Packet p = get_packet(o + i);
+            x[i] = p.x;
+            t[i] = p.y;
+            all = all && p.tag == tag;
+          }
+          return all;
+        }) && got;
+        ux = q4(x[0], x[1], x[2], x[3]);
+        ut = q4(t[0], t[1], t[2], t[3]);
+      };
+      Q4 hx, ht;
+      if (ra == 0 && J.seg > 0) {
+        halo_row(J.seg - 1, 0, hx, ht);
+        store_flux(0, mn, hx, ht);
+      }
+      if (rb == n && J.seg + 1 < J.segs && J.i0 - 2 + n < nr) {
+        halo_row(J.seg + 1, 1, hx, ht);
+        sts4(bux(mn) + kChipRowBytes, hx);
+      }
+      tmem_stores_done();
+      // Lane l fetches side l & 1 of the run's rows ra + l / 2 (+ 16, ...): the t flux of samples -2
+      // and 121 (and, with the isotropic cost, the x flux of sample -2), and puts it in its row: an
+      // element of the row where that is in shared or global memory; rows in tensor memory are
+      // rewritten by the warp.
+      const int e_side = lane & 1, e_strip = J.strip + (e_side ? 1 : -1);
       const bool e_any = e_strip >= 0 && e_strip < J.strips;
-      const float *const e_src = xcol + (mb ? xcol_set : 0) + (static_cast<size_t>(e_strip) * 3 + (lane & 1 ? 0 : 1)) * nr;
-      auto edges = [&](int comp) {
-        float e[kRounds];
+      const PacketMem *const e_src = xcol + (mb ? xcol_set : 0) + (static_cast<size_t>(e_strip) * 2 + (e_side ? 0 : 1)) * nr;
+      float et[kRounds], ex[kRounds];
+      got = poll_warp([&] {
+        bool all = true;
 #pragma unroll
         for (int w = 0; w < kRounds; ++w) {
           const int r = ra + (lane >> 1) + 16 * w, gi = J.i0 - 2 + r;
-          e[w] = r < rb && e_any && gi >= 0 && gi < nr && !(comp == 0 && (lane & 1)) ? __ldcg(e_src + (comp == 0 ? nr : 0) + gi) : 0.0f;
+          et[w] = ex[w] = 0.0f;
+          if (!(r < rb && e_any && gi >= 0 && gi < nr)) continue;
+          const Packet p = get_packet(e_src + gi);
+          et[w] = p.x;
+          ex[w] = p.y;
+          all = all && p.tag == tag;
         }
+        return all;
+      }) && got;
+      auto edges = [&](int comp, const float (&e)[kRounds]) {
+        const bool mine = comp == 1 || !e_side;
 #pragma unroll
         for (int w = 0; w < kRounds; ++w) {
           const int r = ra + (lane >> 1) + 16 * w, i = r - ra;
-          if (r >= rb || i < kWTmemRows || (comp == 0 && (lane & 1))) continue;
-          const unsigned o = lane & 1 ? 125u : 2u;  // the sample's place in the row
+          if (r >= rb || i < kWTmemRows || !mine) continue;
+          const unsigned o = e_side ? 125u : 2u;  // the sample's place in the row
           if (!TALL || i < u_end)
             sts1(u_slot(i, mn) - 16u * lane + comp * kChipRowBytes + 4u * o, e[w]);
           else
             __stcg(tall - 4 * lane + (2 * mn + comp) * tall_plane + r * 128 + o, e[w]);
         }
         // (lane 0 holds row ra: its x flux also lies in the boundary row)
-        if (comp == 0 && lane == 0 && run > 0) sts1(bux(mn) + 8u, e[0]);
+        if (comp == 0 && lane == 0) sts1(bux(mn) + 8u, e[0]);
         Q4 u[kWTmemRows];
         const uint32_t a = tn + 4 * comp;
 #pragma unroll
@@ -590,24 +635,11 @@ __device__ __forceinline__ void chip_worker_w(const ChipCta &X) {
           tmem_store_quad(a + i * kWRowCols, q4(t[0], lane == 31 && comp ? e1 : t[1], lane == 0 ? e0 : t[2], t[3]));
         }
       };
-      auto halo_row = [&](const float *o) {
-        float t[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) t[q] = ln.use[q] ? __ldcg(o + gj0 + q) : 0.0f;
-        return q4(t[0], t[1], t[2], t[3]);
-      };
-      if (run > 0 && ra == 0 && J.seg > 0) {  // row -2
-        const float *o = xr + static_cast<size_t>(J.seg - 1) * 3 * ntp;
-        store_flux(0, mn, halo_row(o), halo_row(o + ntp));
-      }
+      edges(1, et);
+      if (ISO) edges(0, ex);
       tmem_stores_done();
-      edges(1);
-      if (ISO) edges(0);
-      tmem_stores_done();
-
-      if (run > 0 && rb == n && J.seg + 1 < J.segs && J.i0 - 2 + n < nr)  // row h + 1
-        sts4(bux(mn) + kChipRowBytes, halo_row(xr + static_cast<size_t>(J.seg + 1) * 3 * ntp + 2 * ntp));
     }
+    if (!got && lane == 0) sh.bad = 1;
     bar_all<4, NW>();  // the decision
     ++k;
   }
@@ -647,7 +679,6 @@ __device__ __forceinline__ void chip_worker_w(const ChipCta &X) {
     }
     chip_store_gap(X, t);
     bar_all_arrive<2, NW>();
-    bar_all<3, NW>();
   }
 }
 
