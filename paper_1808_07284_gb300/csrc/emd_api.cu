@@ -694,9 +694,28 @@ void fill_result(emd_result &r, const State &st, const Shot &S, const emd_params
   r.tile = tile;
 }
 
-// The on-chip solve of B gathers laid out by `plan`.  A gather whose iterates turn non-finite or
-// whose linesearch fails is handed to the streaming passes, which define what such a solve
-// leaves in phi and m.  *launched = false when the device cannot hold the launch (nothing done).
+// Solves a gather that an on-chip solve gave up (its iterates turned non-finite or its linesearch
+// failed) again by the streaming passes, which define what such a solve leaves in phi and m.
+emd_status solve_again(int b, const float *const *f_obs, const float *const *f_pred, const int *nt, const int *nr,
+                       const double *dt, const double *dx, const emd_params &p, const Shot &S, float *const *phi,
+                       float *const *m, emd_result *results, void *ws, size_t ws_bytes, cudaStream_t stream,
+                       const SolveExtra &x) {
+  emd_params q = p;
+  if (p.trace) q.trace = p.trace + static_cast<size_t>(b) * p.max_iter * 4;
+  q.phi_init = S.phi_init;
+  q.m_init = S.m_init;
+  SolveExtra again;
+  again.no_chip = true;
+  again.no_tune = true;
+  again.no_graph = x.no_graph;
+  const int before = results[b].launches;
+  const emd_status s = solve_impl(1, f_obs + b, f_pred + b, nt + b, nr + b, dt + b, dx + b, &q, phi + b, m + b,
+                                  results + b, ws, ws_bytes, stream, again);
+  results[b].launches += before;
+  return s;
+}
+
+// The on-chip solve of B gathers laid out by `plan`.  *launched = false when the device cannot hold the launch (nothing done).
 emd_status solve_on_chip(int B, const float *const *f_obs, const float *const *f_pred, const int *nt,
                          const int *nr, const double *dt, const double *dx, const emd_params &p,
                          float *const *phi, float *const *m, emd_result *results, void *ws,
@@ -777,17 +796,8 @@ emd_status solve_on_chip(int B, const float *const *f_obs, const float *const *f
   for (int b = 0; b < B; ++b) {
     fill_result(results[b], hs[b], shots[b], p, static_cast<int>(plan.waves.size()), 0);
     if (hs[b].status != EMD_OK) {
-      emd_params q = p;
-      if (p.trace) q.trace = p.trace + static_cast<size_t>(b) * p.max_iter * 4;
-      q.phi_init = shots[b].phi_init;
-      q.m_init = shots[b].m_init;
-      SolveExtra again;
-      again.no_chip = true;
-      again.no_tune = true;
-      again.no_graph = x.no_graph;
-      const emd_status s = solve_impl(1, f_obs + b, f_pred + b, nt + b, nr + b, dt + b, dx + b, &q, phi + b,
-                                      m + b, results + b, ws, ws_bytes, stream, again);
-      results[b].launches += static_cast<int>(plan.waves.size());
+      const emd_status s = solve_again(b, f_obs, f_pred, nt, nr, dt, dx, p, shots[b], phi, m, results, ws, ws_bytes,
+                                       stream, x);
       if (first == EMD_OK && s != EMD_OK) first = s;
     }
   }
@@ -864,7 +874,10 @@ emd_status solve_impl(int B, const float *const *f_obs, const float *const *f_pr
   long long max_cells = 0;
   for (int b = 0; b < B; ++b) max_cells = std::max(max_cells, static_cast<long long>(nt[b]) * nr[b]);
   // Small gathers: one CTA per gather keeps the whole solve in shared memory.
-  const bool resident = p.launch_mode == 0 && p.tile == 0 && max_cells <= emd::kResidentMaxCells;
+  int max_quads = 0;  // quads of four samples of the largest gather, rows padded
+  for (int b = 0; b < B; ++b) max_quads = std::max(max_quads, max_cells <= emd::kResidentMaxCells ? emd::resident_quads(nt[b], nr[b]) : 0);
+  const bool resident = p.launch_mode == 0 && p.tile == 0 && !x.no_chip && max_cells <= emd::kResidentMaxCells &&
+                        4 * max_quads <= emd::kResidentMaxPadded;
   // Gathers whose state fits on the chip are solved there; the others of the batch stream.
   if (p.tile == 0 && p.launch_mode == 0 && !resident && !x.no_chip) {
     std::vector<int> on;
@@ -935,6 +948,7 @@ emd_status solve_impl(int B, const float *const *f_obs, const float *const *f_pr
   ctl.march_nrun = static_cast<int>(march_run.size());
   ctl.n_done = n_done;
   ctl.error = err_flag;
+  ctl.redo_failed = resident;
 
   const size_t smem = smem_bytes(sh);
   if (sh.iter_tma)
@@ -965,10 +979,11 @@ emd_status solve_impl(int B, const float *const *f_obs, const float *const *f_pr
 
   int n_launch = x.ready ? B : 1;  // k_prepare
   if (resident) {
-    const size_t rsmem = emd::resident_smem_bytes(max_cells);
+    const size_t rsmem = emd::resident_smem_bytes(max_quads);
+    const int rwarps = std::min(emd::kResWarps, (max_quads + 31) / 32) + 1;
     EMD_CK(cudaFuncSetAttribute(emd::k_solve_resident, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 static_cast<int>(rsmem)));
-    emd::k_solve_resident<<<B, emd::kResThreads, rsmem, stream>>>(ctl);
+    emd::k_solve_resident<<<B, rwarps * 32, rsmem, stream>>>(ctl);
     EMD_CK(cudaGetLastError());
     n_launch += 1;
   }
@@ -1106,7 +1121,10 @@ emd_status solve_impl(int B, const float *const *f_obs, const float *const *f_pr
   for (int b = 0; b < B; ++b) {
     const State &st = hs[b];
     fill_result(results[b], st, shots[b], p, n_launch, resident ? 0 : si + 1);
-    if (first == EMD_OK && st.status != EMD_OK) first = static_cast<emd_status>(st.status);
+    emd_status s = static_cast<emd_status>(st.status);
+    if (resident && s != EMD_OK)
+      s = solve_again(b, f_obs, f_pred, nt, nr, dt, dx, p, shots[b], phi, m, results, ws, ws_bytes, stream, x);
+    if (first == EMD_OK && s != EMD_OK) first = s;
   }
   return first;
 }

@@ -82,6 +82,8 @@ struct Ctl {
   double eps, xi, zeta, delta, tol, alpha0;
   int max_iter, check_every, ls_max_trials, linesearch, balance, debug_fault;
   int iso;                          // 1: isotropic ground cost ||u||_{1,2}; 0: ||u||_{1,1}
+  int redo_failed;                  // the finalize pass leaves failed gathers' outputs alone: the host
+                                    // solves those again, from a warm start that may lie in them
   const Shot *shots;
   State *states;
   double *acc;                      // [gather][kAccBufs][kSpread][kAcc] FP64 accumulators (zeroed)
@@ -656,6 +658,7 @@ __global__ void __launch_bounds__(kThreads) k_pass(Ctl c) {
   const int4 h0 = __ldcg(reinterpret_cast<const int4 *>(st));
   const int4 h1 = __ldcg(reinterpret_cast<const int4 *>(st) + 1);
   if (!FINAL && h0.y) return;  // this gather has stopped
+  if (FINAL && c.redo_failed && st->status != ST_OK) return;
   const int k = h0.x;
   const float alpha = __int_as_float(h0.z), coef = __int_as_float(h0.w);
   const float theta = __int_as_float(h1.x), inv = __int_as_float(h1.y);

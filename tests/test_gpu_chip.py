@@ -153,3 +153,44 @@ def test_a_wait_that_runs_out_is_reported(P):
     _, _, _, info = P.emd(o, p, DT, DX, max_iter=20, check=False, debug_fault=2)
     assert info["status"] == P.EMD_ERR_TIMEOUT
     check(P.emd(o, p, DT, DX, max_iter=20), P.emd(o, p, DT, DX, max_iter=20, tile=TILE))
+
+
+@pytest.mark.parametrize("norm", [1, 2])
+@pytest.mark.parametrize("nr,nt", [(1, 2), (1, 1024), (1, 7168), (2, 2), (3, 5), (2, 3584), (20, 200), (64, 112),
+                                   (7, 1021), (896, 8), (1433, 5), (200, 33)])
+def test_small_gathers_match_the_plain_pass(P, nr, nt, norm):
+    """The one-CTA solve in shared memory (and, where padding its rows to four samples takes too
+    much of it, the on-chip solve): odd rows, single receivers, one quad a row, the largest."""
+    o, p = pair(nr, nt, seed=6)
+    for dt, dx in spacings(nr, nt):
+        kw = dict(norm=norm)
+        got, ref = P.emd(o, p, dt, dx, max_iter=40, **kw), P.emd(o, p, dt, dx, max_iter=40, tile=PLAIN, **kw)
+        assert got[3]["tile"] == 0
+        check(got, ref)
+        kw.update(phi_init=ref[1], m_init=ref[2])
+        check(P.emd(o, p, dt, dx, max_iter=9, **kw), P.emd(o, p, dt, dx, max_iter=9, tile=PLAIN, **kw), "warm")
+
+
+def test_small_gathers_stop_trace_and_fail_alike(P):
+    o, p = pair(16, 250, seed=7)
+    dt, dx = 1.0 / 249, 1.0 / 15
+    tr = [torch.zeros((1, 2000, 4), dtype=torch.float64, device="cuda") for _ in range(2)]
+    got = P.emd(o, p, dt, dx, max_iter=2000, tol=0.3, trace=tr[0])
+    ref = P.emd(o, p, dt, dx, max_iter=2000, tol=0.3, trace=tr[1], tile=PLAIN)
+    assert got[3]["iters"] < 2000
+    check(got, ref)
+    assert torch.equal(tr[0][..., 2], tr[1][..., 2])
+    assert torch.allclose(tr[0], tr[1], rtol=1e-5, atol=0.0)
+    bad = p.clone()
+    bad[3, 17] = float("inf")
+    assert P.emd(o, bad, dt, dx, max_iter=20, check=False)[3]["status"] == P.EMD_ERR_NONFINITE
+    # a failed solve from a warm start in place reports the same, and leaves what the passes leave
+    out = []
+    for tile in (0, PLAIN):
+        phi, m = ref[1].clone(), ref[2].clone()
+        ws = P.new_workspace(P.emd_workspace_size(250, 16), o.device)
+        res = P.emd_dyn_solve(o, p, dt, dx, P.emd_default_params(max_iter=20, debug_fault=1, tile=tile, phi_init=phi,
+                                                                 m_init=m), phi, m, ws, check=False)
+        assert res.status == P.EMD_ERR_LINESEARCH
+        out.append((phi, m))
+    assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
