@@ -46,6 +46,7 @@ constexpr int kChipTJ = 120;                            // owned time samples of
 constexpr int kChipSets = 3;                            // accumulator sets, used in turn
 constexpr int kChipVals = 8;                            // sums of a pass
 constexpr int kChipSpread = 8;                          // copies of each accumulator
+constexpr int kChipWordSets = 2;                        // word sets of the fast exchange, used in turn
 constexpr int kChipWordCopies = 4;                      // copies of the words of the fast exchange
 constexpr int kChipWords = 16;                          // two words of each value
 
@@ -395,7 +396,10 @@ __device__ __forceinline__ double chip_block_total(const ChipShared &sh) {
 // added as the two words 256 A + 1 and 256 B + 1: the low byte of a word counts the CTAs that have
 // added to it, so one poll brings the totals and says whether they are complete, with no barrier
 // between data and counter (1000 cycles) and no second read (700).  The integers add exactly in
-// any order.  sa puts the last pass's total of the value's family (p: P_pp, P_qq; grad p: G_pp,
+// any order.  The words are never cleared: each CTA keeps the totals that it read last from a set,
+// and a total is the difference (modulo 2^64).  Clearing them would need a fence before the next
+// exchange (1000 cycles a pass); as it is, a set is added to again only after every CTA has added
+// to the other one, which it does after its read of this one.  sa puts the last pass's total of the value's family (p: P_pp, P_qq; grad p: G_pp,
 // G_qq) at 2^24, so a value keeps 24 bits down to 2^-46 of it and may grow 2^14 fold; a CTA whose
 // value does not fit adds 2^47 for it, every CTA sees the total beyond 2^46 and all of them take
 // the FP64 exchange for this pass.  v: the total in FP32; a, b: in fixed point.
@@ -418,13 +422,14 @@ __device__ __forceinline__ void chip_fast_add(const Ctl &c, unsigned long long *
     atomicAdd(w + (cta % kChipWordCopies) * kChipWords + 2 * q + (lane >> 3),
               (static_cast<unsigned long long>(lane < 8 ? ia : ib) << 8) + 1u);
 }
-__device__ __forceinline__ bool chip_fast_poll(unsigned long long *words, int set, int cta, int group, int sa,
-                                               FastTotal &o) {
+// x0, y0: the totals last read from this set, replaced by those read now.
+__device__ __forceinline__ bool chip_fast_poll(const unsigned long long *words, int set, int group, int sa,
+                                               unsigned long long &x0, unsigned long long &y0, FastTotal &o) {
   constexpr unsigned FULL = 0xffffffffu;
   const int lane = threadIdx.x & 31, q = lane & 7;
-  unsigned long long *const w = words + set * (kChipWordCopies * kChipWords);
   unsigned long long x = 0, y = 0;
-  const unsigned long long *const src = w + (lane >> 3) * kChipWords + 2 * q;
+  const unsigned long long *const src =
+      words + set * (kChipWordCopies * kChipWords) + (lane >> 3) * kChipWords + 2 * q;
   const bool ok = poll_warp([&] {
     asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];\n" : "=l"(x), "=l"(y) : "l"(src) : "memory");
 #pragma unroll
@@ -432,17 +437,14 @@ __device__ __forceinline__ bool chip_fast_poll(unsigned long long *words, int se
       x += __shfl_xor_sync(FULL, x, d);
       y += __shfl_xor_sync(FULL, y, d);
     }
-    return static_cast<int>(x & 255u) == group && static_cast<int>(y & 255u) == group;
+    return static_cast<int>((x - x0) & 255u) == group && static_cast<int>((y - y0) & 255u) == group;
   });
-  o.a = static_cast<long long>(x) >> 8;
-  o.b = static_cast<long long>(y) >> 8;
+  o.a = static_cast<long long>(x - x0) >> 8;
+  o.b = static_cast<long long>(y - y0) >> 8;
+  x0 = x;
+  y0 = y;
   o.v = fmaf(__ll2float_rn(o.b), 0x1p-46f, __ll2float_rn(o.a)) * __int_as_float((127 - sa) << 23);
   o.fits = __all_sync(FULL, llabs(o.a) < (1ll << 46));
-  if (cta == 0) {  // the set of the exchange before, which every CTA has read; added to again two exchanges on
-    unsigned long long *const z = words + ((set + kChipSets - 1) % kChipSets) * (kChipWordCopies * kChipWords);
-    z[lane] = 0u;
-    z[32 + lane] = 0u;
-  }
   return ok;
 }
 
@@ -687,7 +689,7 @@ __device__ __forceinline__ void chip_decider(const ChipCta &X) {
   const float rdx = S.rdx, rdt = S.rdt;
   double *const acc = acc_of(c, J.gather);
   constexpr int kSlow = kChipSets * kChipSpread * kChipVals;  // doubles of the FP64 exchange, then the words
-  static_assert(kSlow + kChipSets * kChipWordCopies * kChipWords <= kAccBufs * kSpread * kAcc, "a gather's accumulators");
+  static_assert(kSlow + kChipWordSets * kChipWordCopies * kChipWords <= kAccBufs * kSpread * kAcc, "a gather's accumulators");
   unsigned long long *const words = reinterpret_cast<unsigned long long *>(acc + kSlow);
   // the balancing sums: f, f^2, |Pcal| + |Pobs|, Pcal - Pobs
   bar_all<2, NW>();
@@ -733,6 +735,7 @@ __device__ __forceinline__ void chip_decider(const ChipCta &X) {
   const bool quick = c.linesearch && c.debug_fault != 1;
   // fixed-point exponents of the two families for the next fast exchange
   int fset = 0, e_p = 0, e_g = 0;
+  unsigned long long x0 = 0, y0 = 0, x1 = 0, y1 = 0;  // the totals last read from set fset, from the other
   bool scaled = false;
   const double xl = xi_power(c.xi);
   constexpr unsigned FULL = 0xffffffffu;
@@ -753,7 +756,7 @@ __device__ __forceinline__ void chip_decider(const ChipCta &X) {
 #pragma unroll 1
     for (int real = slow ? 2 : 0; real < 2; ++real) {
       if (real) {
-        ok = chip_fast_poll(words, fset, cta, J.group, sa, ft);
+        ok = chip_fast_poll(words, fset, J.group, sa, x0, y0, ft);
         f = ft.v;
       } else {
         f = hi;
@@ -763,7 +766,12 @@ __device__ __forceinline__ void chip_decider(const ChipCta &X) {
                  __shfl_sync(FULL, pr.theta_lf, w & 31), __shfl_sync(FULL, pr.inv_lf, w & 31));
     }
     if (!slow) {
-      fset = (fset + 1) % kChipSets;
+      fset ^= 1;
+      const unsigned long long tx = x0, ty = y0;  // the other set's
+      x0 = x1;
+      y0 = y1;
+      x1 = tx;
+      y1 = ty;
       slow = !ft.fits;
     }
     if (ok && slow) {
@@ -835,7 +843,6 @@ __device__ __forceinline__ void chip_decider(const ChipCta &X) {
       e_p = (__float_as_int(p2) >> 23) - 127;
       e_g = (__float_as_int(g2) >> 23) - 127;
     }
-    fence_acq_rel_gpu();  // orders this pass's reads and zeros before the next pass's sums
   }
   // the last pass's sums (or, when no pass ran, the balancing ones, which nobody reads)
   const double s_p2 = __shfl_sync(0xffffffffu, v, 0), s_u2 = __shfl_sync(0xffffffffu, v, 6),
