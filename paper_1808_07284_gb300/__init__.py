@@ -132,7 +132,7 @@ def _autograd_function():
             ctx.dt, ctx.dx = float(dt), float(dx)
             ctx.balance = params.get("balance", EMD_BAL_MEAN)
             ctx.info = info
-            return torch.tensor(dist, dtype=torch.float32, device=f_pred.device)
+            return torch.full((), dist, dtype=torch.float32, device=f_pred.device)
 
         @staticmethod
         def backward(ctx, grad_out):
@@ -194,13 +194,13 @@ def _lsd_autograd_function():
             v = emd_lsd(f_obs.detach().contiguous(), f_pred.detach().contiguous(), float(dt), float(dx),
                         grad_pred=gp)
             ctx.save_for_backward(gp)
-            return torch.tensor(v, dtype=torch.float32, device=f_pred.device)
+            return torch.full((), v, dtype=torch.float32, device=f_pred.device)
 
         @staticmethod
         def backward(ctx, grad_out):
             (gp,) = ctx.saved_tensors
             g = grad_out.to(torch.float32) * gp
-            return g, -g, None, None
+            return g, -g if ctx.needs_input_grad[1] else None, None, None
 
     return LSDFunction
 

@@ -173,6 +173,19 @@ def _check_grid(t, nr, nt, name, planes=1):
         raise ValueError(f"{name} must hold {planes} x {nr} x {nt} elements, got {t.numel()}")
 
 
+def _grids(ts, nrs, nts, name, planes=1):
+    """The pointers of a list of grids, each checked as by _check_grid."""
+    import torch
+    ptrs = (c_void_p * len(nrs))()
+    for b, (nr, nt) in enumerate(zip(nrs, nts)):
+        t = ts[b]
+        if not (isinstance(t, torch.Tensor) and t.is_cuda and t.dtype == torch.float32 and t.is_contiguous()
+                and t.numel() == planes * nr * nt):
+            _check_grid(t, nr, nt, f"{name}[{b}]", planes)
+        ptrs[b] = t.data_ptr()
+    return ptrs
+
+
 def emd_default_params(**overrides) -> EmdParams:
     p = EmdParams()
     lib().emd_default_params(ctypes.byref(p))
@@ -266,18 +279,12 @@ def emd_dyn_solve_batched(f_obs, f_pred, dts, dxs, params: EmdParams, phis, ms, 
                           stream=None, check: bool = True):
     """B solves through the C ABI; lists of tensors; returns a list of EmdResult."""
     B = len(f_obs)
-    nts, nrs = [int(t.shape[1]) for t in f_obs], [int(t.shape[0]) for t in f_obs]
-    for b in range(B):
-        _check_grid(f_obs[b], nrs[b], nts[b], f"f_obs[{b}]")
-        _check_grid(f_pred[b], nrs[b], nts[b], f"f_pred[{b}]")
-        _check_grid(phis[b], nrs[b], nts[b], f"phi[{b}]")
-        _check_grid(ms[b], nrs[b], nts[b], f"m[{b}]", planes=2)
-    P = c_void_p * B
+    nrs, nts = zip(*[t.shape for t in f_obs]) if B else ((), ())
     res = (EmdResult * B)()
     st = lib().emd_dyn_solve_batched(
-        B, P(*[_ptr(t) for t in f_obs]), P(*[_ptr(t) for t in f_pred]), (c_int * B)(*nts),
+        B, _grids(f_obs, nrs, nts, "f_obs"), _grids(f_pred, nrs, nts, "f_pred"), (c_int * B)(*nts),
         (c_int * B)(*nrs), (c_double * B)(*dts), (c_double * B)(*dxs), ctypes.byref(params),
-        P(*[_ptr(t) for t in phis]), P(*[_ptr(t) for t in ms]), res, _ptr(workspace),
+        _grids(phis, nrs, nts, "phi"), _grids(ms, nrs, nts, "m", planes=2), res, _ptr(workspace),
         workspace.numel(), _stream(stream))
     if check and st != EMD_OK:
         raise EmdError(st, "emd_dyn_solve_batched")

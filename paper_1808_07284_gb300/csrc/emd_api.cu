@@ -149,7 +149,9 @@ bool size_ok(int nt, int nr) {
 // Workspace: [states | shots | accumulators | tile_shot | n_done + scratch] then, per gather, the
 // pitched planes f, u0 (x,t), u1 (x,t), u2 (x,t), phi0, phi1 (36 bytes per cell).
 struct Layout {
-  size_t states, shots, acc, tiles, units, misc, header, total;
+  // sums, gather states and flags are adjacent: one fill clears them all, one copy brings states
+  // and flags back; the gather records and the tile list go to the device in one copy
+  size_t acc, states, misc, shots, tiles, units, header, total;
   std::vector<size_t> gather;  // offset of each gather's planes
   std::vector<size_t> plane;   // bytes of one plane (256-aligned)
   int max_tiles;
@@ -163,13 +165,13 @@ Layout layout(int B, const int *nt, const int *nr) {
     for (const Shape &s : kShapes) mt = std::max(mt, tiles_of(s, nt[b], nr[b]));
     L.max_tiles += mt;
   }
-  L.states = 0;
-  L.shots = align256(sizeof(State) * B);
-  L.acc = L.shots + align256(sizeof(Shot) * B);
-  L.tiles = L.acc + align256(sizeof(double) * emd::kAccBufs * emd::kSpread * emd::kAcc * B);
+  L.acc = 0;
+  L.states = align256(sizeof(double) * emd::kAccBufs * emd::kSpread * emd::kAcc * B);
+  L.misc = L.states + align256(sizeof(State) * B);
+  L.shots = L.misc + 256;
+  L.tiles = L.shots + align256(sizeof(Shot) * B);
   L.units = L.tiles + align256(sizeof(int) * static_cast<size_t>(L.max_tiles));
-  L.misc = L.units + align256(sizeof(int) * static_cast<size_t>(B));  // the march's gather list
-  L.header = L.misc + 256;
+  L.header = L.units + align256(sizeof(int) * static_cast<size_t>(B));  // the march's gather list
   size_t off = L.header;
   for (int b = 0; b < B; ++b) {
     const size_t pl = align256(sizeof(float) * static_cast<size_t>(nr[b]) * ntp_of(nt[b]));
@@ -180,6 +182,29 @@ Layout layout(int B, const int *nt, const int *nr) {
   L.total = off;
   return L;
 }
+
+// Clears the sums, the gather states and the flags (done, error).
+cudaError_t clear_state(const Layout &L, char *base, cudaStream_t stream) {
+  return cudaMemsetAsync(base + L.acc, 0, L.misc + 2 * sizeof(int) - L.acc, stream);
+}
+
+// The gather states and the flags as they are after the work enqueued on `stream`.
+struct Readback {
+  std::vector<char> bytes;
+  State *states = nullptr;
+  int done = 0, error = 0;
+  cudaError_t fetch(const Layout &L, const char *base, cudaStream_t stream) {
+    bytes.resize(L.misc + 2 * sizeof(int) - L.states);
+    cudaError_t e = cudaMemcpyAsync(bytes.data(), base + L.states, bytes.size(), cudaMemcpyDeviceToHost, stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
+    states = reinterpret_cast<State *>(bytes.data());
+    int flags[2];
+    std::memcpy(flags, bytes.data() + (L.misc - L.states), sizeof(flags));
+    done = flags[0];
+    error = flags[1];
+    return e;
+  }
+};
 
 // Units of the marching solve for T marching warps, dealt round-robin (unit u to warp
 // u mod T).  Every running gather is cut into segments of about H receivers (nseg = ceil(nr /
@@ -760,9 +785,7 @@ emd_status solve_on_chip(int B, const float *const *f_obs, const float *const *f
   ctl.n_done = flags;
   ctl.error = flags + 1;
   EMD_CK(cudaMemcpyAsync(base + L.shots, shots.data(), sizeof(Shot) * B, cudaMemcpyHostToDevice, stream));
-  EMD_CK(cudaMemsetAsync(states, 0, sizeof(State) * B, stream));
-  EMD_CK(cudaMemsetAsync(flags, 0, 2 * sizeof(int), stream));
-  EMD_CK(cudaMemsetAsync(ctl.acc, 0, sizeof(double) * emd::kAccBufs * emd::kSpread * emd::kAcc * B, stream));
+  EMD_CK(clear_state(L, base, stream));
   if (x.stage && *x.stage) {
     const std::function<emd_status()> enqueue = std::move(*x.stage);
     *x.stage = nullptr;
@@ -783,19 +806,16 @@ emd_status solve_on_chip(int B, const float *const *f_obs, const float *const *f
                                        dim3(static_cast<unsigned>(wave.size())), dim3(static_cast<unsigned>((emd::chip_workers(plan.form[w]) + 1) * 32)), args,
                                        smem, stream));
   }
-  std::vector<State> hs(B);
-  int h_flags[2] = {0, 0};
-  EMD_CK(cudaMemcpyAsync(hs.data(), states, sizeof(State) * B, cudaMemcpyDeviceToHost, stream));
-  EMD_CK(cudaMemcpyAsync(h_flags, flags, sizeof(h_flags), cudaMemcpyDeviceToHost, stream));
-  EMD_CK(cudaStreamSynchronize(stream));
-  if (h_flags[1]) {  // a bounded device wait gave up
+  Readback back;
+  EMD_CK(back.fetch(L, base, stream));
+  if (back.error) {  // a bounded device wait gave up
     for (int b = 0; b < B; ++b) results[b].status = EMD_ERR_TIMEOUT;
     return EMD_ERR_TIMEOUT;
   }
   emd_status first = EMD_OK;
   for (int b = 0; b < B; ++b) {
-    fill_result(results[b], hs[b], shots[b], p, static_cast<int>(plan.waves.size()), 0);
-    if (hs[b].status != EMD_OK) {
+    fill_result(results[b], back.states[b], shots[b], p, static_cast<int>(plan.waves.size()), 0);
+    if (back.states[b].status != EMD_OK) {
       const emd_status s = solve_again(b, f_obs, f_pred, nt, nr, dt, dx, p, shots[b], phi, m, results, ws, ws_bytes,
                                        stream, x);
       if (first == EMD_OK && s != EMD_OK) first = s;
@@ -908,7 +928,7 @@ emd_status solve_impl(int B, const float *const *f_obs, const float *const *f_pr
     char *g = base + L.gather[b];
     fill_shot(S, f_obs[b], f_pred[b], nt[b], nr[b], dt[b], dx[b], phi[b], m[b],
               x.phi_init ? x.phi_init[b] : p.phi_init, x.m_init ? x.m_init[b] : p.m_init, g, pl);
-    if (uses_tma(sh) && !encode_tmap(S, g, pl, sh.ti + 4)) return EMD_ERR_CUDA;
+    if (uses_tma(sh) && !resident && !encode_tmap(S, g, pl, sh.ti + 4)) return EMD_ERR_CUDA;
     S.tiles_j = (nt[b] + (sh.w - 8) - 1) / (sh.w - 8);
     S.tile0 = static_cast<int>(tile_shot.size());
     S.ntiles = tiles_of(sh, nt[b], nr[b]);
@@ -928,16 +948,16 @@ emd_status solve_impl(int B, const float *const *f_obs, const float *const *f_pr
   int *err_flag = n_done + 1;
   double *acc = reinterpret_cast<double *>(base + L.acc);
 
-  EMD_CK(cudaMemcpyAsync(dshots, shots.data(), sizeof(Shot) * B, cudaMemcpyHostToDevice, stream));
-  EMD_CK(cudaMemcpyAsync(dtiles, tile_shot.data(), sizeof(int) * tile_shot.size(),
-                         cudaMemcpyHostToDevice, stream));
+  {
+    std::vector<char> records(L.tiles - L.shots + sizeof(int) * tile_shot.size());
+    std::memcpy(records.data(), shots.data(), sizeof(Shot) * B);
+    std::memcpy(records.data() + (L.tiles - L.shots), tile_shot.data(), sizeof(int) * tile_shot.size());
+    EMD_CK(cudaMemcpyAsync(dshots, records.data(), records.size(), cudaMemcpyHostToDevice, stream));
+  }
   if (!march_run.empty())
     EMD_CK(cudaMemcpyAsync(dunits, march_run.data(), sizeof(int) * march_run.size(),
                            cudaMemcpyHostToDevice, stream));
-  EMD_CK(cudaMemsetAsync(states, 0, sizeof(State) * B, stream));
-  EMD_CK(cudaMemsetAsync(n_done, 0, 2 * sizeof(int), stream));
-  EMD_CK(cudaMemsetAsync(acc, 0, sizeof(double) * emd::kAccBufs * emd::kSpread * emd::kAcc * B,
-                         stream));
+  EMD_CK(clear_state(L, base, stream));
 
   Ctl ctl = make_ctl(p);
   ctl.shots = dshots;
@@ -1036,15 +1056,12 @@ emd_status solve_impl(int B, const float *const *f_obs, const float *const *f_pr
         k0 = ke;
         if (k0 >= p.max_iter) break;
         // which gathers are still running (and did a bounded wait give up)?
-        std::vector<State> hs(B);
-        int h_flags[2] = {0, 0};
-        EMD_CK(cudaMemcpyAsync(hs.data(), states, sizeof(State) * B, cudaMemcpyDeviceToHost, stream));
-        EMD_CK(cudaMemcpyAsync(h_flags, n_done, sizeof(h_flags), cudaMemcpyDeviceToHost, stream));
-        EMD_CK(cudaStreamSynchronize(stream));
-        if (h_flags[1] || h_flags[0] >= B) break;
+        Readback back;
+        EMD_CK(back.fetch(L, base, stream));
+        if (back.error || back.done >= B) break;
         std::vector<int> running;
         for (int b = 0; b < B; ++b)
-          if (!hs[b].done) running.push_back(b);
+          if (!back.states[b].done) running.push_back(b);
         if (static_cast<int>(running.size()) == dealt) continue;  // none stopped since the last deal
         // some gathers stopped: deal the running ones' work over every CTA again
         run_shots = shots;
@@ -1053,11 +1070,11 @@ emd_status solve_impl(int B, const float *const *f_obs, const float *const *f_pr
           // finished units restart from k0 times the new count (no kernel is running now)
           items = march_layout(run_shots, running, static_cast<long long>(cap) * sh.nw, sh.nw);
           if (items < 0) return EMD_ERR_ARG;
-          for (int b : running) hs[b].tiles_done = static_cast<unsigned>(k0) * static_cast<unsigned>(run_shots[b].nunits);
+          for (int b : running) back.states[b].tiles_done = static_cast<unsigned>(k0) * static_cast<unsigned>(run_shots[b].nunits);
           ctl.march_nrun = static_cast<int>(running.size());
           EMD_CK(cudaMemcpyAsync(dunits, running.data(), sizeof(int) * running.size(),
                                  cudaMemcpyHostToDevice, stream));
-          EMD_CK(cudaMemcpyAsync(states, hs.data(), sizeof(State) * B, cudaMemcpyHostToDevice, stream));
+          EMD_CK(cudaMemcpyAsync(states, back.states, sizeof(State) * B, cudaMemcpyHostToDevice, stream));
         } else {
           std::vector<int> next;
           for (int b : running) {
@@ -1107,19 +1124,16 @@ emd_status solve_impl(int B, const float *const *f_obs, const float *const *f_pr
   EMD_CK(cudaGetLastError());
   n_launch += passes.launched + 1;
 
-  std::vector<State> hs(B);
-  int h_flags[2] = {0, 0};
-  EMD_CK(cudaMemcpyAsync(hs.data(), states, sizeof(State) * B, cudaMemcpyDeviceToHost, stream));
-  EMD_CK(cudaMemcpyAsync(h_flags, n_done, sizeof(h_flags), cudaMemcpyDeviceToHost, stream));
-  EMD_CK(cudaStreamSynchronize(stream));
-  if (h_flags[1]) {  // a bounded device wait gave up
+  Readback back;
+  EMD_CK(back.fetch(L, base, stream));
+  if (back.error) {  // a bounded device wait gave up
     for (int b = 0; b < B; ++b) results[b].status = EMD_ERR_TIMEOUT;
     return EMD_ERR_TIMEOUT;
   }
 
   emd_status first = EMD_OK;
   for (int b = 0; b < B; ++b) {
-    const State &st = hs[b];
+    const State &st = back.states[b];
     fill_result(results[b], st, shots[b], p, n_launch, resident ? 0 : si + 1);
     emd_status s = static_cast<emd_status>(st.status);
     if (resident && s != EMD_OK)
