@@ -411,11 +411,11 @@ struct ChipPlan {
 };
 
 // Estimated us per pass of a wave whose tallest CTA stages n rows: the pass boundary and the rows.
-// Measured: 4.2 us at 16 rows, 6.1 at 70 and 7.5 at 123 in the tile pass's form; 9.5 at 123 in the
-// marching pass's; 19.7 at 217 and 24.7 at 327 in tall CTAs.
+// Measured: 2.8 us at 16 rows and 5.4 at 70 in the tile pass's form; 8.25 at 123 in the marching
+// pass's; 16.7 at 217 and 23.2 at 327 in tall CTAs.
 double chip_pass_us(int n, bool march) {
-  if (n > emd::kChipMaxRows) return 8.8 + 0.049 * n;
-  return march ? 3.5 + 0.05 * n : 3.6 + 0.033 * n;
+  if (n > emd::kChipMaxRows) return 3.9 + 0.059 * n;
+  return march ? 2.4 + 0.048 * n : 2.0 + 0.049 * n;
 }
 
 // Estimated us per pass of the streaming solves (tile and marching pass) over `cells` cells:

@@ -47,9 +47,10 @@ static_assert(2 * ((kChipMaxRows + kChipWorkers - 1) / kChipWorkers) + 4 <= WLay
               "a run of 9 rows has no streamed values");
 
 // The exchange buffers (packets: ux, ut of the last-but-one owned row; ux of the second one; ut of the
-// second owned sample and ut, ux of the last-but-one) are followed, for tall CTAs, by [cta][5][rows]
+// second owned sample and ut, ux of the last-but-one) are followed, for tall CTAs, by [cta][rows][5]
 // [128] streamed values.
-__host__ __device__ inline size_t chip_w_tall_floats(int rows) { return static_cast<size_t>(rows) * 5 * 128; }
+constexpr int kTallRow = 5 * 128;
+__host__ __device__ inline size_t chip_w_tall_floats(int rows) { return static_cast<size_t>(rows) * kTallRow; }
 
 __device__ __forceinline__ Q4 ldg4(const float *p) {
   const float4 t = __ldcg(reinterpret_cast<const float4 *>(p));
@@ -139,17 +140,12 @@ __device__ __forceinline__ void chip_worker_w(const ChipCta &X) {
   // ---- where the rows of this run live
   const unsigned slots = X.smem + static_cast<unsigned>(warp) * (kWSlots * kChipRowBytes);
   const unsigned a_ph = slots;               // phi of row ra
-  int u_end = 1 << 30, f_lo = 0;             // rows of the run from u_end on / before f_lo stream
-  unsigned a_u, a_f;                         // flux, f of row ra (if those were in slots)
-  float *tall = nullptr;                     // streamed planes ux0, ut0, ux1, ut1, f: row r at + 128 r
-  size_t tall_plane = 0;
+  int nf = 1 << 30;                          // rows of the run from nf on have their f streamed
+  unsigned a_u = 0, a_f;                     // flux, f of row ra (if those were in slots)
+  float *tall = nullptr;                     // streamed values ux0, ut0, ux1, ut1, f: row r at + kTallRow r
   if (TALL) {
-    const int nu = min(max(0, run - kWTmemRows), (kWSlots - run) / 4), nf = min(run, kWSlots - run - 4 * nu);
-    u_end = kWTmemRows + nu;
-    f_lo = run - nf;
-    a_u = slots + static_cast<unsigned>(run - 4 * kWTmemRows) * kChipRowBytes;
-    a_f = slots + static_cast<unsigned>(run + 4 * nu - f_lo) * kChipRowBytes;
-    tall_plane = static_cast<size_t>(J.rows) * 128;
+    nf = min(run, kWSlots - run);
+    a_f = slots + static_cast<unsigned>(run) * kChipRowBytes;
     tall = S.f + chip_exchange_bytes(J.segs, J.strips, nr, ntp) / 4 + X.cta * chip_w_tall_floats(J.rows) + 4 * lane;
   } else {
     constexpr unsigned kRun = (kChipMaxRows + kChipWorkers - 1) / kChipWorkers;
@@ -161,36 +157,36 @@ __device__ __forceinline__ void chip_worker_w(const ChipCta &X) {
     const int i = r - ra;
     if (i < kWTmemRows) {
       tmem_load_flux(X.taddr + i * kWRowCols + 8 * m, ux, ut);
-    } else if (!TALL || i < u_end) {
+    } else if (!TALL) {
       ux = lds4(u_slot(i, m));
       ut = lds4<kChipRowBytes>(u_slot(i, m));
     } else {
-      ux = ldg4(tall + 2 * m * tall_plane + r * 128);
-      ut = ldg4(tall + (2 * m + 1) * tall_plane + r * 128);
+      ux = ldg4(tall + r * kTallRow + 256 * m);
+      ut = ldg4(tall + r * kTallRow + 256 * m + 128);
     }
   };
   auto store_flux = [&](int r, int m, const Q4 &ux, const Q4 &ut) {
     const int i = r - ra;
     if (i < kWTmemRows) {
       tmem_store_flux(X.taddr + i * kWRowCols + 8 * m, ux, ut);
-    } else if (!TALL || i < u_end) {
+    } else if (!TALL) {
       sts4(u_slot(i, m), ux);
       sts4<kChipRowBytes>(u_slot(i, m), ut);
     } else {
-      stg4(tall + 2 * m * tall_plane + r * 128, ux);
-      stg4(tall + (2 * m + 1) * tall_plane + r * 128, ut);
+      stg4(tall + r * kTallRow + 256 * m, ux);
+      stg4(tall + r * kTallRow + 256 * m + 128, ut);
     }
   };
   auto phi_addr = [&](int r) { return a_ph + static_cast<unsigned>(r - ra) * kChipRowBytes; };
   auto load_f = [&](int r) {
-    return !TALL || r - ra >= f_lo ? lds4(a_f + static_cast<unsigned>(r - ra) * kChipRowBytes)
-                                   : ldg4(tall + 4 * tall_plane + r * 128);
+    return !TALL || r - ra < nf ? lds4(a_f + static_cast<unsigned>(r - ra) * kChipRowBytes)
+                                : ldg4(tall + r * kTallRow + 512);
   };
   auto store_f = [&](int r, const Q4 &v) {
-    if (!TALL || r - ra >= f_lo)
+    if (!TALL || r - ra < nf)
       sts4(a_f + static_cast<unsigned>(r - ra) * kChipRowBytes, v);
     else
-      stg4(tall + 4 * tall_plane + r * 128, v);
+      stg4(tall + r * kTallRow + 512, v);
   };
   const unsigned brow = X.smem + kWBound + static_cast<unsigned>(warp) * kChipRowBytes;  // this run's boundary row
   auto bux = [&](int m) { return brow + kWBUx + static_cast<unsigned>(m) * kWBUxSlot; };
@@ -402,49 +398,57 @@ __device__ __forceinline__ void chip_worker_w(const ChipCta &X) {
         sts4<kWBQ>(brow, out.q_dn);
       }
     };
-    // Plain rows: r + 1 owned, not the gather's first receiver, held by no other segment, r + 2 not
-    // the run's last row, no residual sums.  The addresses of row r run along; STREAM: the flux of
-    // rows r - 1 to r + 1 is in global memory, else that of rows r and r + 1 in tensor memory.
+    // Plain rows: r + 1 owned, not the gather's first receiver, held by no other segment, no residual
+    // sums.  The addresses of row r run along, i = r - ra.  STREAM: the values of rows r - 1 to r + 1
+    // stream; else each is looked for where it lies.
     struct At {
       unsigned ph, f;
       uint32_t tb, tn;
       PacketMem *xe;
-      float *g;
+      const float *gb, *gf;  // streamed u^k, f
+      float *gn;             // streamed u^{k-1}, then u^{k+1}
+      int i;
     };
     auto plain_step = [&](auto stream, const At &a, int off, const Carry &in, Carry &out) {
       constexpr bool STREAM = decltype(stream)::value;
-      const int o = -off;  // row r - off
+      const int o = -off, i = a.i - off;  // row r - off
       Pre p;
-      if (STREAM) {
-        const float *const g = a.g + (o - 1) * 128;
-        out.pre.bx = ldg4(g + 2 * mb * tall_plane);
-        out.pre.bt = ldg4(g + (2 * mb + 1) * tall_plane);
-        out.pre.ax = ldg4(g + 2 * mn * tall_plane);
-        out.pre.at = ldg4(g + (2 * mn + 1) * tall_plane);
-        out.pre.f = ldg4(g + 4 * tall_plane);
+      if (TALL) {  // the row above, where it lies
+        if (!STREAM && i <= kWTmemRows) {
+          tmem_load_flux2(a.tb + (o - 1) * kWRowCols, a.tn + (o - 1) * kWRowCols, out.pre.bx, out.pre.bt, out.pre.ax,
+                          out.pre.at);
+        } else {
+          out.pre.bx = ldg4(a.gb + (o - 1) * kTallRow);
+          out.pre.bt = ldg4(a.gb + (o - 1) * kTallRow + 128);
+          out.pre.ax = ldg4(a.gn + (o - 1) * kTallRow);
+          out.pre.at = ldg4(a.gn + (o - 1) * kTallRow + 128);
+        }
+        out.pre.f = !STREAM && i <= nf ? lds4(a.f + (o - 1) * static_cast<int>(kChipRowBytes)) : ldg4(a.gf + (o - 1) * kTallRow);
       } else {
-        Pre &d = TALL ? out.pre : p;
-        constexpr int back = TALL ? 1 : 0;
-        tmem_load_flux2(a.tb + (o - back) * kWRowCols, a.tn + (o - back) * kWRowCols, d.bx, d.bt, d.ax, d.at);
-        d.f = TALL ? ldg4(a.g + (o - 1) * 128 + 4 * tall_plane) : lds4(a.f + o * static_cast<int>(kChipRowBytes));
+        tmem_load_flux2(a.tb + o * kWRowCols, a.tn + o * kWRowCols, p.bx, p.bt, p.ax, p.at);
+        p.f = lds4(a.f + o * static_cast<int>(kChipRowBytes));
       }
       const unsigned ph = a.ph + o * static_cast<int>(kChipRowBytes);
       dual(ph, TALL ? in.pre : p, in.cur.wx, out.cur);
       Q4 nv;
       prox(in.cur, out.cur.ph, rdx4, out.nx_dn, nv);
-      if (STREAM) {
-        float *const g = a.g + (o + 1) * 128;
-        stg4(g + 2 * mn * tall_plane, out.nx_dn);
-        stg4(g + (2 * mn + 1) * tall_plane, nv);
-      } else {
+      if (!TALL || (!STREAM && i + 1 < kWTmemRows)) {
         tmem_store_flux(a.tn + (o + 1) * kWRowCols, out.nx_dn, nv);
+      } else {
+        stg4(a.gn + (o + 1) * kTallRow, out.nx_dn);
+        stg4(a.gn + (o + 1) * kTallRow + 128, nv);
       }
       sts4<kChipRowBytes>(ph, in.cur.ph);
       give_edge(a.xe + o + 1, out.nx_dn, nv);
       flux_row(plain, 0, out.nx_dn, nv, in.cur.bx, in.cur.bt,
                TALL ? in.cur.f : lds4<kChipRowBytes>(a.f + o * static_cast<int>(kChipRowBytes)), in.nx_dn, in.ddx_dn,
                out.p_dn, out.q_dn, out.ddx_dn);
-      grad_row(plain, 0, in.p_dn, in.q_dn, out.p_dn, out.q_dn);
+      if (ISO || i + 2 < run - 1) {
+        grad_row(plain, 0, in.p_dn, in.q_dn, out.p_dn, out.q_dn);
+      } else {
+        sts4<kWBP>(brow, out.p_dn);
+        sts4<kWBQ>(brow, out.q_dn);
+      }
     };
     Carry x, y;
     x.p_dn = x.q_dn = x.nx_dn = x.ddx_dn = q4s(0.0f);
@@ -464,49 +468,38 @@ __device__ __forceinline__ void chip_worker_w(const ChipCta &X) {
         prox_row(rb - 1, s, x.cur.ph, x.nx_dn, nv);
         x.ddx_dn = sub4(x.nx_dn, s.bx);
       }
-      // rows [lo, hi] are plain as the upper row of a step
-      const int lo = max(3, ra + (TALL ? 1 : 0)), hi = need_res ? -1 : min(J.h - 2, rb - 4);
+      // rows [lo, hi] are plain as the upper row of a step; they go two per trip
+      const int lo = max(3, ra + (TALL ? 1 : 0)), hi = need_res ? -1 : ISO ? min(J.h - 2, rb - 4) : J.h - 2;
       int r = rb - 3;
 #pragma unroll 1
       while (r >= ra) {
-        // a stretch of plain row pairs [r - 2 m + 1, r] in one place
-        int m = 0;
-        bool stream = false;
-        if (r <= hi) {
-          const int i = r - ra;
-          if (TALL && i - 2 >= u_end && i < f_lo) {
-            stream = true;
-            m = (min(r - lo + 1, i - 1 - u_end + 1)) / 2;
-          } else if (i + 1 < kWTmemRows && (!TALL || f_lo >= kWTmemRows)) {
-            m = (r - lo + 1) / 2;
-          }
-        }
-        if (m <= 0) {
+        if (r > hi || r <= lo) {
           step(r, x, y);
           x = y;
           --r;
           continue;
         }
+        const int off = r * kTallRow;
         At a{phi_addr(r), a_f + static_cast<unsigned>(r - ra) * kChipRowBytes, tb + (r - ra) * kWRowCols,
-             tn + (r - ra) * kWRowCols, xe + r, tall + r * 128};
-        r -= 2 * m;
-        auto stretch = [&](auto where) {
+             tn + (r - ra) * kWRowCols, xe + r, tall + off + 256 * mb, tall + off + 512, tall + off + 256 * mn, r - ra};
+        auto stretch = [&](auto stream, int end) {
 #pragma unroll 1
-          for (; m > 0; --m) {
-            plain_step(where, a, 0, x, y);
-            plain_step(where, a, 1, y, x);
+          for (; r > end; r -= 2) {
+            plain_step(stream, a, 0, x, y);
+            plain_step(stream, a, 1, y, x);
             a.ph -= 2 * kChipRowBytes;
             a.f -= 2 * kChipRowBytes;
             a.tb -= 2 * kWRowCols;
             a.tn -= 2 * kWRowCols;
             a.xe -= 2;
-            a.g -= 256;
+            a.gb -= 2 * kTallRow;
+            a.gf -= 2 * kTallRow;
+            a.gn -= 2 * kTallRow;
+            a.i -= 2;
           }
         };
-        if (TALL && stream)
-          stretch(BoolConst<TALL>{});
-        else
-          stretch(BoolConst<false>{});
+        if (TALL) stretch(BoolConst<TALL>{}, max(lo, ra + 1 + max(kWTmemRows, nf)));
+        stretch(BoolConst<false>{}, lo);
       }
     }
     // ---- the first row of the run: phi^k of the row above comes from the run before
@@ -614,10 +607,10 @@ __device__ __forceinline__ void chip_worker_w(const ChipCta &X) {
           const int r = ra + (lane >> 1) + 16 * w, i = r - ra;
           if (r >= rb || i < kWTmemRows || !mine) continue;
           const unsigned o = e_side ? 125u : 2u;  // the sample's place in the row
-          if (!TALL || i < u_end)
+          if (!TALL)
             sts1(u_slot(i, mn) - 16u * lane + comp * kChipRowBytes + 4u * o, e[w]);
           else
-            __stcg(tall - 4 * lane + (2 * mn + comp) * tall_plane + r * 128 + o, e[w]);
+            __stcg(tall - 4 * lane + r * kTallRow + (2 * mn + comp) * 128 + o, e[w]);
         }
         // (lane 0 holds row ra: its x flux also lies in the boundary row)
         if (comp == 0 && lane == 0) sts1(bux(mn) + 8u, e[0]);
