@@ -219,7 +219,7 @@ __device__ __forceinline__ void chip_worker_w(const ChipCta &X) {
   // ---- inputs, warm start and the balancing sums
   {
     BalanceSums sums;
-    for (int r = ra; r < rb; ++r) {
+    chip_input_rows(X, ln, [&](int r, const float (&po)[4], const float (&pp)[4]) {
       const int gi = J.i0 - 2 + r;
       const bool rin = gi >= 0 && gi < nr, rown = r >= 2 && r < J.h + 2;
       float f[4], ph[4], ux[4], ut[4];
@@ -228,12 +228,11 @@ __device__ __forceinline__ void chip_worker_w(const ChipCta &X) {
         const int gj = gj0 + q;
         const bool in = rin && ln.use[q];
         const size_t g = static_cast<size_t>(gi) * X.nt + gj;
-        const float po = in ? S.p_obs[g] : 0.0f, pp = in ? S.p_pred[g] : 0.0f;
-        f[q] = pp - po;
+        f[q] = pp[q] - po[q];
         ph[q] = in && S.phi_init ? S.phi_init[g] : 0.0f;
         ux[q] = in && S.m_init ? chip_init_flux(X, 0, gi, gj) : 0.0f;
         ut[q] = (in || (lane == 31 && q == 1)) && S.m_init ? chip_init_flux(X, 1, gi, gj) : 0.0f;
-        if (in && rown && own_lane) sums.add(po, pp);
+        if (in && rown && own_lane) sums.add(po[q], pp[q]);
       }
       const Q4 ux4 = q4(ux[0], ux[1], ux[2], ux[3]), ut4 = q4(ut[0], ut[1], ut[2], ut[3]);
 #pragma unroll
@@ -243,7 +242,7 @@ __device__ __forceinline__ void chip_worker_w(const ChipCta &X) {
       }
       sts4(phi_addr(r), q4(ph[0], ph[1], ph[2], ph[3]));
       store_f(r, q4(f[0], f[1], f[2], f[3]));
-    }
+    });
     if (run > 0 && rb == n) {  // the row below the last one: its x flux
       float ux[4];
 #pragma unroll
@@ -646,13 +645,24 @@ __device__ __forceinline__ void chip_worker_w(const ChipCta &X) {
     Sum2 t[4];
     if (run > 0) {
       Q4 b_dn = lds4(bux(mb) + kChipRowBytes), a_dn = lds4(bux(ma) + kChipRowBytes);
+      Q4 bx, bt, ax, at, f, bx1, bt1, ax1, at1, f1;  // of this row and of the next
+      auto load = [&](int r) {
+        load_flux(r, mb, bx1, bt1);
+        load_flux(r, ma, ax1, at1);
+        f1 = load_f(r);
+      };
+      load(rb - 1);
+#pragma unroll 1
       for (int r = rb - 1; r >= ra; --r) {
-        Q4 bx, bt, ax, at;
-        load_flux(r, mb, bx, bt);
-        load_flux(r, ma, ax, at);
+        bx = bx1;
+        bt = bt1;
+        ax = ax1;
+        at = at1;
+        f = f1;
+        if (r > ra) load(r - 1);
         const Q4 db = div4(sub4(b_dn, bx), diff_right(bt), rdx4, rdt4);
         const Q4 da = div4(sub4(a_dn, ax), diff_right(at), rdx4, rdt4);
-        const Q4 ph = fma4(cf, fma4(th, sub4(db, da), add4(db, load_f(r))), lds4(phi_addr(r)));
+        const Q4 ph = fma4(cf, fma4(th, sub4(db, da), add4(db, f)), lds4(phi_addr(r)));
         sts4(phi_addr(r), ph);
         if (r == rb - 1) sts4(brow, ph);
         b_dn = bx;
@@ -662,12 +672,23 @@ __device__ __forceinline__ void chip_worker_w(const ChipCta &X) {
     bar_workers<NW>();
     const bool vec = chip_vec_out(X);
     Q4 up = run > 0 && ra > 0 ? lds4(brow - kChipRowBytes) : q4s(0.0f);
+    Q4 ux, ut, f, ux1, ut1, f1;
+    if (run > 0) {
+      load_flux(ra, mb, ux1, ut1);
+      f1 = load_f(ra);
+    }
+#pragma unroll 1
     for (int r = ra; r < rb; ++r) {
-      Q4 ux, ut;
-      load_flux(r, mb, ux, ut);
+      ux = ux1;
+      ut = ut1;
+      f = f1;
+      if (r + 1 < rb) {
+        load_flux(r + 1, mb, ux1, ut1);
+        f1 = load_f(r + 1);
+      }
       const Q4 ph = lds4(phi_addr(r)), gtv = diff_left(ph);
       if (r >= 2 && r < J.h + 2 && own_lane)
-        chip_output_row<ISO>(X, vec, J.i0 - 2 + r, ux, ut, ph, up, gtv, load_f(r), t);
+        chip_output_row<ISO>(X, vec, J.i0 - 2 + r, ux, ut, ph, up, gtv, f, t);
       up = ph;
     }
     chip_store_gap(X, t);
