@@ -91,11 +91,14 @@ typedef struct {
   const float *phi_init; /* optional warm start for phi, device [nr][nt]; NULL = zeros   */
   const float *m_init;   /* optional warm start for u, device [2][nr][nt]; NULL = zeros  */
   int tile;          /* stencil tile-shape id (emd_tile_count() of them); 0 = automatic:
-                        gathers of <= 7168 cells are solved in shared memory (one CTA
-                        each, launch_mode 0), thin ones (<= 8 receivers) by the plain
-                        pass, the rest by the TMA pass in the tile shape an autotuner
-                        picks on the first solve of each (device, sizes) configuration
-                        (a few short timed trial solves, then cached per process)       */
+                        with launch_mode 0, gathers of <= 7168 cells are solved in shared
+                        memory (one CTA each) and gathers whose state fits in the shared and
+                        tensor memory of the SMs are solved there (one cooperative launch
+                        per wave of gathers); of the rest, thin ones (<= 8 receivers)
+                        are solved by the plain pass, others by the TMA or marching pass
+                        in the shape an autotuner picks on the first solve of each
+                        (device, sizes) configuration (a few short timed trial solves,
+                        then cached per process)                                        */
   int launch_mode;   /* 0: automatic -- every pass in one persistent cooperative launch when
                         the TMA pass serves the gathers, else graph replays of the pass;
                         1: one plain launch per pass; 2: one launch per pass, replayed
@@ -132,7 +135,8 @@ typedef struct {
   int status;         /* emd_status of this solve                                        */
   int launches;       /* kernel launches this solve made (a graph's nodes count one each) */
   int tile;           /* tile-shape id the solve ran (1..emd_tile_count(); the autotuner's
-                         choice when params->tile was 0); 0 for the shared-memory solve     */
+                         choice when params->tile was 0); 0 for the shared-memory and the
+                         on-chip solve                                                     */
 } emd_result;
 
 /* Fills *p with the defaults listed above.  p must not be NULL. */
@@ -184,10 +188,11 @@ size_t emd_batched_workspace_size(int B, const int *nt, const int *nr);
 /*
  * B independent solves (the paper solves one EMD per shot), each gather with its own
  * linesearch state; gathers that meet tol stop while the rest go on.  How the passes are
- * launched follows params->launch_mode as for emd_dyn_solve: by default (0) one persistent
- * cooperative launch runs every PDHG iteration of every gather (gathers of at most 7168
- * cells each get one shared-memory-resident CTA instead); 1 issues one launch per
- * iteration over all gathers, 2 replays those launches from a captured CUDA graph.  All arrays of pointers and sizes are HOST
+ * launched follows params->launch_mode as for emd_dyn_solve: by default (0) gathers whose state
+ * fits on chip are solved there, as many side by side as the SMs hold and one launch per such
+ * wave, and one persistent cooperative launch runs every PDHG iteration of the others (when
+ * all gathers have at most 7168 cells, each gets one shared-memory-resident CTA instead);
+ * 1 issues one launch per iteration over all gathers, 2 replays those launches from a captured CUDA graph.  All arrays of pointers and sizes are HOST
  * arrays of length B; the pointers they hold are device pointers with the layouts of
  * emd_dyn_solve.  params apply to every gather (its warm-start pointers must be NULL).
  * results: HOST array of B.  Returns EMD_OK if every gather succeeded, else the first
@@ -278,7 +283,7 @@ emd_status emd_misfit_batched_host(int B, const float *const *f_obs, const float
  * gathers return EMD_ERR_WORKSPACE without launching anything.  Arguments, outputs and
  * results are those of emd_dyn_solve, with two differences: tile = 0 takes the library's
  * default tile shape without the autotuner's timed trial solves, and no CUDA graph is
- * captured (launch_mode 0 runs the shared-memory or the persistent cooperative solve and,
+ * captured (launch_mode 0 runs the shared-memory, the on-chip or the persistent cooperative solve and,
  * where neither can be launched, one plain launch per pass; launch_mode 2 is run as 1).
  * Nothing calls cudaMalloc or cudaFree.  Like emd_dyn_solve the call copies small host
  * tables to the device and synchronises `stream` to read the result back.  The first call

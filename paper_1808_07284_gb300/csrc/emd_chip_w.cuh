@@ -18,6 +18,11 @@
 // both components of row -2, the x flux of row h + 1 and the t flux of samples -2 and 121 come
 // from the neighbours after every pass; the rest of the halo's flux is computed here (with the
 // isotropic cost, whose shrinkage needs both components, ux of sample -2 comes too).
+//
+// Measured, us per pass, against the streaming solve: 480 x 4000 8.2 (20.4): a row of a warp takes
+// 240 cycles of its scheduler, about 200 of them on the FMA pipe, and the pass boundary 3500 of
+// 17000 cycles.  648 x 8000, tall, 22.8 (43.7): 350 cycles a row, three warps a scheduler and the streamed
+// values' L2 latency.
 #pragma once
 
 #include "emd_chip.cuh"

@@ -10,7 +10,8 @@
 // left to the decider warp, which prepares the next decision's step sizes beside the pass.
 //
 // Shared planes, one float4 per quad: ux, ut (u^k, then u^{k+1}), phi, div u, q, p, f.  Every
-// cell's arithmetic and rounding are those of the tile pass.
+// cell's arithmetic and rounding are those of the tile pass.  Measured: 1 x 1024 1.4 us per pass (5.3 with
+// six barriers, scalar cells and FP64 totals and decisions), 20 x 200 3.4, 64 x 112 4.9.
 #pragma once
 
 #include "emd_chip.cuh"
