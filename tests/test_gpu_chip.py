@@ -83,6 +83,18 @@ def test_matches_the_streaming_pass(P, nr, nt, norm):
         check(P.emd(o, p, dt, dx, max_iter=1, **kw), P.emd(o, p, dt, dx, max_iter=1, tile=tile, **kw), "one")
 
 
+@pytest.mark.parametrize("scale", [1e-12, 1e-6, 1e4, 1e8])
+@pytest.mark.parametrize("nr,nt", [(64, 256), (353, 4001)])
+def test_amplitudes_match_the_streaming_pass(P, nr, nt, scale):
+    """Sums below 2^-60 and above 2^60 take the FP64 exchange in every pass, the others the
+    fixed-point one."""
+    o, p = pair(nr, nt, seed=4)
+    o, p = o * scale, p * scale
+    tile = streaming(nr * nt, nr)
+    for dt, dx in spacings(nr, nt):
+        check(P.emd(o, p, dt, dx, max_iter=25), P.emd(o, p, dt, dx, max_iter=25, tile=tile), (nr, nt, scale, dt))
+
+
 @pytest.mark.parametrize("kw", [dict(norm=2), dict(balance=0), dict(linesearch=0), dict(tol=1e-30, check_every=7),
                                 dict(xi=0.9), dict(alpha0=1e-3)])
 def test_options_match_the_streaming_pass(P, kw):
