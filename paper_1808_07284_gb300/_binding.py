@@ -174,8 +174,10 @@ def _check_grid(t, nr, nt, name, planes=1):
 
 
 def _grids(ts, nrs, nts, name, planes=1):
-    """The pointers of a list of grids, each checked as by _check_grid."""
+    """The pointers of a list of grids, one for each gather, each checked as by _check_grid."""
     import torch
+    if len(ts) != len(nrs):
+        raise IndexError(f"{name} must be a list of {len(nrs)} tensors, got {len(ts)}")
     ptrs = (c_void_p * len(nrs))()
     for b, (nr, nt) in enumerate(zip(nrs, nts)):
         t = ts[b]
@@ -279,7 +281,8 @@ def emd_dyn_solve_batched(f_obs, f_pred, dts, dxs, params: EmdParams, phis, ms, 
                           stream=None, check: bool = True):
     """B solves through the C ABI; lists of tensors; returns a list of EmdResult."""
     B = len(f_obs)
-    nrs, nts = zip(*[t.shape for t in f_obs]) if B else ((), ())
+    shapes = [t.shape for t in f_obs]
+    nrs, nts = [s[0] for s in shapes], [s[1] for s in shapes]
     res = (EmdResult * B)()
     st = lib().emd_dyn_solve_batched(
         B, _grids(f_obs, nrs, nts, "f_obs"), _grids(f_pred, nrs, nts, "f_pred"), (c_int * B)(*nts),
