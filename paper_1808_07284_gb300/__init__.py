@@ -13,6 +13,8 @@ library's kernels.
 
 from __future__ import annotations
 
+import ctypes
+
 from ._binding import (  # noqa: F401
     EMD_BAL_MEAN, EMD_BAL_NONE, EMD_ERR_ARG, EMD_NORM_ANISO, EMD_NORM_ISO, EMD_ERR_CUDA, EMD_ERR_LINESEARCH,
     EMD_ERR_NONFINITE, EMD_ERR_TIMEOUT, EMD_ERR_WORKSPACE, EMD_OK, EXPORTS,
@@ -117,6 +119,13 @@ def emd_misfit_host(f_obs, f_pred, dts, dxs, grad_preds=None, adjoint=True, work
     return [r.dist for r in res], grad_preds, [r.as_dict() for r in res]
 
 
+def _device_scalar(v, device):
+    """A 0-dim float32 tensor of v, filled on the device.  The rounding to float32 (a value beyond its
+    range becomes infinite) is done here: torch.full refuses such a value."""
+    import torch
+    return torch.full((), ctypes.c_float(v).value, dtype=torch.float32, device=device)
+
+
 def _autograd_function():
     import torch
 
@@ -132,7 +141,7 @@ def _autograd_function():
             ctx.dt, ctx.dx = float(dt), float(dx)
             ctx.balance = params.get("balance", EMD_BAL_MEAN)
             ctx.info = info
-            return torch.full((), dist, dtype=torch.float32, device=f_pred.device)
+            return _device_scalar(dist, f_pred.device)
 
         @staticmethod
         def backward(ctx, grad_out):
@@ -194,7 +203,7 @@ def _lsd_autograd_function():
             v = emd_lsd(f_obs.detach().contiguous(), f_pred.detach().contiguous(), float(dt), float(dx),
                         grad_pred=gp)
             ctx.save_for_backward(gp)
-            return torch.full((), v, dtype=torch.float32, device=f_pred.device)
+            return _device_scalar(v, f_pred.device)
 
         @staticmethod
         def backward(ctx, grad_out):

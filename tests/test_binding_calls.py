@@ -69,3 +69,17 @@ def test_batched_solve_names_the_wrong_tensor(calls):
     with pytest.raises(TypeError, match=r"phi\[0\]"):
         solve(obs, pred, phis, ms)
     assert not calls
+
+
+@pytest.mark.parametrize("value", [0.0, 0.1, -1e-50, 3.4028235e38, 3.4028236e38, -3.5e38, 1e300,
+                                   float("inf"), float("nan")])
+def test_losses_round_to_float32_as_a_conversion_does(monkeypatch, value):
+    """A misfit beyond the range of float32 is an infinite loss."""
+    import paper_1808_07284_gb300 as P
+    f = torch.zeros(3, 8, requires_grad=True)
+    monkeypatch.setattr(P, "emd_lsd", lambda *a, **k: value)
+    monkeypatch.setattr(P, "emd", lambda *a, **k: (value, torch.zeros(3, 8), None, {}))
+    want = torch.tensor(value, dtype=torch.float32)
+    for loss in (P.lsd_loss(f, torch.zeros(3, 8), 1.0, 1.0), P.emd_loss(f, torch.zeros(3, 8), 1.0, 1.0)):
+        assert loss.dtype == torch.float32 and loss.shape == () and loss.requires_grad
+        assert torch.equal(loss.detach().view(torch.int32), want.view(torch.int32)) or value != value and loss != loss
