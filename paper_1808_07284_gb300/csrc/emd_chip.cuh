@@ -567,26 +567,46 @@ struct ChipCta {
   unsigned smem;     // this lane's column of the first 512-byte row of shared memory
 };
 
-// The balancing sums over a lane's cells: f, f^2, |Pcal| + |Pobs| and Pcal - Pobs, each to about
-// 48 bits in FP32 pairs.
+// A sum in three floats: what rounding leaves of each addition goes to the next one.  Terms of a
+// lane's run (a few hundred) add to within 2^-66 of the sum of their magnitudes.
+struct Sum3 {
+  float hi = 0.0f, mid = 0.0f, lo = 0.0f;
+  __device__ __forceinline__ void add_low(float x) {
+    float e;
+    two_sum(mid, x, mid, e);
+    lo += e;
+  }
+  __device__ __forceinline__ void add(float x) {
+    float e;
+    two_sum(hi, x, hi, e);
+    add_low(e);
+  }
+  __device__ __forceinline__ double value() const {
+    return static_cast<double>(hi) + (static_cast<double>(mid) + static_cast<double>(lo));
+  }
+};
+
+// The balancing sums over a lane's cells: f, f^2, |Pcal| + |Pobs| and Pcal - Pobs.  The linear ones are
+// added in three floats, at least as exact as the FP64 sums of k_prepare (an FP64 instruction takes a
+// scheduler 64 cycles); the squares, which leave the range of FP32 where f is below 1e-19 or above
+// 1e18, in FP64.
 struct BalanceSums {
-  Sum2 f, f2, ab;
-  float de = 0.0f;  // rounding errors of the differences f = Pcal - Pobs
+  Sum3 f, ab;
+  Sum2 de;  // rounding errors of the differences f = Pcal - Pobs
+  double f2 = 0.0;
   __device__ __forceinline__ void add(float po, float pp) {
     float d, e;
     two_sum(pp, -po, d, e);
-    de += e;
+    de.add(e);
     f.add(d);
-    const float dd = d * d;
-    f2.add(dd);
-    f2.lo += fmaf(d, d, -dd);
+    f2 = fma(static_cast<double>(d), static_cast<double>(d), f2);
     two_sum(fabsf(pp), fabsf(po), d, e);
     ab.add(d);
-    ab.lo += e;
+    ab.add_low(e);
   }
   __device__ __forceinline__ void store(const ChipCta &X) {
-    const double t0 = warp_sum_d(f.value()), t1 = warp_sum_d(f2.value()), t2 = warp_sum_d(ab.value());
-    const double t3 = warp_sum_d(f.value() + static_cast<double>(de));
+    const double s = f.value();
+    const double t0 = warp_sum_d(s), t1 = warp_sum_d(f2), t2 = warp_sum_d(ab.value()), t3 = warp_sum_d(s + de.value());
     if (X.lane < 4) X.sh.dpart[X.warp][X.lane] = X.lane == 0 ? t0 : X.lane == 1 ? t1 : X.lane == 2 ? t2 : t3;
   }
 };
@@ -753,15 +773,20 @@ __device__ __forceinline__ void chip_decider(const ChipCta &X) {
   };
   publish_sc(sh.sc, static_cast<float>(pr.alpha), 0.0f, 1.0f, 1.0f / (1.0f + static_cast<float>(c.eps * pr.alpha)));
   if (lane >= 16 && lane < 24) sh.sc[lane >> 2][lane & 3] = lane < 20 ? rdx : rdt;
+  // Sums that left the range of FP32, or inputs that are not finite: the gather is handed back (the
+  // streaming solve adds these sums in FP64).
+  const bool summed = isfinite(m4[0]) && isfinite(m4[1]) && isfinite(m4[2]) && isfinite(m4[3]);
+  bool done = !summed;
+  int status = summed ? ST_OK : ST_NONFINITE;
   if (lane == 0) {
     sh.fmean = static_cast<float>(fmean);
+    sh.done = done;
+    sh.status = status;
     if (!ok) sh.bad = 1;
   }
   bar_all<4, NW>();
   int trials = 0;
   double r_feas = -1.0, r_step = -1.0;
-  bool done = false;
-  int status = ST_OK;
   const bool quick = c.linesearch && c.debug_fault != 1;
   // fixed-point exponents of the two families for the next fast exchange
   int fset = 0, e_p = 0, e_g = 0;

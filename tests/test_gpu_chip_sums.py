@@ -1,0 +1,86 @@
+"""The balancing sums of the on-chip solve (f, f^2, |Pcal| + |Pobs|, Pcal - Pobs) against exact ones,
+in its three forms, at amplitudes whose squares leave the range of FP32.
+
+The linear sums are added in more than 53 bits within a lane and in FP64 above it: at most 5 additions
+in a warp, 4 in a CTA, 19 + 2 across the CTAs of a copy and the copies, each rounded to 2^-53 of a
+partial sum, so they are exact to 30 * 2^-53 < 4e-15 of the sum of the magnitudes.  The reported
+residual is sqrt(sum p^2) / |f|, whose numerator is a sum of FP32 squares in every solve: 1e-5, as
+between any two of them."""
+
+import math
+
+import numpy as np
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+PLAIN, TILE, MARCH = 2, 7, 10
+SIZES = [(64, 256), (353, 4001), (640, 5000)]  # the tile form, the marching one, tall CTAs
+
+
+@pytest.fixture(scope="module")
+def P():
+    import paper_1808_07284_gb300 as pkg
+    assert torch.cuda.is_available()
+    return pkg
+
+
+def noise(nr, nt, seed):
+    return np.random.default_rng(seed).standard_normal((nr, nt))
+
+
+def solve(P, obs, pred, **kw):
+    o, p = (torch.from_numpy(np.ascontiguousarray(a, dtype=np.float32)).cuda() for a in (obs, pred))
+    return P.emd(o, p, 1.0, 1.0, **kw)
+
+
+@pytest.mark.parametrize("nr,nt", SIZES)
+@pytest.mark.parametrize("offset", [0.0, 1e3])
+def test_masses_are_exact_to_fp64(P, nr, nt, offset):
+    obs = noise(nr, nt, 1).astype(np.float32)
+    pred = (noise(nr, nt, 2) + offset).astype(np.float32)
+    info = solve(P, obs, pred, max_iter=1)[3]
+    assert info["status"] == 0 and info["tile"] == 0
+    o, p = obs.astype(np.float64).ravel(), pred.astype(np.float64).ravel()
+    total, net = math.fsum(np.abs(o)) + math.fsum(np.abs(p)), math.fsum(p - o)  # p - o is exact in FP64
+    bound = 4e-15 * total
+    assert abs(info["mass_mu"] + info["mass_nu"] - total) <= bound
+    assert abs(info["imbalance"] - net) <= bound
+
+
+@pytest.mark.parametrize("nr,nt", SIZES)
+def test_residual_of_small_amplitudes(P, nr, nt):
+    """Squares of 1e-44: a few of FP32's smallest steps, so a norm of f that is summed in FP32 is off
+    by a thousandth or more (the numerator's squares are those steps in every solve)."""
+    obs, pred = 1e-22 * noise(nr, nt, 3), 1e-22 * noise(nr, nt, 4)
+    got = solve(P, obs, pred, max_iter=5, alpha0=1e-4)[3]
+    ref = solve(P, obs, pred, max_iter=5, alpha0=1e-4, tile=TILE if nr * nt < 1.4e6 else MARCH)[3]
+    assert got["status"] == ref["status"] == 0 and got["tile"] == 0
+    assert math.isclose(got["r_feas"], ref["r_feas"], rel_tol=1e-5), (got["r_feas"], ref["r_feas"])
+
+
+def check_like_streaming(P, obs, pred):
+    nr, nt = obs.shape
+    got = solve(P, obs, pred, max_iter=5, alpha0=1e-4)
+    ref = solve(P, obs, pred, max_iter=5, alpha0=1e-4, tile=TILE if nr * nt < 1.4e6 else MARCH)
+    assert got[3]["status"] == ref[3]["status"] == 0
+    for key in ("r_feas", "mass_mu", "mass_nu", "dist"):
+        assert math.isclose(got[3][key], ref[3][key], rel_tol=1e-5), (key, got[3][key], ref[3][key])
+    return got
+
+
+@pytest.mark.parametrize("nr,nt", SIZES)
+def test_residual_above_a_common_level(P, nr, nt):
+    """Pcal on a level whose squares FP32 cannot add up.  Balancing takes the level out, so the pass's
+    own sums stay in range."""
+    got = check_like_streaming(P, np.zeros((nr, nt)), 8e18 + 1e16 * noise(nr, nt, 5))
+    assert got[3]["tile"] == 0
+
+
+@pytest.mark.parametrize("nr,nt", SIZES)
+def test_masses_beyond_the_range_of_a_float(P, nr, nt):
+    """Equal values of 1e37 in both gathers: f is zero there, but a lane's mass is not a float.  The
+    gather goes back to the streaming solve."""
+    big = noise(nr, nt, 6) < 0.0
+    check_like_streaming(P, np.where(big, 1e37, 0.0), np.where(big, 1e37, noise(nr, nt, 7)))
