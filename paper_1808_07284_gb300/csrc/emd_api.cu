@@ -13,6 +13,7 @@
 #include <vector>
 
 #include "emd_gb300.h"
+#include "emd_chip_plan.cuh"
 #include "emd_chip_w.cuh"
 #include "emd_kernels.cuh"
 #include "emd_lsd.cuh"
@@ -27,6 +28,10 @@ using emd::Ctl;
 using emd::kThreads;
 using emd::Shot;
 using emd::State;
+using emd::align256;
+using emd::ChipPlan;
+using emd::ntp_of;
+using emd::pick;
 
 #define EMD_CK(x)                                  \
   do {                                             \
@@ -135,8 +140,6 @@ int sm_count() {
   return n;
 }
 
-size_t align256(size_t x) { return (x + 255u) & ~static_cast<size_t>(255u); }
-int ntp_of(int nt) { return (nt + 31) / 32 * 32; }
 int tiles_of(const Shape &s, int nt, int nr) {
   return ((nr + s.ti - 1) / s.ti) * ((nt + (s.w - 8) - 1) / (s.w - 8));
 }
@@ -401,184 +404,6 @@ emd_status solve_impl(int B, const float *const *f_obs, const float *const *f_pr
                       const int *nr, const double *dt, const double *dx, const emd_params *pp,
                       float *const *phi, float *const *m, emd_result *results, void *ws,
                       size_t ws_bytes, cudaStream_t stream, const SolveExtra &x = SolveExtra{});
-
-// How the on-chip solve (emd_chip.cuh) lays a batch out: waves of gathers that are on chip side
-// by side, one cooperative launch per wave.
-struct ChipPlan {
-  std::vector<std::vector<emd::ChipJob>> waves;
-  std::vector<int> form;  // a wave's kernel: emd::ChipForm
-  double cost = 0.0;      // estimated time of one pass over every gather, us
-};
-
-// Estimated us per pass of a wave whose tallest CTA stages n rows: the pass boundary and the rows.
-// Measured: 2.8 us at 16 rows and 5.4 at 70 in the tile pass's form; 8.25 at 123 in the marching
-// pass's; 16.7 at 217 and 23.2 at 327 in tall CTAs.
-double chip_pass_us(int n, bool march) {
-  if (n > emd::kChipMaxRows) return 3.9 + 0.059 * n;
-  return march ? 2.4 + 0.048 * n : 2.0 + 0.049 * n;
-}
-
-// Estimated us per pass of the streaming solves (tile and marching pass) over `cells` cells:
-// about 10 us of decision chain and 5.9 us per million cells, from L2 or from HBM alike.
-double stream_pass_us(double cells) { return 10.0 + 5.9e-6 * cells; }
-
-int chip_strips(int nt) { return (nt + emd::kChipTJ - 1) / emd::kChipTJ; }
-
-// Staged rows of a gather's CTAs at the fewest rows that `cap` CTAs allow (0: it needs more CTAs
-// however tall they are).
-int chip_min_rows(int nt, int nr, int cap) {
-  const int segs = cap / chip_strips(nt);
-  return segs < 1 ? 0 : (nr + segs - 1) / segs + 3;
-}
-
-// Whether a gather's state fits on `cap` SMs, and in its planes what the on-chip solve keeps there:
-// the exchange buffers and, for tall CTAs, their streamed values.
-bool chip_fits(int nt, int nr, int cap, bool march) {
-  const int strips = chip_strips(nt), ntp = ntp_of(nt), rows = chip_min_rows(nt, nr, cap);
-  if (rows == 0 || rows > (march ? emd::kWMaxRows : emd::kChipMaxRows)) return false;
-  const size_t planes = 9 * align256(sizeof(float) * static_cast<size_t>(nr) * ntp);
-  const int lowest = emd::kChipWorkers - 3;  // receivers of the lowest CTAs (chip_plan)
-  size_t need = emd::chip_exchange_bytes((nr + lowest - 1) / lowest, strips, nr, ntp);
-  if (march && nr > emd::kChipMaxRows - 3) {
-    const int tall = (nr + emd::kChipMaxRows - 3) / (emd::kChipMaxRows - 2);  // segments of tall CTAs at most
-    need = std::max(need, emd::chip_exchange_bytes(tall, strips, nr, ntp) +
-                              4 * static_cast<size_t>(tall) * strips * emd::chip_w_tall_floats((nr + tall - 1) / tall + 3));
-  }
-  return need <= planes;
-}
-
-// The plan whose estimated pass is shortest, over the height of the CTAs (taller ones put more
-// gathers beside each other, lower ones spread a gather over more SMs); no waves when a gather
-// does not fit.
-ChipPlan chip_plan(int B, const int *nt, const int *nr, int cap, bool march) {
-  // staged rows of the tallest CTA: whole rows per worker warp, up to what the layout holds
-  std::vector<int> heights;
-  for (int n = emd::kChipWorkers; n < emd::kChipMaxRows; n += emd::kChipWorkers) heights.push_back(n);
-  heights.push_back(emd::kChipMaxRows);
-  if (march)
-    for (int n = emd::kChipMaxRows / emd::kTallWorkers * emd::kTallWorkers + emd::kTallWorkers; n <= emd::kWMaxRows;
-         n += emd::kTallWorkers)
-      heights.push_back(n);
-  auto is_tall = [](int n) { return n > emd::kChipMaxRows; };
-  std::vector<emd::ChipJob> g(B);
-  std::vector<int> order(B), used, rows;
-  std::vector<std::vector<int>> members;
-  auto lay_out = [&](int height) -> double {  // estimated us per pass, or -1
-    for (int b = 0; b < B; ++b) {
-      emd::ChipJob &J = g[b];
-      J.gather = b;
-      J.strips = chip_strips(nt[b]);
-      const int nseg = (nr[b] + height - 4) / (height - 3);
-      J.h = std::max(nr[b] > 1 ? 2 : 1, (nr[b] + nseg - 1) / nseg);
-      J.segs = (nr[b] + J.h - 1) / J.h;
-      if (static_cast<long long>(J.strips) * J.segs > cap) return -1.0;
-      J.group = J.strips * J.segs;
-      J.rows = J.h + 3;
-      order[b] = b;
-    }
-    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return g[a].group > g[b].group; });
-    used.clear();
-    rows.clear();
-    members.clear();
-    size_t open = 0;  // waves before this one are full
-    for (int b : order) {  // first fit, largest first; a wave's gathers share a layout
-      while (open < used.size() && used[open] + g[order.back()].group > cap) ++open;
-      size_t w = open;
-      while (w < used.size() && (used[w] + g[b].group > cap || is_tall(rows[w]) != is_tall(g[b].rows))) ++w;
-      if (w == used.size()) {
-        used.push_back(0);
-        rows.push_back(g[b].rows);
-        members.emplace_back();
-      }
-      used[w] += g[b].group;
-      rows[w] = std::max(rows[w], g[b].rows);
-      members[w].push_back(b);
-    }
-    double cost = 0.0;
-    for (int n : rows) cost += chip_pass_us(n, march);
-    return cost;
-  };
-  ChipPlan plan;
-  int best = 0;
-  for (const int height : heights) {
-    const double cost = lay_out(height);
-    if (cost < 0.0 || (best && cost >= plan.cost)) continue;
-    best = height;
-    plan.cost = cost;
-  }
-  if (!best) return plan;
-  lay_out(best);
-  for (size_t w = 0; w < members.size(); ++w) {
-    plan.waves.emplace_back();
-    plan.form.push_back(!march ? emd::kChipTile : is_tall(rows[w]) ? emd::kChipMarchTall : emd::kChipMarch);
-    for (int b : members[w])
-      for (int seg = 0; seg < g[b].segs; ++seg)
-        for (int strip = 0; strip < g[b].strips; ++strip) {
-          emd::ChipJob J = g[b];
-          J.seg = seg;
-          J.strip = strip;
-          J.i0 = seg * g[b].h;
-          J.h = std::min(g[b].h, nr[b] - J.i0);
-          plan.waves.back().push_back(J);
-        }
-  }
-  return plan;
-}
-
-// Copies of the elements `idx` of an array (empty for a null one).
-template <class T>
-std::vector<T> pick(const T *a, const std::vector<int> &idx) {
-  std::vector<T> v;
-  if (a)
-    for (int b : idx) v.push_back(a[b]);
-  return v;
-}
-
-// The gathers of a batch that are solved on chip (`on`, in order) and their plan.  Of three ways
-// the one whose estimated pass is shortest: every gather that fits, only those whose own pass
-// there is shorter than their share of a streamed pass, or none.
-//
-// *march: the form whose rounding the streaming solve of this batch has, the tile pass up to
-// about 1.4 million cells (and for thin gathers), where the autotuner takes it, the marching pass
-// above.  Measured crossing, single gathers: 400 x 3000 and 648 x 2000 take the tile pass, 400 x
-// 3500 and 300 x 5000 the march.
-ChipPlan choose_on_chip(int B, const int *nt, const int *nr, int cap, bool whole_only, std::vector<int> &on,
-                        bool *march) {
-  double cells = 0.0;
-  int receivers = 0;
-  for (int b = 0; b < B; ++b) {
-    cells += static_cast<double>(nt[b]) * nr[b];
-    receivers = std::max(receivers, nr[b]);
-  }
-  *march = cells >= 1.4e6 && receivers > 8;
-  ChipPlan plan;
-  double best = stream_pass_us(cells);
-  on.clear();
-  size_t tried = 0;
-  for (const bool all : {true, false}) {
-    std::vector<int> sub;
-    double left = cells;
-    for (int b = 0; b < B; ++b) {
-      const double n = static_cast<double>(nt[b]) * nr[b];
-      if (!chip_fits(nt[b], nr[b], cap, *march)) continue;
-      const int rows = chip_min_rows(nt[b], nr[b], cap);
-      if (!all && rows > emd::kChipMaxRows && chip_pass_us(rows, *march) > stream_pass_us(n) - stream_pass_us(0.0))
-        continue;
-      sub.push_back(b);
-      left -= n;
-    }
-    const int nb = static_cast<int>(sub.size());
-    if (nb == 0 || sub.size() == tried || (whole_only && nb < B)) continue;
-    tried = sub.size();
-    ChipPlan q = chip_plan(nb, pick(nt, sub).data(), pick(nr, sub).data(), cap, *march);
-    const double cost = q.cost + (nb < B ? stream_pass_us(left) : 0.0);
-    if (q.waves.empty() || cost >= best) continue;
-    best = cost;
-    on = std::move(sub);
-    plan = std::move(q);
-  }
-  return plan;
-}
 
 // Tile-shape autotuner of the TMA pass.  The first default-tile solve of a (device,
 // gather sizes) configuration times each TMA shape on the caller's own data -- two short
@@ -902,7 +727,7 @@ emd_status solve_impl(int B, const float *const *f_obs, const float *const *f_pr
   if (p.tile == 0 && p.launch_mode == 0 && !resident && !x.no_chip) {
     std::vector<int> on;
     bool march = false, launched = false;
-    const ChipPlan plan = choose_on_chip(B, nt, nr, std::min(sm_count(), emd::kChipMaxCtas), p.trace != nullptr, on,
+    const ChipPlan plan = emd::choose_on_chip(B, nt, nr, std::min(sm_count(), emd::kChipMaxCtas), p.trace != nullptr, on,
                                          &march);
     if (!on.empty()) {
       const emd_status s = static_cast<int>(on.size()) == B

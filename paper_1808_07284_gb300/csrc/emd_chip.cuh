@@ -36,17 +36,15 @@
 // 2.9 (8.5), 400 x 3000 5.4 (16.7).
 #pragma once
 
+#include "emd_chip_plan.cuh"
 #include "emd_pass_tma.cuh"
 
 namespace emd {
 
-constexpr int kChipWorkers = 15;                        // worker warps of a CTA (and a decider warp)
 constexpr int kChipTmemCols = 128;                      // tensor memory columns of a warp
 constexpr int kChipRowCols = 12;                        // ... of one row: ux, ut, phi
-constexpr int kChipMaxRows = 128;                       // staged rows of a CTA at most (shared memory)
 static_assert((kChipMaxRows + kChipWorkers - 1) / kChipWorkers * kChipRowCols <= kChipTmemCols, "a run's rows");
 
-constexpr int kChipTJ = 120;                            // owned time samples of a strip
 constexpr int kChipSets = 3;                            // accumulator sets, used in turn
 constexpr int kChipVals = 8;                            // sums of a pass
 constexpr int kChipSpread = 8;                          // copies of each accumulator
@@ -54,25 +52,10 @@ constexpr int kChipWordSets = 2;                        // word sets of the fast
 constexpr int kChipWordCopies = 4;                      // copies of the words of the fast exchange
 constexpr int kChipWords = 16;                          // two words of each value
 
-// One CTA's part of a gather.
-struct ChipJob {
-  int gather, seg, strip, segs, strips, i0, h;
-  int group, rows;  // CTAs of the gather, staged rows of its tallest CTA
-};
-constexpr int kChipMaxCtas = 160;  // CTAs of a launch at most (its jobs are a kernel argument)
 struct ChipJobs {
   ChipJob job[kChipMaxCtas];
 };
 
-// Exchange buffers of a gather, in the workspace of its planes: packets of the cells that other CTAs
-// hold as halo, two rows of every segment ([parity][seg][which][ntp]) and two samples of every
-// strip ([parity][strip][side][nr]).
-__host__ __device__ inline size_t chip_row_packets(int segs, int ntp) {
-  return segs > 1 ? static_cast<size_t>(2) * segs * 2 * ntp : 0;
-}
-__host__ __device__ inline size_t chip_exchange_bytes(int segs, int strips, int nr, int ntp) {
-  return 16 * (chip_row_packets(segs, ntp) + static_cast<size_t>(2) * strips * 2 * nr);
-}
 // Dynamic shared memory of a CTA: the planes div u, q and f at a fixed stride (so that one row
 // address serves the three of them), then four boundary rows per warp.
 constexpr unsigned kChipRowBytes = 512;

@@ -30,7 +30,6 @@
 namespace emd {
 
 constexpr int kWRowCols = 16;      // tensor memory columns of a row: two slots of ux, ut
-constexpr int kTallWorkers = 11;   // worker warps of a tall CTA: 168 registers a thread
 
 // The storage of a CTA of NW worker warps.
 template <int NW>
@@ -46,16 +45,10 @@ struct WLayout {
   static constexpr unsigned kBP = NW * kChipRowBytes, kBQ = 2 * kBP, kBUx = 3 * kBP;
   static constexpr unsigned kBUxSlot = (NW + 1) * kChipRowBytes;
 };
-constexpr int kWMaxRows = WLayout<kTallWorkers>::kMaxRows;
+static_assert(kWMaxRows == WLayout<kTallWorkers>::kMaxRows, "staged rows of a tall CTA at most");
 static_assert(2 * ((kChipMaxRows + kChipWorkers - 1) / kChipWorkers) + 4 <= WLayout<kChipWorkers>::kSlots &&
                   (kChipMaxRows + kChipWorkers - 1) / kChipWorkers <= WLayout<kChipWorkers>::kTmemRows + 1,
               "a run of 9 rows has no streamed values");
-
-// The exchange buffers (packets: ux, ut of the last-but-one owned row; ux of the second one; ut of the
-// second owned sample and ut, ux of the last-but-one) are followed, for tall CTAs, by [cta][rows][5]
-// [128] streamed values.
-constexpr int kTallRow = 5 * 128;
-__host__ __device__ inline size_t chip_w_tall_floats(int rows) { return static_cast<size_t>(rows) * kTallRow; }
 
 __device__ __forceinline__ Q4 ldg4(const float *p) {
   const float4 t = __ldcg(reinterpret_cast<const float4 *>(p));
@@ -700,8 +693,6 @@ __device__ __forceinline__ void chip_worker_w(const ChipCta &X) {
     bar_all_arrive<2, NW>();
   }
 }
-
-enum ChipForm { kChipTile = 0, kChipMarch = 1, kChipMarchTall = 2 };
 
 __host__ __device__ constexpr int chip_workers(int form) { return form == kChipMarchTall ? kTallWorkers : kChipWorkers; }
 
