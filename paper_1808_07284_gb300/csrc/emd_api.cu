@@ -727,8 +727,8 @@ emd_status solve_impl(int B, const float *const *f_obs, const float *const *f_pr
   if (p.tile == 0 && p.launch_mode == 0 && !resident && !x.no_chip) {
     std::vector<int> on;
     bool march = false, launched = false;
-    const ChipPlan plan = emd::choose_on_chip(B, nt, nr, std::min(sm_count(), emd::kChipMaxCtas), p.trace != nullptr, on,
-                                         &march);
+    const ChipPlan plan = emd::choose_on_chip(B, nt, nr, std::min(sm_count(), emd::kChipMaxCtas),
+                                              p.norm == EMD_NORM_ISO, p.trace != nullptr, on, &march);
     if (!on.empty()) {
       const emd_status s = static_cast<int>(on.size()) == B
                                ? solve_on_chip(B, f_obs, f_pred, nt, nr, dt, dx, p, phi, m, results, ws, ws_bytes,

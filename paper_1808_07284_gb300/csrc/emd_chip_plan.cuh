@@ -60,15 +60,22 @@ struct ChipPlan {
 
 // Estimated us per pass of a wave whose tallest CTA stages n rows: the pass boundary and the rows.
 // Measured: 2.8 us at 16 rows and 5.4 at 70 in the tile pass's form; 8.25 at 123 in the marching
-// pass's; 16.7 at 217 and 23.2 at 327 in tall CTAs.
-inline double chip_pass_us(int n, bool march) {
+// pass's; 16.7 at 217 and 23.2 at 327 in tall CTAs.  With the isotropic cost, whose square root and division
+// take issue slots: 3.3 at 14 rows, 7.4 at 70; 11.8 at 92, 14.6 at 123; 22.5 at 150, 32.9 at 253, 44.8 at 327 and
+// 58.3 at 383, where the streamed rows no longer stay in L2.
+inline double chip_pass_us(int n, bool march, bool iso) {
+  if (iso) {
+    if (n > kChipMaxRows) return 4.5 + 0.12 * n + 0.13 * std::max(0, n - 327);
+    return march ? 2.4 + 0.099 * n : 2.2 + 0.076 * n;
+  }
   if (n > kChipMaxRows) return 3.9 + 0.059 * n;
   return march ? 2.4 + 0.048 * n : 2.0 + 0.049 * n;
 }
 
 // Estimated us per pass of the streaming solves (tile and marching pass) over `cells` cells:
-// about 10 us of decision chain and 5.9 us per million cells, from L2 or from HBM alike.
-inline double stream_pass_us(double cells) { return 10.0 + 5.9e-6 * cells; }
+// about 10 us of decision chain and 5.9 us per million cells, from L2 or from HBM alike; with the
+// isotropic cost 23.5 us at 1.4 million cells, 38 at 3.2, 54 at 5.2, 172 at 20.7 and 256 at 30.7.
+inline double stream_pass_us(double cells, bool iso) { return iso ? 12.0 + 7.8e-6 * cells : 10.0 + 5.9e-6 * cells; }
 
 inline int chip_strips(int nt) { return (nt + kChipTJ - 1) / kChipTJ; }
 
@@ -98,7 +105,7 @@ inline bool chip_fits(int nt, int nr, int cap, bool march) {
 // The plan whose estimated pass is shortest, over the height of the CTAs (taller ones put more
 // gathers beside each other, lower ones spread a gather over more SMs); no waves when a gather
 // does not fit.
-inline ChipPlan chip_plan(int B, const int *nt, const int *nr, int cap, bool march) {
+inline ChipPlan chip_plan(int B, const int *nt, const int *nr, int cap, bool march, bool iso) {
   // staged rows of the tallest CTA: whole rows per worker warp, up to what the layout holds
   std::vector<int> heights;
   for (int n = kChipWorkers; n < kChipMaxRows; n += kChipWorkers) heights.push_back(n);
@@ -143,7 +150,7 @@ inline ChipPlan chip_plan(int B, const int *nt, const int *nr, int cap, bool mar
       members[w].push_back(b);
     }
     double cost = 0.0;
-    for (int n : rows) cost += chip_pass_us(n, march);
+    for (int n : rows) cost += chip_pass_us(n, march, iso);
     return cost;
   };
   ChipPlan plan;
@@ -190,7 +197,7 @@ std::vector<T> pick(const T *a, const std::vector<int> &idx) {
 // about 1.4 million cells (and for thin gathers), where the autotuner takes it, the marching pass
 // above.  Measured crossing, single gathers: 400 x 3000 and 648 x 2000 take the tile pass, 400 x
 // 3500 and 300 x 5000 the march.
-inline ChipPlan choose_on_chip(int B, const int *nt, const int *nr, int cap, bool whole_only,
+inline ChipPlan choose_on_chip(int B, const int *nt, const int *nr, int cap, bool iso, bool whole_only,
                                std::vector<int> &on, bool *march) {
   double cells = 0.0;
   int receivers = 0;
@@ -200,7 +207,7 @@ inline ChipPlan choose_on_chip(int B, const int *nt, const int *nr, int cap, boo
   }
   *march = cells >= 1.4e6 && receivers > 8;
   ChipPlan plan;
-  double best = stream_pass_us(cells);
+  double best = stream_pass_us(cells, iso);
   on.clear();
   size_t tried = 0;
   for (const bool all : {true, false}) {
@@ -210,7 +217,8 @@ inline ChipPlan choose_on_chip(int B, const int *nt, const int *nr, int cap, boo
       const double n = static_cast<double>(nt[b]) * nr[b];
       if (!chip_fits(nt[b], nr[b], cap, *march)) continue;
       const int rows = chip_min_rows(nt[b], nr[b], cap);
-      if (!all && rows > kChipMaxRows && chip_pass_us(rows, *march) > stream_pass_us(n) - stream_pass_us(0.0))
+      if (!all && rows > kChipMaxRows &&
+          chip_pass_us(rows, *march, iso) > stream_pass_us(n, iso) - stream_pass_us(0.0, iso))
         continue;
       sub.push_back(b);
       left -= n;
@@ -218,8 +226,8 @@ inline ChipPlan choose_on_chip(int B, const int *nt, const int *nr, int cap, boo
     const int nb = static_cast<int>(sub.size());
     if (nb == 0 || sub.size() == tried || (whole_only && nb < B)) continue;
     tried = sub.size();
-    ChipPlan q = chip_plan(nb, pick(nt, sub).data(), pick(nr, sub).data(), cap, *march);
-    const double cost = q.cost + (nb < B ? stream_pass_us(left) : 0.0);
+    ChipPlan q = chip_plan(nb, pick(nt, sub).data(), pick(nr, sub).data(), cap, *march, iso);
+    const double cost = q.cost + (nb < B ? stream_pass_us(left, iso) : 0.0);
     if (q.waves.empty() || cost >= best) continue;
     best = cost;
     on = std::move(sub);
