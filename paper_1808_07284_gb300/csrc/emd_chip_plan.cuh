@@ -116,8 +116,7 @@ inline ChipPlan chip_plan(int B, const int *nt, const int *nr, int cap, bool mar
       heights.push_back(n);
   auto is_tall = [](int n) { return n > kChipMaxRows; };
   std::vector<ChipJob> g(B);
-  std::vector<int> order(B), used, rows;
-  std::vector<std::vector<int>> members;
+  std::vector<int> order(B), wave(B), start, used, rows;
   auto lay_out = [&](int height) -> double {  // estimated us per pass, or -1
     for (int b = 0; b < B; ++b) {
       ChipJob &J = g[b];
@@ -129,25 +128,33 @@ inline ChipPlan chip_plan(int B, const int *nt, const int *nr, int cap, bool mar
       if (static_cast<long long>(J.strips) * J.segs > cap) return -1.0;
       J.group = J.strips * J.segs;
       J.rows = J.h + 3;
-      order[b] = b;
     }
-    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return g[a].group > g[b].group; });
+    start.assign(cap + 1, 0);  // the gathers in falling order of their CTAs (a counting sort)
+    for (int b = 0; b < B; ++b) ++start[cap - g[b].group + 1];
+    for (int i = 1; i <= cap; ++i) start[i] += start[i - 1];
+    for (int b = 0; b < B; ++b) order[start[cap - g[b].group]++] = b;
     used.clear();
     rows.clear();
-    members.clear();
-    size_t open = 0;  // waves before this one are full
-    for (int b : order) {  // first fit, largest first; a wave's gathers share a layout
+    // First fit, largest first; a wave's gathers share a layout.  Gathers of as many CTAs and the same
+    // layout look on from the last one's wave, since no wave before it can take them: the waves are
+    // walked once for each number of CTAs, not once for each gather (20,000 uneven gathers: 240 ms).
+    size_t open = 0, from[2] = {0, 0};  // waves before `open` are full
+    int group = -1;
+    for (int b : order) {
       while (open < used.size() && used[open] + g[order.back()].group > cap) ++open;
-      size_t w = open;
-      while (w < used.size() && (used[w] + g[b].group > cap || is_tall(rows[w]) != is_tall(g[b].rows))) ++w;
+      if (g[b].group != group) from[0] = from[1] = open;
+      group = g[b].group;
+      const bool tall = is_tall(g[b].rows);
+      size_t w = std::max(open, from[tall]);
+      while (w < used.size() && (used[w] + group > cap || is_tall(rows[w]) != tall)) ++w;
       if (w == used.size()) {
         used.push_back(0);
         rows.push_back(g[b].rows);
-        members.emplace_back();
       }
-      used[w] += g[b].group;
+      used[w] += group;
       rows[w] = std::max(rows[w], g[b].rows);
-      members[w].push_back(b);
+      from[tall] = w;
+      wave[b] = static_cast<int>(w);
     }
     double cost = 0.0;
     for (int n : rows) cost += chip_pass_us(n, march, iso);
@@ -163,6 +170,8 @@ inline ChipPlan chip_plan(int B, const int *nt, const int *nr, int cap, bool mar
   }
   if (!best) return plan;
   lay_out(best);
+  std::vector<std::vector<int>> members(used.size());
+  for (int b : order) members[wave[b]].push_back(b);
   for (size_t w = 0; w < members.size(); ++w) {
     plan.waves.emplace_back();
     plan.form.push_back(!march ? kChipTile : is_tall(rows[w]) ? kChipMarchTall : kChipMarch);

@@ -127,3 +127,46 @@ def test_the_isotropic_cost_streams_where_tall_ctas_are_slower(plan):
         assert len(p["on"]) == len(s)
     for s, p in zip(chip, plan([(1, s) for s in chip])):
         assert len(p["on"]) == len(s)
+
+
+def first_fit(sizes, p):
+    """The gathers of each wave by first fit, the ones of most CTAs first, at the heights of the plan."""
+    jobs = {J[0]: J for wave in p["waves"] for J in wave["jobs"]}
+    waves = []
+    for g in sorted(jobs, key=lambda g: (-jobs[g][7], g)):
+        group, rows = jobs[g][7:]
+        for w in waves:
+            if w["used"] + group <= CAP and w["tall"] == (rows > 128):
+                break
+        else:
+            w = dict(used=0, tall=rows > 128, members=[])
+            waves.append(w)
+        w["used"] += group
+        w["members"].append(g)
+    return [w["members"] for w in waves]
+
+
+def uneven(n, seed):
+    rng = random.Random(seed)
+    return [(rng.randint(16, 76), rng.randint(600, 2100)) for _ in range(n)]
+
+
+def test_waves_are_filled_by_first_fit(plan):
+    rng = random.Random(9)
+    batches = [[(log_int(rng, 9, 1200), log_int(rng, 64, 9000)) for _ in range(rng.randint(2, 60))] for _ in range(150)]
+    batches += [uneven(400, 1), [(100, 1500), (643, 6915), (30, 700)] * 50, [(64, 8000)] * 30]
+    answers = plan([(0, s) for s in batches])
+    assert sum(1 for p in answers if len(p["waves"]) > 3) > 50
+    for sizes, p in zip(batches, answers):
+        got = []
+        for wave in p["waves"]:
+            seen = dict.fromkeys(J[0] for J in wave["jobs"])
+            got.append(list(seen))
+        assert got == first_fit(sizes, p)
+
+
+def test_a_plan_takes_time_in_proportion_to_the_batch(plan):
+    """First fit over every wave for every gather took the square of it: 4 ms for 2000, 240 for 20,000."""
+    small, large = uneven(2000, 2), uneven(20000, 3)
+    ms = [min(p["ms"] for p in plan([(0, s)] * 3)) for s in (small, large)]
+    assert ms[1] < 25.0 * ms[0], ms
