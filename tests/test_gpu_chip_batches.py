@@ -1,0 +1,109 @@
+"""Batches of on-chip solves in which gathers fail, against single streaming solves: the gathers that a
+solve gives up are solved again in the workspace of the batch, by the passes of its rounding, and the
+others keep what they have."""
+
+import math
+
+import numpy as np
+import pytest
+import torch
+
+import synth
+
+pytestmark = pytest.mark.gpu
+
+PLAIN, TILE, MARCH = 2, 7, 10
+
+
+@pytest.fixture(scope="module")
+def P():
+    import paper_1808_07284_gb300 as pkg
+    assert torch.cuda.is_available()
+    return pkg
+
+
+def pairs(sizes, seed):
+    out = []
+    for i, (nr, nt) in enumerate(sizes):
+        obs, pred = synth.gather_pair_hyperbolic(nt=nt, nr=nr, seed=seed + i)
+        noise = 0.05 * np.random.default_rng(seed + i).standard_normal(obs.shape).astype(np.float32)
+        out.append((torch.from_numpy(obs).cuda(), torch.from_numpy(pred + noise).cuda()))
+    return [o for o, _ in out], [p for _, p in out]
+
+
+def unit(sizes):
+    return [1.0 / (nt - 1) for _, nt in sizes], [1.0 / max(nr - 1, 1) for nr, _ in sizes]
+
+
+def streaming(sizes):
+    if max(nr for nr, _ in sizes) <= 8 or all(nr * nt <= 7168 for nr, nt in sizes):
+        return PLAIN
+    return TILE if sum(nr * nt for nr, nt in sizes) < 1.4e6 else MARCH
+
+
+def same(got, ref, what):
+    """Equal iterates (but for a decision that sums of another order take otherwise, of which there is
+    none in these few iterations), and distances of two float sums of equal terms."""
+    (d, phi, m, info), (d0, phi0, m0, info0) = got, ref
+    assert info["status"] == info0["status"] and info["iters"] == info0["iters"], what
+    assert info["ls_trials"] == info0["ls_trials"], what
+    for a, b, name in ((phi, phi0, "phi"), (m, m0, "m")):
+        rel = float((a.double() - b.double()).norm() / b.double().norm().clamp_min(1e-300))
+        assert rel <= 1e-6, (what, name, rel)
+    assert math.isclose(d, d0, rel_tol=1e-6), (what, d, d0)
+
+
+BATCHES = [[(20, 200)] * 4, [(64, 256)] * 4, [(353, 4001)] * 3, [(640, 5000), (64, 256), (300, 5041)],
+           [(64, 256), (400, 3000), (20, 8000), (700, 9000), (33, 401)]]
+
+
+@pytest.mark.parametrize("sizes", BATCHES)
+@pytest.mark.parametrize("bad", ["first", "last", "all but one"])
+def test_failed_gathers_leave_the_others_alone(P, sizes, bad):
+    obs, pred = pairs(sizes, 20)
+    dts, dxs = unit(sizes)
+    n = len(sizes)
+    broken = {"first": [0], "last": [n - 1], "all but one": [b for b in range(n) if b != 1]}[bad]
+    for b in broken:
+        pred[b] = pred[b].clone()
+        pred[b][1, 17] = float("nan")
+    d, phis, ms, infos = P.emd_batched(obs, pred, dts, dxs, max_iter=20, check=False)
+    assert any(i["tile"] == 0 for b, i in enumerate(infos) if b not in broken)
+    for b in range(n):
+        if b in broken:
+            assert infos[b]["status"] == P.EMD_ERR_NONFINITE
+            continue
+        ref = P.emd(obs[b], pred[b], dts[b], dxs[b], max_iter=20, tile=infos[b]["tile"] or streaming(sizes))
+        same((d[b], phis[b], ms[b], infos[b]), ref, (sizes[b], bad))
+
+
+@pytest.mark.parametrize("sizes", BATCHES)
+def test_failed_linesearches_leave_what_the_passes_of_their_rounding_leave(P, sizes):
+    """One trial a decision from small steps: a few iterations pass, then the linesearch gives up.  phi and m
+    are the iterates of the streaming passes of the batch's rounding there (those of the tile and the
+    marching pass differ by then), and every gather has its trace."""
+    obs, pred = pairs(sizes, 40)
+    dts, dxs = unit(sizes)
+    n, iters = len(sizes), 60
+    kw = dict(max_iter=iters, ls_max_trials=1, alpha0=1e-7, check=False)
+    tile = streaming(sizes)
+    chip = [i["tile"] == 0 for i in P.emd_batched(obs, pred, dts, dxs, max_iter=2)[3]]
+    d, phis, ms, infos = P.emd_batched(obs, pred, dts, dxs, **kw)
+    failed = 0
+    for b in range(n):
+        if not chip[b]:
+            continue
+        ref = P.emd(obs[b], pred[b], dts[b], dxs[b], tile=tile, **kw)
+        assert infos[b]["status"] == ref[3]["status"]
+        failed += ref[3]["status"] == P.EMD_ERR_LINESEARCH and ref[3]["iters"] > 0
+        same((d[b], phis[b], ms[b], infos[b]), ref, sizes[b])
+        assert torch.equal(phis[b], ref[1]) and torch.equal(ms[b], ref[2]), sizes[b]
+    assert failed
+    trace = torch.zeros((n, iters, 4), dtype=torch.float64, device="cuda")
+    infos = P.emd_batched(obs, pred, dts, dxs, trace=trace, **kw)[3]
+    for b in range(n):
+        one = torch.zeros((1, iters, 4), dtype=torch.float64, device="cuda")
+        ref = P.emd(obs[b], pred[b], dts[b], dxs[b], tile=tile, trace=one, **kw)[3]
+        assert infos[b]["iters"] == ref["iters"]
+        k = infos[b]["iters"]
+        assert torch.allclose(trace[b, :k], one[0, :k], rtol=1e-5, atol=0.0), sizes[b]
