@@ -725,14 +725,12 @@ emd_status solve_split(int B, const float *const *f_obs, const float *const *f_p
       s = solve_impl(nb, a_obs.data(), a_pred.data(), a_nt.data(), a_nr.data(), a_dt.data(), a_dx.data(), &p,
                      a_phi.data(), a_m.data(), res.data(), ws, ws_bytes, stream, y);
     }
-    for (int i = 0; i < nb; ++i) results[idx[i]] = res[i];
     if (s == EMD_ERR_TIMEOUT)
       for (int b = 0; b < B; ++b) results[b].status = s;
-    if (s == EMD_ERR_CUDA || s == EMD_ERR_TIMEOUT) return s;
+    if (of_the_call(s)) return s;  // a half that did not run has no results
+    for (int i = 0; i < nb; ++i) results[idx[i]] = res[i];
   }
-  for (int b = 0; b < B; ++b)
-    if (results[b].status != EMD_OK) return static_cast<emd_status>(results[b].status);
-  return EMD_OK;
+  return first_status(B, results);
 }
 
 emd_status solve_impl(int B, const float *const *f_obs, const float *const *f_pred, const int *nt,
@@ -1429,8 +1427,7 @@ emd_status emd_misfit_batched_host(int B, const float *const *f_obs, const float
   x.stage = &stage;
   const emd_status st = solve_impl(B, d_obs.data(), d_pred.data(), nt, nr, dt, dx, &p, d_phi.data(),
                                    d_m.data(), results, base, solve_ws, stream, x);
-  if (st == EMD_ERR_ARG || st == EMD_ERR_CUDA || st == EMD_ERR_TIMEOUT || st == EMD_ERR_WORKSPACE)
-    return st;
+  if (of_the_call(st)) return st;
   if (grad_pred) {
     const emd_status sa = emd_adjoint_batched(B, d_phi.data(), nt, nr, dt, dx, p.balance, nullptr,
                                               d_gp.data(), nullptr, base + align256(solve_ws),
