@@ -279,12 +279,12 @@ __device__ __forceinline__ void bar_all_arrive() {
   asm volatile("bar.arrive %0, %1;\n" ::"n"(ID), "n"((NW + 1) * 32) : "memory");
 }
 
-// Warp totals of eight values: lane l ends with the total of value l & 7 (all 32 lanes summed,
-// FP32, pairwise).  The first three steps exchange halves of the values, so nine shuffles do.
-__device__ __forceinline__ float warp_sum8(const float (&v)[8]) {
+// Totals of eight values over each group of eight lanes: lane l ends with the total of value l & 7
+// over its group (FP32, pairwise).  Each step exchanges halves of the values, so seven shuffles do.
+__device__ __forceinline__ float group_sum8(const float (&v)[8]) {
   constexpr unsigned FULL = 0xffffffffu;
   const int lane = threadIdx.x & 31;
-  float a[4], b[2], s;
+  float a[4], b[2];
 #pragma unroll
   for (int i = 0; i < 4; ++i) {  // lanes with bit 2 set keep values 4..7
     const bool hi = lane & 4;
@@ -297,13 +297,27 @@ __device__ __forceinline__ float warp_sum8(const float (&v)[8]) {
     const float keep = hi ? a[i + 2] : a[i], send = hi ? a[i] : a[i + 2];
     b[i] = keep + __shfl_xor_sync(FULL, send, 2);
   }
-  {
-    const bool hi = lane & 1;
-    const float keep = hi ? b[1] : b[0], send = hi ? b[0] : b[1];
-    s = keep + __shfl_xor_sync(FULL, send, 1);
-  }
-  s += __shfl_xor_sync(FULL, s, 8);
-  s += __shfl_xor_sync(FULL, s, 16);
+  const bool hi = lane & 1;
+  const float keep = hi ? b[1] : b[0], send = hi ? b[0] : b[1];
+  return keep + __shfl_xor_sync(FULL, send, 1);
+}
+
+// Warp totals of eight values: lane l ends with the total of value l & 7 (all 32 lanes summed, FP32).
+__device__ __forceinline__ float warp_sum8(const float (&v)[8]) {
+  float s = group_sum8(v);
+  s += __shfl_xor_sync(0xffffffffu, s, 8);
+  s += __shfl_xor_sync(0xffffffffu, s, 16);
+  return s;
+}
+
+// The same with the last two additions, whose rounding counts most, in a pair of floats.
+__device__ __forceinline__ float warp_sum8_pair(const float (&v)[8], float &low) {
+  constexpr unsigned FULL = 0xffffffffu;
+  float s = group_sum8(v), t, e;
+  two_sum(s, __shfl_xor_sync(FULL, s, 8), t, e);
+  const float t16 = __shfl_xor_sync(FULL, t, 16), e16 = __shfl_xor_sync(FULL, e, 16);
+  two_sum(t, t16, s, low);
+  low += e + e16;
   return s;
 }
 
@@ -324,6 +338,7 @@ struct ChipShared {
   alignas(16) float sc[6][4];
   float warm[6][4];                          // takes what the decision writes when it runs for nothing
   float part[16][kChipVals];                 // warp totals of a pass (zero for warps that are not there)
+  float low[16][kChipVals];                  // tall CTAs: their low parts
   double dpart[16][4];                       // warp totals of the balancing sums
 };
 
@@ -355,7 +370,10 @@ __device__ __forceinline__ bool chip_exchange(const Ctl &c, State *st, double *a
 // The totals over a CTA's warps of their FP32 totals, to a pair (hi, lo) of floats that every lane
 // holds for value lane & 7.  (Two-sums are 4-cycle operations; FP64 takes 64 cycles for each of
 // the nine conversions and additions.)
-__device__ __forceinline__ void chip_block_pair(const float (&part)[16][kChipVals], float &s, float &e) {
+// LOW: the warps' totals are pairs themselves, with these low parts.
+template <bool LOW>
+__device__ __forceinline__ void chip_block_pair(const float (&part)[16][kChipVals], const float (&low)[16][kChipVals],
+                                                float &s, float &e) {
   constexpr unsigned FULL = 0xffffffffu;
   const int lane = threadIdx.x & 31, g = lane >> 3, q = lane & 7;
   float s0, e0, s1, e1;
@@ -363,6 +381,7 @@ __device__ __forceinline__ void chip_block_pair(const float (&part)[16][kChipVal
   two_sum(part[g + 8][q], part[g + 12][q], s1, e1);
   two_sum(s0, s1, s, e);
   e += e0 + e1;
+  if (LOW) e += (low[g][q] + low[g + 4][q]) + (low[g + 8][q] + low[g + 12][q]);
 #pragma unroll
   for (int o = 8; o <= 16; o <<= 1) {
     const float so = __shfl_xor_sync(FULL, s, o), eo = __shfl_xor_sync(FULL, e, o);
@@ -374,7 +393,7 @@ __device__ __forceinline__ void chip_block_pair(const float (&part)[16][kChipVal
 // hi in lanes 0..7 and lo in the others, so that lanes 0..15 add both.
 __device__ __forceinline__ double chip_block_total(const ChipShared &sh) {
   float s, e;
-  chip_block_pair(sh.part, s, e);
+  chip_block_pair<false>(sh.part, sh.low, s, e);
   return static_cast<double>((threadIdx.x & 31) < 8 ? s : e);
 }
 
@@ -713,7 +732,9 @@ __device__ __forceinline__ void chip_input_rows(const ChipCta &X, const ChipLane
 }
 
 // Warp totals of a pass's eight packed sums (the two lanes that only feed neighbours leave theirs
-// out), for the decider.
+// out), for the decider.  LOW: in pairs, for the long runs of tall CTAs (with plain warp totals their
+// reported residual was 1.5 times as far from 64 bits as the streaming solve's; now 0.8 times).
+template <bool LOW = false>
 __device__ __forceinline__ void chip_store_sums(const ChipCta &X, const f32x2 (&v)[8], bool own) {
   float t[8];
 #pragma unroll
@@ -722,8 +743,10 @@ __device__ __forceinline__ void chip_store_sums(const ChipCta &X, const f32x2 (&
     upk(v[q], x, y);
     t[q] = own ? x + y : 0.0f;
   }
-  const float tot = warp_sum8(t);
+  float low = 0.0f;
+  const float tot = LOW ? warp_sum8_pair(t, low) : warp_sum8(t);
   if (X.lane < 8) X.sh.part[X.warp][X.lane] = tot;
+  if (LOW && X.lane < 8) X.sh.low[X.warp][X.lane] = low;
 }
 
 // The decider warp: the balancing constants, every pass's decision and the gather's final state.
@@ -800,7 +823,7 @@ __device__ __forceinline__ void chip_decider(const ChipCta &X) {
     bool slow = !scaled || check || pr.k + 1 >= c.max_iter;
     bar_all<2, NW>();
     float hi, lo, f = 0.0f;
-    chip_block_pair(sh.part, hi, lo);
+    chip_block_pair<NW == kTallWorkers>(sh.part, sh.low, hi, lo);
     FastTotal ft;
     const int sa = 24 - ((lane & 7) < 3 ? e_p : e_g);
     // The decision's instructions have left the instruction cache since the last pass (1300 cycles

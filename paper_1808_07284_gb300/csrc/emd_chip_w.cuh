@@ -541,7 +541,7 @@ __device__ __forceinline__ void chip_worker_w(const ChipCta &X) {
     if (run > 0 && ra >= 2 && ra < n - 1)
       grad_row(any, ra, p_a, q_a, lds4<kWBP - kChipRowBytes>(brow), lds4<kWBQ - kChipRowBytes>(brow));
 
-    chip_store_sums(X, v, own_lane);
+    chip_store_sums<TALL>(X, v, own_lane);
     bar_all_arrive<2, NW>();
     // ---- halo flux of the pass
     bool got = true;
@@ -712,7 +712,7 @@ __global__ void __launch_bounds__((chip_workers(FORM) + 1) * 32, 1) k_solve_chip
     sh.status = ST_OK;
     sh.bad = 0;
   }
-  if (threadIdx.x < 16 * kChipVals) (&sh.part[0][0])[threadIdx.x] = 0.0f;  // of warps that are not there
+  if (threadIdx.x < 16 * kChipVals) (&sh.part[0][0])[threadIdx.x] = (&sh.low[0][0])[threadIdx.x] = 0.0f;  // of warps that are not there
   if (threadIdx.x < 16 * 4) (&sh.dpart[0][0])[threadIdx.x] = 0.0;
   asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
   __syncthreads();
