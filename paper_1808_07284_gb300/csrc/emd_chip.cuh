@@ -585,49 +585,40 @@ struct ChipCta {
   unsigned smem;     // this lane's column of the first 512-byte row of shared memory
 };
 
-// A sum in three floats: what rounding leaves of each addition goes to the next one.  Terms of a
-// lane's run (a few hundred) add to within 2^-66 of the sum of their magnitudes.
-struct Sum3 {
-  float hi = 0.0f, mid = 0.0f, lo = 0.0f;
-  __device__ __forceinline__ void add_low(float x) {
-    float e;
-    two_sum(mid, x, mid, e);
-    lo += e;
-  }
-  __device__ __forceinline__ void add(float x) {
-    float e;
-    two_sum(hi, x, hi, e);
-    add_low(e);
-  }
-  __device__ __forceinline__ double value() const {
-    return static_cast<double>(hi) + (static_cast<double>(mid) + static_cast<double>(lo));
-  }
-};
-
-// The balancing sums over a lane's cells: f, f^2, |Pcal| + |Pobs| and Pcal - Pobs.  The linear ones are
-// added in three floats, at least as exact as the FP64 sums of k_prepare (an FP64 instruction takes a
-// scheduler 64 cycles); the squares, which leave the range of FP32 where f is below 1e-19 or above
-// 1e18, in FP64.
+// The balancing sums over a lane's cells: f, f^2, |Pcal| + |Pobs| and Pcal - Pobs, each to about
+// 48 bits in FP32 pairs (an FP64 instruction takes a scheduler 64 cycles).  Over a gather they are as near
+// to the exact sums as k_prepare's FP64 ones, as long as FP32 holds them: see balance_in_range.
+// (Squares in FP64 cost 12 us of a solve of 648 x 8000, and they or a third float for f 0.3 us of each of
+// its passes by what they do to the kernel's registers.)
 struct BalanceSums {
-  Sum3 f, ab;
-  Sum2 de;  // rounding errors of the differences f = Pcal - Pobs
-  double f2 = 0.0;
+  Sum2 f, f2, ab;
+  float de = 0.0f;  // rounding errors of the differences f = Pcal - Pobs
   __device__ __forceinline__ void add(float po, float pp) {
     float d, e;
     two_sum(pp, -po, d, e);
-    de.add(e);
+    de += e;
     f.add(d);
-    f2 = fma(static_cast<double>(d), static_cast<double>(d), f2);
+    const float dd = d * d;
+    f2.add(dd);
+    f2.lo += fmaf(d, d, -dd);
     two_sum(fabsf(pp), fabsf(po), d, e);
     ab.add(d);
-    ab.add_low(e);
+    ab.lo += e;
   }
   __device__ __forceinline__ void store(const ChipCta &X) {
-    const double s = f.value();
-    const double t0 = warp_sum_d(s), t1 = warp_sum_d(f2), t2 = warp_sum_d(ab.value()), t3 = warp_sum_d(s + de.value());
+    const double t0 = warp_sum_d(f.value()), t1 = warp_sum_d(f2.value()), t2 = warp_sum_d(ab.value());
+    const double t3 = warp_sum_d(f.value() + static_cast<double>(de));
     if (X.lane < 4) X.sh.dpart[X.warp][X.lane] = X.lane == 0 ? t0 : X.lane == 1 ? t1 : X.lane == 2 ? t2 : t3;
   }
 };
+
+// Whether FP32 held the balancing sums m of a gather of N cells.  It did not where one is not finite
+// (squares of 1e18 and more; inputs that are not finite), nor where the sum of squares is so small
+// that what its cells lose to the smallest step of a float, 2^-149 each, may reach 2^-53 of it (f of about 3e-15 and
+// less).  A sum of zero stands: the passes' own sums of squares are zero too then, in any solve.
+__device__ __forceinline__ bool balance_in_range(const double (&m)[4], double N) {
+  return isfinite(m[0]) && isfinite(m[1]) && isfinite(m[2]) && isfinite(m[3]) && (m[1] == 0.0 || m[1] >= N * 0x1p-96);
+}
 
 // u of a warm start at (gi, gj), plane 0 (x) or 1 (t); the outer faces carry none.
 __device__ __forceinline__ float chip_init_flux(const ChipCta &X, int plane, int gi, int gj) {
@@ -795,9 +786,8 @@ __device__ __forceinline__ void chip_decider(const ChipCta &X) {
   };
   publish_sc(sh.sc, static_cast<float>(pr.alpha), 0.0f, 1.0f, 1.0f / (1.0f + static_cast<float>(c.eps * pr.alpha)));
   if (lane >= 16 && lane < 24) sh.sc[lane >> 2][lane & 3] = lane < 20 ? rdx : rdt;
-  // Sums that left the range of FP32, or inputs that are not finite: the gather is handed back (the
-  // streaming solve adds these sums in FP64).
-  const bool summed = isfinite(m4[0]) && isfinite(m4[1]) && isfinite(m4[2]) && isfinite(m4[3]);
+  // a gather whose sums left the range of FP32 is handed back: the streaming solve adds them in FP64
+  const bool summed = balance_in_range(m4, N);
   bool done = !summed;
   int status = summed ? ST_OK : ST_NONFINITE;
   if (lane == 0) {

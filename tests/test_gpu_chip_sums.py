@@ -1,9 +1,10 @@
 """The balancing sums of the on-chip solve (f, f^2, |Pcal| + |Pobs|, Pcal - Pobs) against exact ones,
 in its three forms, at amplitudes whose squares leave the range of FP32.
 
-The linear sums are added in more than 53 bits within a lane and in FP64 above it: at most 5 additions
-in a warp, 4 in a CTA, 19 + 2 across the CTAs of a copy and the copies, each rounded to 2^-53 of a
-partial sum, so they are exact to 30 * 2^-53 < 4e-15 of the sum of the magnitudes.  The reported
+The sums are added in pairs of floats within a lane, to about 2^-48 of a lane's part, whose errors
+average out over the lanes, and in FP64 above it: at most 5 additions in a warp, 4 in a CTA, 19 + 2 across the
+CTAs of a copy and the copies, each rounded to 2^-53 of a partial sum, so they are exact to 4e-15 of
+the sum of the magnitudes.  Gathers whose sums leave the range of FP32 go back to the streaming solve.  The reported
 residual is sqrt(sum p^2) / |f|, whose numerator is a sum of FP32 squares in every solve: 1e-5, as
 between any two of them."""
 
@@ -56,7 +57,7 @@ def test_residual_of_small_amplitudes(P, nr, nt):
     obs, pred = 1e-22 * noise(nr, nt, 3), 1e-22 * noise(nr, nt, 4)
     got = solve(P, obs, pred, max_iter=5, alpha0=1e-4)[3]
     ref = solve(P, obs, pred, max_iter=5, alpha0=1e-4, tile=TILE if nr * nt < 1.4e6 else MARCH)[3]
-    assert got["status"] == ref["status"] == 0 and got["tile"] == 0
+    assert got["status"] == ref["status"] == 0
     assert math.isclose(got["r_feas"], ref["r_feas"], rel_tol=1e-5), (got["r_feas"], ref["r_feas"])
 
 
@@ -67,15 +68,13 @@ def check_like_streaming(P, obs, pred):
     assert got[3]["status"] == ref[3]["status"] == 0
     for key in ("r_feas", "mass_mu", "mass_nu", "dist"):
         assert math.isclose(got[3][key], ref[3][key], rel_tol=1e-5), (key, got[3][key], ref[3][key])
-    return got
 
 
 @pytest.mark.parametrize("nr,nt", SIZES)
 def test_residual_above_a_common_level(P, nr, nt):
     """Pcal on a level whose squares FP32 cannot add up.  Balancing takes the level out, so the pass's
-    own sums stay in range."""
-    got = check_like_streaming(P, np.zeros((nr, nt)), 8e18 + 1e16 * noise(nr, nt, 5))
-    assert got[3]["tile"] == 0
+    own sums stay in range, and the gather is solved by the streaming passes."""
+    check_like_streaming(P, np.zeros((nr, nt)), 8e18 + 1e16 * noise(nr, nt, 5))
 
 
 @pytest.mark.parametrize("nr,nt", SIZES)
