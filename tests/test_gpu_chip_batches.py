@@ -107,3 +107,25 @@ def test_failed_linesearches_leave_what_the_passes_of_their_rounding_leave(P, si
         assert infos[b]["iters"] == ref["iters"]
         k = infos[b]["iters"]
         assert torch.allclose(trace[b, :k], one[0, :k], rtol=1e-5, atol=0.0), sizes[b]
+
+
+@pytest.mark.parametrize("sizes,tol", [([(64, 256), (40, 300), (100, 400), (64, 256), (12, 700), (33, 401)], 0.1),
+                                       ([(64, 256)] * 40, 0.1), ([(200, 2000)] * 6, 0.3),
+                                       ([(640, 5000), (300, 5041), (353, 4001)], 0.2),
+                                       ([(64, 256), (400, 3000), (700, 9000), (33, 401)], 0.5)])
+def test_gathers_of_a_batch_stop_by_themselves(P, sizes, tol):
+    """Gathers that stop at a tolerance while their neighbours, and the waves after them, go on: passes
+    with a stopping test take the FP64 exchange between others of the fixed-point one, and the streamed
+    part of a split batch is dealt again."""
+    obs, pred = pairs(sizes, 60)
+    for b in range(len(sizes)):  # predicted gathers from near to far from the observed ones
+        pred[b] = obs[b] + (0.02 + b / len(sizes)) * (pred[b] - obs[b])
+        obs[b] = obs[b] * (1.0 - 0.3 * (b % 3))
+    dts, dxs = unit(sizes)
+    kw = dict(max_iter=4000, tol=tol, check_every=5)
+    d, phis, ms, infos = P.emd_batched(obs, pred, dts, dxs, **kw)
+    assert sum(i["tile"] == 0 for i in infos) >= len(sizes) - 1
+    assert len({i["iters"] for i in infos}) > 1 and min(i["iters"] for i in infos) < 4000
+    for b in range(len(sizes)):
+        ref = P.emd(obs[b], pred[b], dts[b], dxs[b], tile=infos[b]["tile"] or streaming(sizes), **kw)
+        same((d[b], phis[b], ms[b], infos[b]), ref, (b, sizes[b]))
