@@ -129,3 +129,36 @@ def test_gathers_of_a_batch_stop_by_themselves(P, sizes, tol):
     for b in range(len(sizes)):
         ref = P.emd(obs[b], pred[b], dts[b], dxs[b], tile=infos[b]["tile"] or streaming(sizes), **kw)
         same((d[b], phis[b], ms[b], infos[b]), ref, (b, sizes[b]))
+
+
+def test_solves_of_two_threads_at_a_time(P):
+    """Two threads with a stream and a workspace each: cooperative launches wait for one another on the
+    device, and neither solve sees the other's state."""
+    import threading
+    sizes = [[(64, 256), (400, 3000)], [(353, 4001), (33, 401)]]
+    work = []
+    for i, s in enumerate(sizes):
+        obs, pred = pairs(s, 80 + 10 * i)
+        dts, dxs = unit(s)
+        work.append((obs, pred, dts, dxs, P.emd_batched(obs, pred, dts, dxs, max_iter=30)))
+    torch.cuda.synchronize()
+    errors, gate = [], threading.Barrier(2)
+
+    def run(obs, pred, dts, dxs, ref):
+        try:
+            stream = torch.cuda.Stream()
+            with torch.cuda.stream(stream):
+                gate.wait(60)
+                for _ in range(20):
+                    got = P.emd_batched(obs, pred, dts, dxs, max_iter=30)
+                    for b in range(len(obs)):
+                        same([g[b] for g in got], [r[b] for r in ref], b)
+        except BaseException as e:
+            errors.append(e)
+
+    threads = [threading.Thread(target=run, args=w) for w in work]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
