@@ -160,6 +160,19 @@ def _ran(tile):
     return f"{kname}{kargs} (tile id {tile}, the autotuner's choice)"
 
 
+def _reductions(tile):
+    """How the sums behind a solve's decisions and residuals are added."""
+    if tile == 0:
+        return ("FP32 within a warp, pairs of floats within a CTA, fixed point across CTAs (FP64 for passes with a "
+                "residual); FP64 decision where an FP32 one with a margin does not settle it")
+    return "f64 above the warp"
+
+
+def _hbm_gbs(tiles, cells, t_pass):
+    """GB/s of a pass that streams its state, 36 B per cell; None where a gather stays on chip."""
+    return None if 0 in tiles else CELL_BYTES * cells / t_pass / 1e9
+
+
 def _roofline(tile, cells, t_pass, traffic, dev):
     """The bound of the pass: the state's 36 B per cell through HBM where it streams, the FP32
     lanes where it stays on chip."""
@@ -443,7 +456,6 @@ def run_marine(a):
     n1, n2 = 20, 100
     timed_solve(n1)
     t_pass = (timed_solve(n2) - timed_solve(n1)) / (n2 - n1)
-    achieved = CELL_BYTES * cells / t_pass / 1e9
     kname, _ = _kernel_of(res[0].tile)
     traffic = _traffic(f"{kname}_tile{res[0].tile}_traffic_marine.json", cells)
 
@@ -553,11 +565,11 @@ def run_marine(a):
                        "step": "emd_dyn_solve_batched (prepare, every pass, finalize) "
                                "+ emd_adjoint_batched",
                        "l2": "not flushed: inputs larger than L2 (5.3 GB of gathers per step)",
-                       "reductions": "f64 above the warp", "parallelism": f"shots sharded over {world} ranks, "
-                                                                          "no collective",
+                       "reductions": _reductions(res[0].tile),
+                       "parallelism": f"shots sharded over {world} ranks, no collective",
                        "data_generation_s": t_gen},
             "solves_per_s": N_SHOTS / t_step,
-            "hbm_gbs_algorithmic": achieved,
+            "hbm_gbs_algorithmic": _hbm_gbs({r.tile for r in res}, cells, t_pass),
             "roofline": {**_roofline(res[0].tile, cells, t_pass, traffic, dev), "kernel": _ran(res[0].tile)},
             "cpu_baseline": cpu,
             "e2e": {"value": e2e_v, "unit": "cell-updates/s", "h2d_bytes_per_step": 2 * cells * 4,
@@ -608,8 +620,10 @@ def _marine_single_extra(P, obs, pred, phis, ms, stream):
     t2, r = timed(lambda: solve(0, 200))
     t_pass = (t2 - t1) / 180
     t_all, _ = timed(lambda: [solve(b, M_ITERS) for b in range(len(obs))])
+    gbs = _hbm_gbs({r.tile}, M_NT * M_NR, t_pass)
     return {"pass_us_8000x648": 1e6 * t_pass,
-            "hbm_frac_8000x648": CELL_BYTES * M_NT * M_NR / t_pass / 1e9 / _peaks()[0],
+            "hbm_frac_8000x648": None if gbs is None else gbs / _peaks()[0],
+            "fp32_frac_8000x648": _roofline(0, M_NT * M_NR, t_pass, None, dev)["frac"] if r.tile == 0 else None,
             "kernel_8000x648": _ran(r.tile),
             "solves_per_s_one_by_one": len(obs) / t_all,
             "note": f"{len(obs)} gathers solved one after another, {M_ITERS} iterations, forward only; the "
@@ -753,16 +767,16 @@ def _uneven48_extra(P, dev, a):
         torch.cuda.synchronize()
         e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
         e0.record()
-        fn()
+        out = fn()
         e1.record()
         torch.cuda.synchronize()
-        return e0.elapsed_time(e1) / 1e3
+        return e0.elapsed_time(e1) / 1e3, out
 
-    tb = timed(lambda: P.emd_batched(O_, P_, DT, DX, workspace=wsb, max_iter=200))
-    ts = timed(lambda: [P.emd(o, p, DT, DX, workspace=wss, max_iter=200) for o, p in zip(O_, P_)])
+    tb, (_, _, _, infos) = timed(lambda: P.emd_batched(O_, P_, DT, DX, workspace=wsb, max_iter=200))
+    ts, _ = timed(lambda: [P.emd(o, p, DT, DX, workspace=wss, max_iter=200) for o, p in zip(O_, P_)])
     return {"solves_per_s_batched": 48 / tb, "solves_per_s_one_by_one": 48 / ts, "batched_speedup": ts / tb,
             "cells": cells, "cell_updates_per_s_batched": cells * 200 / tb,
-            "hbm_gbs_algorithmic_batched": CELL_BYTES * cells * 200 / tb / 1e9}
+            "hbm_gbs_algorithmic_batched": _hbm_gbs({i["tile"] for i in infos}, cells, tb / 200)}
 
 
 # --------------------------------------------------------------------------- other workloads
@@ -889,7 +903,7 @@ def run_uneven48(a):
                    "parallelism": f"shots sharded over {world} ranks, no collective"},
         "sequential_solves_per_s": 48 / ts_, "batched_speedup": ts_ / tb, "scaling": "strong",
         "cell_updates_per_s_batched": total_cells * iters / tb,
-        "hbm_gbs_algorithmic_batched": CELL_BYTES * total_cells * iters / tb / 1e9,
+        "hbm_gbs_algorithmic_batched": _hbm_gbs({i["tile"] for i in ib}, total_cells, tb / iters),
         "max_rel_dist_diff_batched_vs_sequential": worst,
     }), flush=True)
 
