@@ -149,8 +149,9 @@ bool size_ok(int nt, int nr) {
   return static_cast<long long>(nr) * ntp_of(nt) < (1ll << 30);
 }
 
-// Workspace: [states | shots | accumulators | tile_shot | n_done + scratch] then, per gather, the
-// pitched planes f, u0 (x,t), u1 (x,t), u2 (x,t), phi0, phi1 (36 bytes per cell).
+// Workspace: [accumulators | states | flags + scratch | gather records | tile list | march list] then,
+// per gather, the pitched planes f, u0 (x,t), u1 (x,t), u2 (x,t), phi0, phi1 (36 bytes per cell; the
+// on-chip solve has its exchange buffers and streamed rows there).
 struct Layout {
   // sums, gather states and flags are adjacent: one fill clears them all, one copy brings states
   // and flags back; the gather records and the tile list go to the device in one copy
@@ -1152,8 +1153,10 @@ emd_status mg_impl(int B, const float *const *f_obs, const float *const *f_pred,
   emd::k_prolong_time<<<pgrid, emd::kIpThreads, 0, stream>>>(djobs, emd::TimeJob{});
   EMD_CK(cudaGetLastError());
 
-  // 4. the fine solve, warm-started from phi and m in place (its prepare pass copies them
-  //    into the workspace before anything writes phi or m again)
+  // 4. the fine solve, warm-started from phi and m in place.  Nothing writes them before all of a
+  //    gather's are read: the prepare pass of a streaming or one-CTA solve copies them into the workspace,
+  //    and in an on-chip solve every CTA reads its part before the balancing exchange, which all its
+  //    CTAs pass before any writes its outputs
   std::vector<const float *> phi_init(phi, phi + B), m_init(m, m + B);
   SolveExtra x;
   x.phi_init = g.interpolate_phi ? phi_init.data() : nullptr;

@@ -259,12 +259,6 @@ __device__ __forceinline__ void tmem_stores_done() {
 
 // ------------------------------------------------------------------ barriers
 
-// A compile-time bool as a value (selects a lambda's instantiation).
-template <bool B>
-struct BoolConst {
-  static constexpr bool value = B;
-};
-
 // Barriers of a CTA of NW worker warps: the workers alone, or with the decider warp.
 template <int NW = kChipWorkers>
 __device__ __forceinline__ void bar_workers() {

@@ -26,7 +26,6 @@
 // values go to the gather's accumulators by FP64 atomics.
 #pragma once
 
-#include "emd_chip.cuh"
 #include "emd_pass_tma.cuh"
 
 namespace emd {

@@ -67,6 +67,12 @@ __device__ __forceinline__ unsigned long long global_ns() {
   return t;
 }
 
+// A compile-time bool as a value (selects a lambda's instantiation).
+template <bool B>
+struct BoolConst {
+  static constexpr bool value = B;
+};
+
 // Bound of every wait on another warp or CTA: a wait that outlasts it sets the solve's
 // error flag (EMD_ERR_TIMEOUT) and the kernel winds down instead of hanging.
 constexpr unsigned long long kSpinLimitNs = 4000000000ull;  // 4 s
