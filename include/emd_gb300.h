@@ -133,7 +133,9 @@ typedef struct {
   int iters;          /* accepted PDHG iterations                                        */
   int ls_trials;      /* linesearch trials in total (>= iters)                           */
   int status;         /* emd_status of this solve                                        */
-  int launches;       /* kernel launches this solve made (a graph's nodes count one each) */
+  int launches;       /* kernel launches this solve made (a graph's nodes count one each;
+                         of both solves where an on-chip one handed the gather back to the
+                         streaming passes: failed, or out of the range of FP32 sums)     */
   int tile;           /* tile-shape id the solve ran (1..emd_tile_count(); the autotuner's
                          choice when params->tile was 0); 0 for the shared-memory and the
                          on-chip solve                                                     */
